@@ -101,6 +101,8 @@ struct gamma_ctx {
     // cell table
     std::vector<TableEntry> table;
     TableEntry* table_dev = nullptr;
+    gk::WalkEntry* walk_dev = nullptr;   // the table as the warp-evaluated walk reads it (table_dev lies
+                                         // behind it in the same allocation)
     float key0_far2[8] = {};
     double r_cover = 0;
     int64_t table_cap = 1 << 17;
@@ -121,6 +123,9 @@ struct gamma_ctx {
     unsigned long long* row_sorted = nullptr;
     // warp-evaluated walk: voxels left to its finishing pass (tail_cap entries)
     unsigned* fix_list = nullptr;
+    unsigned* plane_raw = nullptr;    // ... the cells of the plane seeds (tail_cap entries each, allocated
+                                      //     with fix_list)
+    unsigned* plane_sorted = nullptr;
     int group_bucket = 9;             // ... queued voxels of this cost bucket and above walk 4 lanes each
                                       //     (< 0: the walk chooses the parts from the queue)
     int group_auto_pct = 100;         // ... with this slack (percent)
@@ -257,12 +262,30 @@ int build_table(gamma_ctx* h)
         h->table[i].key = round_down(all[i].key);
     }
     h->r_cover = cover;
-    if (h->table_dev) { cudaFree(h->table_dev); h->table_dev = nullptr; }
-    if (keep) {
-        CK(cudaMalloc(&h->table_dev, keep * sizeof(TableEntry)));
-        CK(cudaMemcpy(h->table_dev, h->table.data(), keep * sizeof(TableEntry),
-                      cudaMemcpyHostToDevice));
+    // both forms of the table in one buffer and one copy: the walk's entries
+    // (16-byte aligned), then the plain ones
+    const size_t nwalk = keep + gk::kWalkPad, wbytes = nwalk * sizeof(gk::WalkEntry);
+    std::vector<gk::WalkEntry> walk;
+    try {
+        walk.resize(nwalk + (keep * sizeof(TableEntry) + sizeof(gk::WalkEntry) - 1) / sizeof(gk::WalkEntry),
+                    gk::WalkEntry{INFINITY, 0, 0u, 0});
+    } catch (const std::bad_alloc&) {
+        return GAMMA_ERR_OOM;
     }
+    int margin = 0;
+    for (size_t i = 0; i < keep; ++i) {
+        const int c[3] = {all[i].x, all[i].y, all[i].z};
+        for (int a = 0; a < nd; ++a) margin = std::max(margin, std::max(-c[a], c[a] + 1));
+        const int64_t lin = c[0] + (int64_t)c[1] * h->nx + (int64_t)c[2] * h->nx * h->ny;
+        walk[i] = gk::WalkEntry{h->table[i].key, (int)lin, h->table[i].off, margin};
+    }
+    if (keep) std::memcpy((char*)walk.data() + wbytes, h->table.data(), keep * sizeof(TableEntry));
+    cudaFree(h->walk_dev);
+    h->walk_dev = nullptr;
+    h->table_dev = nullptr;
+    CK(cudaMalloc(&h->walk_dev, walk.size() * sizeof(gk::WalkEntry)));
+    h->table_dev = (TableEntry*)((char*)h->walk_dev + wbytes);
+    CK(cudaMemcpy(h->walk_dev, walk.data(), walk.size() * sizeof(gk::WalkEntry), cudaMemcpyHostToDevice));
     return GAMMA_OK;
 }
 
@@ -302,6 +325,7 @@ Problem make_problem(const gamma_ctx* h, float* out)
     P.tau = (float)h->tau;
     P.stats = h->stats;
     P.table = h->table_dev;
+    P.walk = h->walk_dev;
     P.ntable = (int)h->table.size();
     gk::fill_bucket_keys(h->table.data(), P.ntable, P.bucket_key);
     for (int s = 0; s < 8; ++s) P.key0_far2[s] = h->key0_far2[s];
@@ -318,6 +342,10 @@ Problem make_problem(const gamma_ctx* h, float* out)
     P.seed_Y = h->seed_Y;
     P.seed_cap = h->seed_cap;
     P.fix_list = h->fix_list;
+    if (h->walk == 3) {
+        P.plane_raw = h->plane_raw;
+        P.plane_sorted = h->plane_sorted;
+    }
     P.cq_group_bucket = h->group_bucket;
     P.cq_group8_bucket = h->group8_bucket;
     P.cq_group32_bucket = h->group32_bucket;
@@ -360,7 +388,7 @@ void free_ctx(gamma_ctx* h)
     cudaFree(h->slab_flags);
     for (auto& st : h->pipe_s)
         if (st) cudaStreamDestroy(st);
-    cudaFree(h->table_dev);
+    cudaFree(h->walk_dev);
     cudaFree(h->ctr);
     cudaFree(h->tail_raw);
     cudaFree(h->tail_bucket);
@@ -417,6 +445,7 @@ struct BatchState {
         unsigned* item_start = nullptr;
         unsigned* items_v = nullptr;
         unsigned short* items_p = nullptr;
+        unsigned* items_s = nullptr;
         unsigned* head = nullptr;          // walk, shell tiles, seed rows, seeding work,
                                            // warp-evaluated walk parts (3), its fix count
         float4* metric4 = nullptr;         // per pair: metric constants of the warp-evaluated walk
@@ -447,6 +476,7 @@ void free_group(BatchState::Group& g)
     cudaFree(g.item_start);
     cudaFree(g.items_v);
     cudaFree(g.items_p);
+    cudaFree(g.items_s);
     cudaFree(g.head);
     cudaFree(g.fix_v);
     cudaFree(g.metric4);
@@ -498,6 +528,7 @@ int batch_upload(gamma_ctx* h)
             c->stats = 0;
             c->sort_tail = 1;
             c->shell_minblocks = h->shell_minblocks;
+            c->walk = h->walk;
             probs[k] = make_problem(c, b->outs[mem[k]]);
             std::memset(&maps[k], 0, sizeof(CUtensorMap));
             use[k] = gk::encode_tile_map(probs[k], &maps[k]) ? 1 : 0;
@@ -517,6 +548,7 @@ int batch_upload(gamma_ctx* h)
             for (int k = 0; k < np; ++k) cap += b->pairs[mem[k]]->tail_cap;
             CK(cudaMalloc(&G.items_v, sizeof(unsigned) * std::max<size_t>(cap, 1)));
             CK(cudaMalloc(&G.items_p, sizeof(unsigned short) * std::max<size_t>(cap, 1)));
+            CK(cudaMalloc(&G.items_s, sizeof(unsigned) * std::max<size_t>(cap, 1)));
             CK(cudaMalloc(&G.fix_v, sizeof(unsigned) * std::max<size_t>(cap, 1)));
             CK(cudaMalloc(&G.metric4, sizeof(float4) * 3 * np));
             CK(cudaMalloc(&G.fix_p, sizeof(unsigned short) * std::max<size_t>(cap, 1)));
@@ -554,13 +586,15 @@ int batch_upload(gamma_ctx* h)
         d.item_start = G.item_start;
         d.items_v = G.items_v;
         d.items_p = G.items_p;
+        d.items_s = G.items_s;
         d.head = G.head;
         d.shell_next = G.head + 1;
         d.group_bucket = h->walk == 3 ? h->group_bucket : 0;
         d.group8_bucket = h->walk == 3 ? h->group8_bucket : 0;
         d.group32_bucket = h->walk == 3 ? h->group32_bucket : 0;
         d.auto_scale = 0.01f * (float)h->group_auto_pct;
-        d.walk_lanes = (unsigned)(gk::device_sm_count() * std::min(4, std::max(1, h->tail_minblocks)) * 256);
+        const int per_sm = std::min(4, std::max(1, h->tail_minblocks));
+        d.walk_lanes = (unsigned)(gk::device_sm_count() * per_sm * gk::cq_threads(per_sm));
         d.part_head = G.head + 4;
         d.metric4 = G.metric4;
         d.fix_v = G.fix_v;
@@ -604,6 +638,8 @@ int batch_enqueue(gamma_ctx* h, cudaStream_t s)
     for (auto& G : b->grp) CK(gk::launch_batch_prepare(G.host, s));
     if (tm) CK(cudaEventRecord(h->tev[2], s));
     for (auto& G : b->grp) CK(gk::launch_batch_shell(G.host, h->shell_minblocks, s));
+    if (h->walk == 3)
+        for (auto& G : b->grp) CK(gk::launch_batch_plane_seed(G.host, s));
     if (h->model) {
         // learned seeding of every pair's queued voxels past the cost gate
         gk::MlpWeights W;
@@ -688,7 +724,10 @@ int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev,
     if ((e = cudaMalloc(&h->tail_raw, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = cudaMalloc(&h->tail_sorted, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = cudaMalloc(&h->tail_bucket, nvox)) != cudaSuccess) return fail(cuda_fail(e));
-    if ((e = cudaMalloc(&h->fix_list, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
+    // one allocation for the three lists of the warp-evaluated walk
+    if ((e = cudaMalloc(&h->fix_list, 3 * sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
+    h->plane_raw = h->fix_list + nvox;
+    h->plane_sorted = h->plane_raw + nvox;
     {
         Problem P0 = make_problem(h, nullptr);
         const int tiles = gk::block_tiles(P0);
@@ -880,6 +919,7 @@ static int enqueue_search(gamma_handle h, const Problem& P, cudaStream_t s)
     CK(cudaMemsetAsync(h->ctr, 0, sizeof(Counters), s));
     CK(gk::launch_prepare(P, s, 1));
     CK(gk::launch_shell(P, s));
+    CK(gk::launch_plane_seed(P, s));
     return enqueue_walk(h, P, s, false);
 }
 
@@ -972,6 +1012,7 @@ int gamma_run(gamma_handle h, float* gamma_out_dev, void* cuda_stream)
         return GAMMA_OK;
     }
     CK(gk::launch_shell(P, s));
+    CK(gk::launch_plane_seed(P, s));
     if (h->model) {
         gk::MlpWeights W;
         gk::model_weights(h->model, &W);
@@ -1109,6 +1150,7 @@ int run_host_pipelined(gamma_handle h, const float* eval_host, float* gamma_out_
     CK(cudaMemcpyAsync(gamma_out_host, h->own_out, bytes, cudaMemcpyDeviceToHost, o));
     if (tm) CK(cudaEventRecord(h->tev_out, o));
     CK(cudaEventRecord(E[5], o));
+    CK(gk::launch_plane_seed(P, c));
     if (int rc = enqueue_walk(h, P, c, tm)) return rc;
     if (tm) CK(cudaEventRecord(h->tev[5], c));
     CK(cudaStreamWaitEvent(c, E[5], 0));

@@ -39,6 +39,12 @@ __device__ __forceinline__ bool is_evaluated(const Problem& P, float dr, float t
     return dr >= thr && (!P.local || dr > 0.f);
 }
 
+// Dose e relative to the reference dose dr in units of Delta D (inv = 1 /
+// Delta D).  The rounded product is kept: a compiler that fused it into the
+// face evaluation's differences would give another last bit than the walks
+// that pass the relative doses on through memory or a call.
+__device__ __forceinline__ float rel_dose(float e, float dr, float inv) { return __fmul_rn(e - dr, inv); }
+
 // --------------------------------------------------------------------------
 // FP64 redo of one cell whose Gram matrices are near singular
 // --------------------------------------------------------------------------
@@ -52,7 +58,7 @@ __device__ __noinline__ float cell_redo_f64(const float* __restrict__ ev, long l
     double q[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.0;
+        q[u] = (double)kNaN;
         if (u < (1 << N) && ((ok >> u) & 1u)) {
             const long long o = p + ((u & 1) ? 1 : 0) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0);
             q[u] = ((double)ev[o] - drd) * invd;
@@ -61,7 +67,7 @@ __device__ __noinline__ float cell_redo_f64(const float* __restrict__ ev, long l
     CellGeom<double> g;
     cell_geom<N, double>(cx, cy, cz, mtd, g);
     bool ill = false;
-    const double b = cell_min_d2<N, double>(q, ok, g, mtd, (double)kInf, (double)kInf, ill);
+    const double b = cell_min_d2<N, double>(q, g, mtd, (double)kInf, (double)kInf, ill);
     atomicAdd(fp64_counter, 1u);
     return (float)b;
 }
@@ -78,7 +84,7 @@ __device__ __noinline__ float cell_recheck(const Problem& P, uint32_t ok, int cx
     float q[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.f;
+        q[u] = kNaN;
         if (u < (1 << N) && ((ok >> u) & 1u)) {
             const long long o = p + ((u & 1) ? 1 : 0) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0);
             q[u] = (__ldg(P.ev + o) - dr) * inv;
@@ -104,7 +110,7 @@ __device__ __noinline__ float cell_all_faces(const Problem& P, float q0, float q
     CellGeom<float> g;
     cell_geom<N, float>(cx, cy, cz, P.mt, g);
     bool ill = false;
-    float cb = cell_min_d2<N, float>(q, ok, g, P.mt, ill_dmax(P), kInf, ill);
+    float cb = cell_min_d2<N, float>(q, g, P.mt, ill_dmax(P), kInf, ill);
     if (ill) ill = cell_gram_ill<N>(q, ok, P.mt.kappa, P.tau);
     if (ill) {
         const double drd = dr;

@@ -41,10 +41,23 @@
 namespace gk {
 
 constexpr float kInf = __builtin_huge_valf();
+constexpr float kNaN = __builtin_nanf("");
 
 __host__ __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __host__ __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float div_(float a, float b) { return __fdividef(a, b); }
+// A product that is rounded by itself wherever it stands: the cell constants
+// below are sums of products, and a compiler that fused them differently from
+// one kernel to the next would give the walks other last bits for one cell.
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+// a / b for b >= 1 (D of a face): one reciprocal, without the scaling that
+// __fdividef adds for divisors near the largest float
+__device__ __forceinline__ float div_(float a, float b)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return a * r;
+}
 __device__ __forceinline__ double div_(double a, double b) { return a / b; }
 __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
@@ -69,13 +82,12 @@ using Metric = MetricT<float>;
 // Cell constants for the lower-corner offset c (voxel units from the
 // reference point; integer on a coincident grid, real otherwise).
 template <int N, typename T, typename C>
-__host__ __device__ __forceinline__ void cell_geom(C cx, C cy, C cz, const MetricT<T>& mt,
-                                          CellGeom<T>& g)
+__device__ __forceinline__ void cell_geom(C cx, C cy, C cz, const MetricT<T>& mt, CellGeom<T>& g)
 {
     const T c[3] = {T(cx), T(cy), T(cz)};
     T t[3] = {T(0), T(0), T(0)};
 #pragma unroll
-    for (int a = 0; a < N; ++a) t[a] = mt.hn2[a] * c[a] * c[a];
+    for (int a = 0; a < N; ++a) t[a] = mul_(mul_(mt.hn2[a], c[a]), c[a]);
 #pragma unroll
     for (int A = 0; A < 8; ++A) { g.beta[A] = T(0); g.br[A] = T(0); g.tsum[A] = T(0); }
 #pragma unroll
@@ -100,20 +112,21 @@ __host__ __device__ __forceinline__ void cell_geom(C cx, C cy, C cz, const Metri
 #pragma unroll
         for (int b = a + 1; b < N; ++b) {
             const T dc = c[a] - c[b];
-            g.br[(1 << a) | (1 << b)] = mt.hn2[a] * mt.hn2[b] * dc * dc * mt.kappa[(1 << a) | (1 << b)];
+            g.br[(1 << a) | (1 << b)] = mul_(mt.hn2[a] * mt.hn2[b] * dc * dc, mt.kappa[(1 << a) | (1 << b)]);
         }
     if constexpr (N == 3) {
         const T dxy = c[0] - c[1], dxz = c[0] - c[2], dyz = c[1] - c[2];
-        T s = mt.hn2[0] * mt.hn2[1] * dxy * dxy;
+        T s = mul_(mt.hn2[0] * mt.hn2[1] * dxy, dxy);
         s = fma_(mt.hn2[0] * mt.hn2[2], dxz * dxz, s);
         s = fma_(mt.hn2[1] * mt.hn2[2], dyz * dyz, s);
-        g.br[7] = s * mt.kappa[7];
+        g.br[7] = mul_(s, mt.kappa[7]);
     }
 }
 
 // Projection of the origin onto the owned face with chain (U1[, U2[, U3]]).
 // d2 is the squared distance, or +inf when the projection falls outside the
-// face or the face leaves the grid; mu are the coefficients of the chain
+// face or the face leaves the grid (the relative dose of a vertex outside it is
+// NaN, which makes every condition of its faces false); mu are the coefficients of the chain
 // increments (the foot point is s0 + sum_i mu_i e_i).
 //
 // Near-singular Gram matrices.  With the increments scaled to unit spatial
@@ -129,7 +142,7 @@ struct FaceFoot {
 };
 
 template <int M, int U1, int U2, int U3, typename T>
-__device__ __forceinline__ FaceFoot<T> face_core(const T (&q)[8], uint32_t ok, const CellGeom<T>& g,
+__device__ __forceinline__ FaceFoot<T> face_core(const T (&q)[8], const CellGeom<T>& g,
                                                  const T (&kappa)[8], T dmax, bool& ill)
 {
     constexpr int UM = M == 1 ? U1 : (M == 2 ? U2 : U3);
@@ -172,16 +185,16 @@ __device__ __forceinline__ FaceFoot<T> face_core(const T (&q)[8], uint32_t ok, c
         }
         ill = ill || (D > dmax);
     }
-    valid = valid && (last >= T(0)) && ((ok >> UM) & 1u);
+    valid = valid && (last >= T(0));
     f.d2 = valid ? fma_(L, r, rho2) : T(kInf);
     return f;
 }
 
 template <int M, int U1, int U2, int U3, typename T>
-__device__ __forceinline__ T face_d2(const T (&q)[8], uint32_t ok, const CellGeom<T>& g,
+__device__ __forceinline__ T face_d2(const T (&q)[8], const CellGeom<T>& g,
                                      const T (&kappa)[8], T dmax, bool& ill)
 {
-    return face_core<M, U1, U2, U3, T>(q, ok, g, kappa, dmax, ill).d2;
+    return face_core<M, U1, U2, U3, T>(q, g, kappa, dmax, ill).d2;
 }
 
 template <int M, int U1, int U2, int U3>
@@ -216,31 +229,30 @@ template <int N>
 constexpr int kFacesPerCell = N == 3 ? 26 : 6;
 
 template <typename T, int M, int U1, int U2, int U3>
-__device__ __forceinline__ void apply_face(Face<M, U1, U2, U3>, const T (&q)[8], uint32_t ok,
+__device__ __forceinline__ void apply_face(Face<M, U1, U2, U3>, const T (&q)[8],
                                            const CellGeom<T>& g, const T (&kappa)[8], T dmax,
                                            T& best, bool& ill)
 {
-    best = min_(best, face_d2<M, U1, U2, U3, T>(q, ok, g, kappa, dmax, ill));
+    best = min_(best, face_d2<M, U1, U2, U3, T>(q, g, kappa, dmax, ill));
 }
 
 template <typename T, typename... Fs>
-__device__ __forceinline__ void apply_all(std::tuple<Fs...>*, const T (&q)[8], uint32_t ok,
+__device__ __forceinline__ void apply_all(std::tuple<Fs...>*, const T (&q)[8],
                                           const CellGeom<T>& g, const T (&kappa)[8], T dmax,
                                           T& best, bool& ill)
 {
-    (apply_face(Fs{}, q, ok, g, kappa, dmax, best, ill), ...);
+    (apply_face(Fs{}, q, g, kappa, dmax, best, ill), ...);
 }
 
 // Minimum squared distance over all faces owned by one cell.  q holds the
 // relative normalised doses of the cell's 2^N vertices (index = axis mask;
-// entries of vertices outside the grid must be finite), ok has bit u set when
-// vertex u lies inside the grid (bit 0 must be set).
+// NaN for a vertex outside the grid, which vertex 0 must not be).
 template <int N, typename T>
-__device__ __forceinline__ T cell_min_d2(const T (&q)[8], uint32_t ok, const CellGeom<T>& g,
+__device__ __forceinline__ T cell_min_d2(const T (&q)[8], const CellGeom<T>& g,
                                          const MetricT<T>& mt, T dmax, T best, bool& ill)
 {
     best = min_(best, fma_(q[0], q[0], g.tsum[0]));            // the vertex itself
-    apply_all<T>((typename FaceList<N>::type*)nullptr, q, ok, g, mt.kappa, dmax, best, ill);
+    apply_all<T>((typename FaceList<N>::type*)nullptr, q, g, mt.kappa, dmax, best, ill);
     return best;
 }
 
@@ -285,12 +297,12 @@ __device__ __forceinline__ bool cell_gram_ill(const float (&q)[8], uint32_t ok, 
 // Argmin variant: the minimum over the cell's faces of the squared distance
 // and the foot point, in voxel units relative to the cell's lower corner.
 template <typename T, int M, int U1, int U2, int U3>
-__device__ __forceinline__ void arg_face(Face<M, U1, U2, U3>, const T (&q)[8], uint32_t ok,
+__device__ __forceinline__ void arg_face(Face<M, U1, U2, U3>, const T (&q)[8],
                                          const CellGeom<T>& g, const T (&kappa)[8], T& best,
                                          T (&foot)[3])
 {
     bool ill = false;
-    const FaceFoot<T> f = face_core<M, U1, U2, U3, T>(q, ok, g, kappa, T(kInf), ill);
+    const FaceFoot<T> f = face_core<M, U1, U2, U3, T>(q, g, kappa, T(kInf), ill);
     if (f.d2 < best) {
         best = f.d2;
         constexpr int A1 = U1, A2 = U2 ^ U1, A3 = U3 ^ U2;
@@ -302,15 +314,15 @@ __device__ __forceinline__ void arg_face(Face<M, U1, U2, U3>, const T (&q)[8], u
 }
 
 template <typename T, typename... Fs>
-__device__ __forceinline__ void arg_all(std::tuple<Fs...>*, const T (&q)[8], uint32_t ok,
+__device__ __forceinline__ void arg_all(std::tuple<Fs...>*, const T (&q)[8],
                                         const CellGeom<T>& g, const T (&kappa)[8], T& best,
                                         T (&foot)[3])
 {
-    (arg_face(Fs{}, q, ok, g, kappa, best, foot), ...);
+    (arg_face(Fs{}, q, g, kappa, best, foot), ...);
 }
 
 template <int N, typename T>
-__device__ __forceinline__ void cell_argmin(const T (&q)[8], uint32_t ok, const CellGeom<T>& g,
+__device__ __forceinline__ void cell_argmin(const T (&q)[8], const CellGeom<T>& g,
                                             const MetricT<T>& mt, T& best, T (&foot)[3])
 {
     const T dv = fma_(q[0], q[0], g.tsum[0]);
@@ -318,7 +330,7 @@ __device__ __forceinline__ void cell_argmin(const T (&q)[8], uint32_t ok, const 
         best = dv;
         foot[0] = foot[1] = foot[2] = T(0);
     }
-    arg_all<T>((typename FaceList<N>::type*)nullptr, q, ok, g, mt.kappa, best, foot);
+    arg_all<T>((typename FaceList<N>::type*)nullptr, q, g, mt.kappa, best, foot);
 }
 
 }  // namespace gk

@@ -106,7 +106,7 @@ __device__ __forceinline__ float grid_cell(const GridProblem& G, const int (&p)[
     uint32_t ok = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
-        q[w] = 0.f;
+        q[w] = kNaN;
         if (w < (1 << N)) {
             const bool present = (!(w & 1) || ex) && (!(w & 2) || ey) && (!(w & 4) || ez);
             if (present) {
@@ -130,7 +130,7 @@ __device__ __forceinline__ float grid_cell(const GridProblem& G, const int (&p)[
     cell_geom<N, float>(cf[0], cf[1], N == 3 ? cf[2] : 0.f, G.mt, g);
     bool ill = false;
     const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
-    float cb = cell_min_d2<N, float>(q, ok, g, G.mt, dmax, kInf, ill);
+    float cb = cell_min_d2<N, float>(q, g, G.mt, dmax, kInf, ill);
     if (ill) ill = cell_gram_ill<N>(q, ok, G.mt.kappa, G.tau);
     if (ill) {
         const double drd = dr;
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_cq(const __grid_constant__ Grid
         float q[8], cf[3] = {0.f, 0.f, 0.f};
         uint32_t ok = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) q[u] = 0.f;
+        for (int u = 0; u < 8; ++u) q[u] = kNaN;
         if (walking) {
             const float bst = __uint_as_float(V.best[ws]);
             ended = t0 >= ntable || k0 * k0 >= bst;           // A1 step 4b-ii, exact
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_cq(const __grid_constant__ Grid
                 cell_geom<N, float>(V.cf[0][slot], V.cf[1][slot], N == 3 ? V.cf[2][slot] : 0.f, G.mt, cg);
                 bool ill = false;
                 const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
-                const float cb = cell_min_d2<N, float>(cq, cok, cg, G.mt, dmax, kInf, ill);
+                const float cb = cell_min_d2<N, float>(cq, cg, G.mt, dmax, kInf, ill);
                 if (ill && cell_gram_ill<N>(cq, cok, G.mt.kappa, G.tau))
                     atomicOr(&W.fixm[owner >> 5], 1u << (owner & 31));   // searched again
                 else

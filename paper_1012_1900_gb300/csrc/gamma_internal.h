@@ -23,6 +23,11 @@ constexpr int kDefaultLanesPerVoxel = 8;
 constexpr int kDefaultShellBlocksPerSm = 2;
 constexpr int kDefaultTailBlocksPerSm = 2;
 
+// Threads per block of the warp-evaluated walk sized for per_sm resident blocks
+// per SM: at the default of two blocks, twelve warps each fill the registers
+// (80 per thread) better than eight (the evaluation needs no more than 80).
+constexpr int cq_threads(int per_sm) { return per_sm == 2 ? 384 : 256; }
+
 // Flags raised by kernels (Counters::flags).
 enum : uint32_t {
     kFlagNonFinite = 1u,     // a NaN or Inf dose was seen
@@ -44,6 +49,19 @@ struct TableEntry {
     uint32_t off;
     float key;
 };
+
+// The same table as the warp-evaluated walk reads it (16 bytes): with the
+// offset's index distance on the pair's grid, and the largest margin (voxels
+// between the voxel and the nearest grid face) that this entry or an earlier
+// one needs for its cell to lie in the grid with every vertex.  Padded with
+// kWalkPad entries of infinite key, which no walk reaches.
+struct alignas(16) WalkEntry {
+    float key;
+    int lin;
+    uint32_t off;
+    int margin;
+};
+constexpr int kWalkPad = 128;
 
 __host__ __device__ inline int unpack10(uint32_t v, int shift)
 {
@@ -142,6 +160,7 @@ struct Problem {
     float tau;               // FP64 redo when det(G)/prod(G_ii) < tau (0: never)
     int stats;               // count cells in the tail search
     const TableEntry* table;
+    const WalkEntry* walk;   // the table for the warp-evaluated walk
     int ntable;
     // cost bucket thresholds: bucket_key[b] (b >= 1) is the key of table entry
     // ceil(2^((b - 1) / 2)) - 1 (+inf past the table), so that the cost bucket
@@ -189,6 +208,10 @@ struct Problem {
     int cq_group32_bucket;
     float cq_auto_scale;         // ... with this slack
     unsigned* fix_list;
+    // ... and the packed offset of the cell each queued voxel's plane seed
+    // evaluated, in discovery and in cost order (null: the other walks)
+    unsigned* plane_raw;
+    unsigned* plane_sorted;
 };
 
 // Readiness of the evaluation dose by z slab, for a shell launch that starts
@@ -214,6 +237,7 @@ struct BatchDesc {
                                    // the ends of the first three parts (k_bucket_scan_batch)
     unsigned* items_v;             // [sum of tail_cap] queued voxels in that order
     unsigned short* items_p;       // [sum of tail_cap] their pair
+    unsigned* items_s;             // [sum of tail_cap] the cell of their plane seed
     unsigned* head;                // work counter of the group's table walk
     // warp-evaluated walk: cost buckets from which the queued voxels walk 4,
     // 8 and 32 lanes each (the queue's parts, costliest first; all 0 keeps one
@@ -278,9 +302,13 @@ void shell_layers(const Problem& P, int* tiles_per_layer, int* layers, int* laye
 // host memory.
 cudaError_t launch_patch_host(const Problem& P, float* host_out_mapped, Counters* host_ctr_mapped,
                               cudaStream_t s);
+// Bounds of the queued voxels from the affine parts of the cells around them
+// (before the ordering; only the warp-evaluated walk's problems).
+cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s);
 cudaError_t launch_order_tail(const Problem& P, cudaStream_t s);
 cudaError_t launch_tail(const Problem& P, int lanes_per_voxel, int tail_minblocks, cudaStream_t s);
-// one lane per queued voxel, surviving cells evaluated by the whole warp
+// 1 to 32 lanes per queued voxel in step, surviving cells evaluated by the
+// whole warp
 cudaError_t launch_tail_cq(const Problem& P, int tail_minblocks, cudaStream_t s);
 // Tile-staged walk (P.tile_mask set): order the tiles with queued voxels by
 // cost, then one block per tile stages the tile's evaluation-dose halo box in
@@ -367,6 +395,7 @@ cudaError_t launch_labels(const Problem& P, const float* gmap, const unsigned* v
 // Batched launches over one group: prepare, shell, ordering, table walk.
 cudaError_t launch_batch_prepare(const BatchGroup& g, cudaStream_t s);
 cudaError_t launch_batch_shell(const BatchGroup& g, int shell_minblocks, cudaStream_t s);
+cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s);
 cudaError_t launch_batch_order(const BatchGroup& g, cudaStream_t s);
 // walk: 3 the warp-evaluated walk, else the voxel walk with lanes_per_voxel.
 cudaError_t launch_batch_tail(const BatchGroup& g, int walk, int lanes_per_voxel, int tail_minblocks,

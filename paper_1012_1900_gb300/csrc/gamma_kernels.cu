@@ -746,6 +746,10 @@ __global__ void __launch_bounds__(256, MINB)
     }
 }
 
+// Table cells a queued voxel of cost bucket b is estimated to key: the middle
+// of the bucket.
+__device__ __forceinline__ float bucket_cells(int b) { return b > 0 ? exp2f((2 * b - 1) * 0.25f) : 0.5f; }
+
 // The queue's parts chosen from the queue itself (option group_bucket < 0):
 // a queued voxel of cost bucket b is estimated to key c(b) = 2^((2b - 1) / 4)
 // table cells (the middle of the bucket), the walk's W = sum of c over the
@@ -805,7 +809,10 @@ __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem
         if (threadIdx.x < kNumBuckets && cnt[threadIdx.x])
             base[threadIdx.x] = start[threadIdx.x] + atomicAdd(&P.ctr->cursor[threadIdx.x], cnt[threadIdx.x]);
         __syncthreads();
-        if (b >= 0) P.tail_sorted[base[b] + rank] = P.tail_raw[i];
+        if (b >= 0) {
+            P.tail_sorted[base[b] + rank] = P.tail_raw[i];
+            if (P.plane_raw) P.plane_sorted[base[b] + rank] = P.plane_raw[i];
+        }
         __syncthreads();
     }
 }
@@ -998,6 +1005,7 @@ __global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restri
             const unsigned pos = base[b] + rank;
             bd->items_v[pos] = P.tail_raw[i];
             bd->items_p[pos] = (unsigned short)blockIdx.y;
+            if (P.plane_raw) bd->items_s[pos] = P.plane_raw[i];
         }
         __syncthreads();
     }
@@ -1028,7 +1036,7 @@ __device__ __forceinline__ float visit_cell(const Problem& P, int x, int y, int 
     float qmin = kInf, qmax = -kInf;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.f;
+        q[u] = kNaN;
         if (u < (1 << N)) {
             const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
             if (present) {
@@ -1211,64 +1219,279 @@ __global__ void __launch_bounds__(256, MINB)
 }
 
 // --------------------------------------------------------------------------
-// k_tail_cq: surviving cells of the walks evaluated 32 at a time by the warp
+// Plane seeds: a queued voxel's bound before its table walk
 // --------------------------------------------------------------------------
 
-// In k_tail the face evaluation of a cell (the bulk of the work) runs with
-// only the lanes whose cell passed the dose-gap test active.  Here a voxel's
-// walk appends each cell that passes the test, with its vertex doses, to a
-// ring buffer of the warp instead of evaluating it; whenever 32 cells wait,
-// the whole warp evaluates them together, one per lane, and lowers each
-// owner's running bound in shared memory (atomicMin on the bits of a
-// non-negative float).  A walk may therefore key and test a few cells against
-// a bound that is not yet the lowest: the stop (key >= bound) and the prune
-// (key^2 + gap^2 >= bound) stay exact with any bound that is at least the
-// true minimum, and each cell is evaluated with the arithmetic of k_tail, so
-// the map is the one k_tail writes.  A voxel is final once every cell it
-// appended has been evaluated; a walker has two voxel slots so that it can
-// start its next voxel while the cells of the previous one still wait.
+// minimum / maximum of three (one instruction on sm_100 and later)
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The affine part of the 2^N vertex doses e of a cell: the value m at the
+// cell's centre, the slope G per voxel along each axis, and eps, a bound on
+// how far a vertex (hence, by linearity in each simplex, any point of the
+// interpolant) lies from it: the sum of the magnitudes of the remaining
+// Walsh-Hadamard coefficients.
+template <int N>
+struct CellPlane {
+    float m, G[3], eps;
+};
+
+template <int N>
+__device__ __forceinline__ CellPlane<N> cell_plane(const float (&e)[8])
+{
+    CellPlane<N> c;
+    if constexpr (N == 3) {
+        const float a0 = e[1] - e[0], a1 = e[3] - e[2], a2 = e[5] - e[4], a3 = e[7] - e[6];
+        const float m0 = e[1] + e[0], m1 = e[3] + e[2], m2 = e[5] + e[4], m3 = e[7] + e[6];
+        const float xlo = a0 + a1, xhi = a2 + a3, ylo = a1 - a0, yhi = a3 - a2;
+        const float plo = m0 + m1, phi = m2 + m3, rlo = m1 - m0, rhi = m3 - m2;
+        c.m = 0.125f * (plo + phi);
+        c.G[0] = 0.25f * (xlo + xhi);
+        c.G[1] = 0.25f * (rlo + rhi);
+        c.G[2] = 0.25f * (phi - plo);
+        c.eps = 0.125f * ((fabsf(xhi - xlo) + fabsf(ylo + yhi)) + (fabsf(yhi - ylo) + fabsf(rhi - rlo)));
+    } else {
+        const float a0 = e[1] - e[0], a1 = e[3] - e[2], m0 = e[1] + e[0], m1 = e[3] + e[2];
+        c.m = 0.25f * (m0 + m1);
+        c.G[0] = 0.5f * (a0 + a1);
+        c.G[1] = 0.5f * (m1 - m0);
+        c.G[2] = 0.f;
+        c.eps = 0.25f * fabsf(a1 - a0);
+    }
+    return c;
+}
+
+// A lower bound on the squared gamma distance from the voxel to the surface
+// over the cell with lower corner c (voxels from the voxel).  With p the
+// cell's affine part (in units of Delta D), the surface satisfies |d - p(s)|
+// <= eps, so its squared distance at s is at least
+//     f(s) = |s|^2 + max(|p(s)| - eps, 0)^2 .
+// Where the plane's value L at the voxel exceeds eps, f is bounded below by
+// the convex |s|^2 + max(+-p(s) - eps, 0)^2, whose minimum is (|L| - eps)^2 / D
+// at the foot point s* (D = 1 + |grad p|^2), and which grows by at least
+// |s - s*|^2 away from it: so f >= (|L| - eps)^2 / D + dist(s*, box)^2.  Below
+// eps the same formula with s* = 0 gives the box distance alone.  eps takes
+// up the rounding of L (ten operations on terms whose magnitudes it sums).
+template <int N>
+__device__ __forceinline__ float plane_bound(const float (&e)[8], const float (&c)[3], float dr, float inv,
+                                             const float (&hn2)[3], const float (&kap)[3])
+{
+    const CellPlane<N> p = cell_plane<N>(e);
+    float L = p.m - dr, mag = fabsf(p.m) + fabsf(dr), D = 0.f, gk[3];
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+        const float t = p.G[a] * (c[a] + 0.5f);
+        L -= t;
+        mag += fabsf(t);
+        gk[a] = p.G[a] * kap[a];
+        D = fmaf(p.G[a], gk[a], D);
+    }
+    const float inv2 = inv * inv;
+    D = fmaf(D, inv2, 1.f);
+    const float Lm = fmaxf(fabsf(L) - fmaf(2e-6f, mag + p.eps, p.eps), 0.f);     // dose units
+    const float r = __fdividef(Lm * inv2, D);
+    float b = Lm * r;
+    const float sr = L > 0.f ? -r : r;
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+        const float s = sr * gk[a];                          // the foot point, in voxels
+        const float w = max3(c[a] - s, s - (c[a] + 1.f), 0.f);
+        b = fmaf(hn2[a] * w, w, b);
+    }
+    return b;
+}
+// A cell is left out when plane_bound reaches best by more than its rounding:
+// the foot point and the box distance carry a relative error of some 1e-6 of
+// the distances involved, which are below sqrt(best) plus a voxel.
+constexpr float kPlaneSlack = 1.f + 3e-5f;
+constexpr unsigned kNoSeed = 0xffffffffu;         // no table offset packs to this (two bits stay zero)
+constexpr int kPlaneSteps = 3;
+
+// The bound of a queued voxel from its own neighbourhood: kPlaneSteps steps
+// that each replace the surface by the affine part of one cell, starting with
+// the voxel's own, and move to the cell that holds the foot point on it; then
+// every face of the last cell.  On the smooth doses of a plan the last cell
+// holds the nearest point itself for 70 to 99 % of the queued voxels, so the
+// walk starts from the final gamma: it keys no cell past it, plane_bound
+// leaves few of the others to evaluate, and the cost buckets (recomputed
+// here) are those of the walk that follows.  The bound is a true distance to
+// the surface, so the result does not depend on it.  One thread per voxel;
+// the cells differ per lane but every lane evaluates exactly one.  Bound by
+// the latency of the dependent dose loads on short queues, by issue on long
+// ones (53 %): 648 k voxels of a 200x200x150 map take 36 us, 5.9 M of a
+// 320x320x240 map 270 us, and spare the walk half of its time there.
+template <int N, bool BATCH>
+__global__ void __launch_bounds__(256)
+    k_plane_seed(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd)
+{
+    __shared__ unsigned sh_hist[kNumBuckets];
+    const Problem& P = BATCH ? bd->probs[blockIdx.y] : P0;
+    const unsigned total = min(P.ctr->tail_count, P.tail_cap);
+    if (blockIdx.x * blockDim.x >= total) return;             // block-uniform
+    if (threadIdx.x < kNumBuckets) sh_hist[threadIdx.x] = 0;
+    __syncthreads();
+    const float dnorm = resolve_dnorm(P);
+    const float hn2[3] = {P.mt.hn2[0], P.mt.hn2[1], P.mt.hn2[2]};
+    const float kap[3] = {P.mt.kappa[1], P.mt.kappa[2], P.mt.kappa[4]};
+    const int nx = P.nx, ny = P.ny, nz = P.nz, sz = nx * ny;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned v = P.tail_raw[i];
+        const int x = (int)(v % (unsigned)nx);
+        const unsigned r1 = v / (unsigned)nx;
+        const int y = (int)(r1 % (unsigned)ny), z = (int)(r1 / (unsigned)ny);
+        const float dr = __ldg(P.ref + v);
+        const float inv = 1.0f / (P.dd_frac * (P.local ? dr : dnorm));
+        const float best = P.out[v];
+        // cells whose every vertex lies in the grid, at most the bound (and
+        // the packed offset's range) away
+        int lo[3], hi[3], c[3] = {0, 0, 0};
+        const int xyz[3] = {x, y, z}, dim[3] = {nx, ny, nz};
+        float e[8];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = a < N ? max(-xyz[a], -511) : 0;
+            hi[a] = a < N ? min(dim[a] - 2 - xyz[a], 510) : 0;
+            c[a] = max(lo[a], min(hi[a], 0));
+        }
+        const float rmax = sqrtf(best);
+#pragma unroll 1
+        for (int it = 0;; ++it) {
+            const float* q = P.ev + ((int)v + c[0] + c[1] * nx + c[2] * sz);
+#pragma unroll
+            for (int u = 0; u < (1 << N); ++u)
+                e[u] = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
+            if (it == kPlaneSteps) break;
+            const CellPlane<N> p = cell_plane<N>(e);
+            float L = p.m - dr, D = 0.f, gk[3];
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                L = fmaf(-p.G[a], (float)c[a] + 0.5f, L);
+                gk[a] = p.G[a] * kap[a];
+                D = fmaf(p.G[a], gk[a], D);
+            }
+            const float inv2 = inv * inv;
+            const float r = __fdividef(L * inv2, fmaf(D, inv2, 1.f));
+            bool same = true;
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                const float lim = rmax * rsqrtf(hn2[a]);
+                const float s = fminf(fmaxf(-r * gk[a], -lim), lim);
+                const int t = max(lo[a], min(hi[a], __float2int_rd(s)));
+                same = same && t == c[a];
+                c[a] = t;
+            }
+            if (same) break;                                  // e holds this cell's doses
+        }
+        // of the cells around the voxel itself only the faces off the voxel
+        // (its vertex taken out), and the walk looks at them again: the faces
+        // through the voxel have their value from the reduced form, from
+        // which the general one could differ in the last bit
+        bool own = true;
+        int self = 0;                                         // the voxel as a vertex of the cell
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            own = own && (unsigned)(c[a] + 1) < 2u;
+            self |= c[a] < 0 ? 1 << a : 0;
+        }
+        float q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            q[u] = u < (1 << N) && !(own && u == self) ? rel_dose(e[u], dr, inv) : kNaN;
+        CellGeom<float> g;
+        cell_geom<N, float>(c[0], c[1], c[2], P.mt, g);
+        bool ill = false;
+        const float cb = cell_min_d2<N, float>(q, g, P.mt, ill_dmax(P), kInf, ill);
+        if (own) {
+            // the walk redoes the whole cell in FP64 if any of its faces is
+            // near singular: not a seed unless the range of its doses rules
+            // that out (D <= 1 + 3 range^2 / min hn2)
+            float qlo = e[0], qhi = e[0];
+#pragma unroll
+            for (int u = 1; u < (1 << N); ++u) {
+                qlo = fminf(qlo, e[u]);
+                qhi = fmaxf(qhi, e[u]);
+            }
+            const float rg = (qhi - qlo) * inv;
+            const float kmax = fmaxf(fmaxf(kap[0], kap[1]), N == 3 ? kap[2] : 0.f);
+            ill = fmaf(3.f * kmax * rg, rg, 1.f) > ill_dmax(P);
+        } else if (ill) {
+            ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, P.mt.kappa, P.tau);
+        }
+        // a near-singular cell is left to the walk (and its FP64 redo)
+        P.plane_raw[i] = ill || own ? kNoSeed : pack10(c[0], c[1], c[2]);
+        if (!ill && cb < best) {
+            P.out[v] = cb + 0.f;                              // -0 -> +0
+            const int was = P.tail_bucket[i], now = cost_bucket_of(P.bucket_key, sqrtf(fmaxf(cb, 0.f)));
+            if (now != was) {
+                P.tail_bucket[i] = (unsigned char)now;
+                atomicAdd(&sh_hist[now], 1u);
+                atomicSub(&sh_hist[was], 1u);                 // wraps; the sum over the block is exact
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < kNumBuckets && sh_hist[threadIdx.x])
+        atomicAdd(&P.ctr->hist[threadIdx.x], sh_hist[threadIdx.x]);
+}
+
+// --------------------------------------------------------------------------
+// k_tail_cq: the table walk, surviving cells evaluated 32 at a time by the warp
+// --------------------------------------------------------------------------
+
+// A warp takes a batch of up to 32 queued voxels of about the same cost, sets
+// them up one per lane, and walks the table for 32 / g of them at a time, g
+// lanes each (a round): lane l of a voxel looks at entry t + l, and the round
+// ends when no lane's key is below its voxel's bound (the exact stop of A1
+// step 4b-ii).  A cell below the bound is tested in three tiers, each of which
+// leaves a fraction of the cells, so each runs with a full warp on the cells
+// that the tier before has collected in a ring buffer:
+//   1. the dose gap of its vertices with the key, in the round itself;
+//   2. plane_bound, 32 cells at a time;
+//   3. its faces, 32 cells at a time, which lower the owner's bound in shared
+//      memory (atomicMin on the bits of a non-negative float).
+// From the plane seed on the bound is nearly final, so a test against a bound
+// that is not yet the lowest keeps few cells more, and it never drops one:
+// each cell is evaluated with the arithmetic of k_tail and the map is the one
+// k_tail writes.  The cell the plane seed evaluated is passed over.  The rings
+// are emptied once per batch, not per round, so that few passes run part full.
 //
 // The queue is ordered by cost bucket, most expensive first: the voxels of
-// bucket cq_group8_bucket and above walk 8 lanes each (8 table entries per
-// step), those of bucket cq_group_bucket and above 4 lanes each, which
-// shortens the longest walks; the rest walk one lane each.  The
-// rare paths (a cell whose Gram matrix is near singular, a walk that runs past
-// a truncated table) are not taken here: such a voxel goes to fix_list with
-// its bound, and k_tail_fix finishes it, so that this kernel's registers stay
-// those of the FP32 evaluation.
-constexpr int kCqRing = 64;               // ring of pending cells per warp
-constexpr int kCqMinWalking = 16;         // flush a partial batch below this many walking lanes
+// the costliest buckets walk 32, 8 or 4 lanes each (options group32_bucket,
+// group8_bucket, group_bucket), the rest one lane each.  The rare paths (a
+// cell whose Gram matrix is near singular, a bound past a truncated table) are
+// not taken here: such a voxel goes to fix_list with its bound, and k_tail_fix
+// finishes it, so that this kernel's registers stay those of the FP32
+// evaluation.
+//
+// What bounds it: issue (56 % at 25 % occupancy), about a third each in the
+// three tiers; the dose loads hit L1 at 92 %.  Before, one walker per lane or
+// group collected the cells past the dose gap alone and evaluated all of them
+// (21.8 per queued voxel of a 320x320x240 map at 3 %/3 mm, 36.5 at 1 %/1 mm
+// local; now 3.9 and 8.5): 10.5 ms there and 23.6 ms, now 3.6 ms and 10.2 ms
+// (twelve warps in each of two blocks per SM); 420 us and 180 us on a
+// 200x200x150 map at 2 %/2 mm.
+constexpr int kCqRing = 64;               // cells in each ring of a warp
 
-// Per-warp shared state.  A walker's state (one lane, or the first lane of a
-// group) lives here rather than in registers.
 struct CqWarp {
-    float q[8][kCqRing];       // vertex doses of a pending cell (relative, normalised)
-    unsigned off[kCqRing];     // its offset from the voxel, packed as in the table
-    unsigned meta[kCqRing];    // owner slot (bits 0-5), vertices inside the grid (bits 8-15)
-    unsigned best[64];         // running squared gamma per voxel slot (float bits)
-    unsigned vox[64];          // voxel index per slot
-    float dr[64];              // reference dose per slot
-    float inv[64];             // 1 / Delta D per slot
-    unsigned fixm[2];          // slots whose voxel goes to the finishing pass
-    int xyz[3][32];            // the walking voxel's grid position, per walker
-    int t[32];                 // its next table entry
-    unsigned wseq[32];         // sequence number of the last cell it appended
-    unsigned dseq[32];         // the same for the voxel in the drain slot
-    unsigned state[32];        // kCq* bits below
-    unsigned cnt[2][32];       // voxels finished and passed
-    int cpair[32];             // batched: the pair those counts belong to
-    unsigned short pair[64];   // batched: the pair of each voxel slot
-    unsigned long long stat[3][32];    // cells visited, pruned, keyed (option "stats")
+    unsigned ring[2][kCqRing]; // pending cells of tiers 2 and 3: table entry << 5 | slot of the voxel
+    unsigned best[32];         // per slot: running squared gamma (float bits),
+    unsigned vox[32];          // voxel, reference dose, 1 / Delta D, grid position,
+    float dr[32], inv[32];
+    int xyz[3][32];
+    unsigned skip[32];         // the plane seed's cell
+    unsigned short pair[32];   // batched: its pair
+    unsigned fixm;             // slots whose voxel goes to the finishing pass
 };
-// Batched launches: the walking voxel's grid and table, per walker, cached
-// when it takes the voxel (a pair's Problem lives in global memory).
-struct CqWalkDims {
-    int dim[4][32];            // nx, ny, nz, table length
-    const TableEntry* tab[32];
-    const float* ev[32];
-};
-constexpr unsigned kCqWalk = 1u, kCqEnded = 2u, kCqWPend = 4u, kCqDBusy = 8u, kCqDPend = 16u,
-                   kCqDOver = 32u, kCqSlot = 64u;     // slot bit: the walking slot is walker + 32
 
 // Lanes per voxel of the four parts of the queue.
 constexpr int kCqParts = 4;
@@ -1277,46 +1500,24 @@ __device__ __forceinline__ int cq_part_lanes(int part)
     return part == 0 ? 32 : (part == 1 ? 8 : (part == 2 ? 4 : 1));
 }
 
-// The problem a voxel slot belongs to: the launch's own, or (batched) that of
-// the slot's pair.
-template <bool BATCH>
-__device__ __forceinline__ const Problem& cq_prob(const Problem& P0, const BatchDesc* bd,
-                                                  volatile const CqWarp& V, int slot)
-{
-    if constexpr (BATCH) return bd->probs[V.pair[slot]];
-    else return P0;
-}
-
-// Hands a walker's counts to their pair (batched launches).
-__device__ __forceinline__ void cq_flush_counts(const BatchDesc* bd, volatile CqWarp& V, int w)
-{
-    const int pr = V.cpair[w];
-    if (pr >= 0) {
-        Counters* c = bd->probs[pr].ctr;
-        if (V.cnt[0][w]) atomicAdd(&c->n_eval, (unsigned long long)V.cnt[0][w]);
-        if (V.cnt[1][w]) atomicAdd(&c->n_pass, (unsigned long long)V.cnt[1][w]);
-    }
-    V.cnt[0][w] = 0;
-    V.cnt[1][w] = 0;
-}
-
 template <int N, int MINB, bool BATCH>
-__global__ void __launch_bounds__(256, MINB)
+__global__ void __launch_bounds__(cq_threads(MINB), MINB)
     k_tail_cq(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd)
 {
-    __shared__ CqWarp cqw[8];
-    __shared__ CqWalkDims cqd[BATCH ? 8 : 1];
+    __shared__ CqWarp cqw[cq_threads(MINB) / 32];
     __shared__ unsigned s_end[kCqParts];   // the parts of the queue end at these items
-    __shared__ float s_dnorm;              // single pair: its dose norm
+    __shared__ unsigned long long s_stat[4];   // option "stats": visited, pruned, keyed, lane slots
+    __shared__ unsigned s_cnt[2];          // single pair: voxels finished and passed
+    __shared__ unsigned s_start[kNumBuckets];  // ... first item of each cost bucket (the costliest is 0)
+    __shared__ float s_cells;              // ... estimated table cells of the whole queue
     CqWarp& W = cqw[threadIdx.x >> 5];
     volatile CqWarp& V = cqw[threadIdx.x >> 5];
-    volatile CqWalkDims& VD = cqd[BATCH ? threadIdx.x >> 5 : 0];
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
     if (threadIdx.x < 32) {
         if constexpr (BATCH) {
-            // the group's queue: voxels of bucket >= the group bucket of every
-            // pair first, then the rest (k_bucket_scan_batch)
+            // the group's queue: the parts of every pair, costliest part first
+            // (k_bucket_scan_batch)
             if (lane == 0) {
                 const int nb = kNumBuckets * bd->npairs;
                 s_end[0] = bd->item_start[nb + 1];
@@ -1341,287 +1542,334 @@ __global__ void __launch_bounds__(256, MINB)
                 h8 += __shfl_xor_sync(kFull, h8, o);
                 h4 += __shfl_xor_sync(kFull, h4, o);
             }
+            unsigned above = hb;               // items of this bucket and costlier ones
+            float cells = (float)hb * bucket_cells(lane);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned u = __shfl_down_sync(kFull, above, o);
+                if (lane + o < 32) above += u;
+                cells += __shfl_xor_sync(kFull, cells, o);
+            }
+            s_start[lane] = above - hb;
             if (lane == 0) {
-                s_dnorm = resolve_dnorm(P);
                 s_end[0] = min(h32, total);
                 s_end[1] = min(h8, total);
                 s_end[2] = min(h4, total);
                 s_end[3] = total;
+                s_cnt[0] = s_cnt[1] = 0;
+                s_cells = cells;
             }
+            if (lane < 4) s_stat[lane] = 0;
         }
     }
-    W.state[lane] = 0;
-    W.wseq[lane] = W.dseq[lane] = 0;
-    W.cnt[0][lane] = W.cnt[1][lane] = 0;
-    W.cpair[lane] = -1;
-    W.pair[lane] = W.pair[lane + 32] = 0;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) W.stat[k][lane] = 0;
-    if (lane < 2) W.fixm[lane] = 0;
+    if (lane == 0) W.fixm = 0;
     __syncthreads();
     unsigned* const heads = BATCH ? bd->part_head : P0.ctr->head_part;
+    const float dnorm0 = BATCH ? 0.f : resolve_dnorm(P0);
+    const bool stats = !BATCH && P0.stats;
+    const unsigned nwarps = gridDim.x * (blockDim.x >> 5);
 
-    int part = 0;                      // the part of the queue this warp takes voxels from
-    while (part < kCqParts - 1 && s_end[part] == (part ? s_end[part - 1] : 0u)) ++part;
-    int g = cq_part_lanes(part);       // its lanes per voxel
-    unsigned head = 0, count = 0;      // the ring: pending cells are [head, head + count)
-    bool queue_done = false;           // warp-uniform, for the current part
-    unsigned long long steps = 0;      // loop steps of this warp (option "stats")
-    for (;;) {
-        if (!BATCH && P0.stats) ++steps;
-        const int gl = lane & (g - 1), ld = lane - gl;
-        const bool leader = gl == 0;
-        const unsigned gmask = g == 32 ? kFull : ((1u << g) - 1u) << ld;
-        unsigned sta = V.state[ld];
-        if (leader) {
-            // 1. a drained voxel whose cells are all evaluated is final
-            if ((sta & kCqDBusy) && (!(sta & kCqDPend) || (int)(head - V.dseq[ld]) > 0)) {
-                const int ds = ld + ((sta & kCqSlot) ? 0 : 32);
-                const Problem& Q = cq_prob<BATCH>(P0, bd, V, ds);
-                const float best = __uint_as_float(V.best[ds]);
-                const unsigned v = V.vox[ds];
-                if (((V.fixm[ds >> 5] >> (ds & 31)) & 1u) ||
-                    ((sta & kCqDOver) && best > Q.r_cover * Q.r_cover)) {
-                    Q.out[v] = best;                        // gamma^2: k_tail_fix completes it
+    for (int part = 0; part < kCqParts; ++part) {
+        const unsigned lo = part ? s_end[part - 1] : 0u, hi = s_end[part];
+        if (lo >= hi) continue;
+        const int g = cq_part_lanes(part);         // lanes per voxel
+        const unsigned nv = 32u / (unsigned)g;     // voxels per round
+        unsigned nb = nv;                          // voxels per batch
+        unsigned at = lo;                          // where the queue stood when this warp last looked
+        const int gl = lane & (g - 1);
+        for (;;) {
+            // as many rounds per batch as keep it below an eighth of a warp's
+            // share of the queue's estimated cells, from the cost bucket at
+            // the last known position (costs only fall from there); in a
+            // batch group, whose parts mix pairs and costs, two rounds
+            if constexpr (BATCH) {
+                nb = min(32u, 2u * nv);
+            } else if (P0.sort_tail) {
+                const unsigned m = __ballot_sync(kFull, s_start[lane] <= at && (lane == 0 || s_start[lane - 1] > at));
+                const float share = s_cells / (8.f * (float)nwarps * bucket_cells(m ? 31 - __clz(m) : 0));
+                nb = min(32u, max(nv, (unsigned)fminf(share, 32.f) / nv * nv));
+            }
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(&heads[part], nb);
+            base = __shfl_sync(kFull, base, 0) + lo;
+            if (base >= hi) break;                 // warp-uniform
+            at = base;
+            const unsigned nlive = min(nb, hi - base);
+            // ---- the batch's voxels, one per lane ----
+            if ((unsigned)lane < nlive) {
+                const unsigned item = base + (unsigned)lane;
+                unsigned v, skip;
+                int pr = 0;
+                if constexpr (BATCH) {
+                    v = bd->items_v[item];
+                    pr = bd->items_p[item];
+                    skip = bd->items_s[item];
+                } else {
+                    v = P0.sort_tail ? P0.tail_sorted[item] : P0.tail_raw[item];
+                    skip = P0.sort_tail ? P0.plane_sorted[item] : P0.plane_raw[item];
+                }
+                const Problem& Q = BATCH ? bd->probs[pr] : P0;
+                const float dr = __ldg(Q.ref + v);
+                V.best[lane] = __float_as_uint(Q.out[v]);      // squared gamma, an upper bound
+                V.vox[lane] = v;
+                V.skip[lane] = skip;
+                V.xyz[0][lane] = (int)(v % (unsigned)Q.nx);
+                const unsigned r1 = v / (unsigned)Q.nx;
+                V.xyz[1][lane] = (int)(r1 % (unsigned)Q.ny);
+                V.xyz[2][lane] = (int)(r1 / (unsigned)Q.ny);
+                V.dr[lane] = dr;
+                V.inv[lane] = 1.0f / (Q.dd_frac * (Q.local ? dr : (BATCH ? resolve_dnorm(Q) : dnorm0)));
+                if (BATCH) V.pair[lane] = (unsigned short)pr;
+            }
+            __syncwarp();
+            unsigned head1 = 0, cnt1 = 0, head2 = 0, cnt2 = 0;   // the rings: [head, head + cnt)
+            unsigned r0 = 0;                       // first slot of the next round
+            int slot = 0, t = -1;                  // this lane's voxel and table entry (t < 0: no round)
+            for (;;) {
+                const bool rest = t < 0 && r0 >= nlive;        // every round is done: empty the rings
+                if (cnt2 >= 32u || (rest && cnt1 == 0u && cnt2 > 0u)) {
+                    // ---- tier 3: the faces of the oldest pending cells ----
+                    const unsigned n = min(cnt2, 32u);
+                    if ((unsigned)lane < n) {
+                        const unsigned w = V.ring[1][(head2 + (unsigned)lane) & (kCqRing - 1)];
+                        const int own = (int)(w & 31u);
+                        const Problem& O = BATCH ? bd->probs[V.pair[own]] : P0;
+                        const WalkEntry oe = O.walk[w >> 5];
+                        const float odr = V.dr[own], oinv = V.inv[own];
+                        const int onx = O.nx, osz = onx * O.ny;
+                        const int cx = unpack10(oe.off, 0), cy = unpack10(oe.off, 10), cz = unpack10(oe.off, 20);
+                        const bool ex = V.xyz[0][own] + cx + 1 < onx, ey = V.xyz[1][own] + cy + 1 < O.ny,
+                                   ez = N == 3 && V.xyz[2][own] + cz + 1 < O.nz;
+                        const float* q = O.ev + ((int)V.vox[own] + oe.lin);
+                        float cq[8];
+                        uint32_t ok = 0;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            cq[u] = kNaN;
+                            if (u < (1 << N) && (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
+                                cq[u] = rel_dose(__ldg(q + (u & 1) + ((u & 2) ? onx : 0) + ((u & 4) ? osz : 0)), odr, oinv);
+                                ok |= 1u << u;
+                            }
+                        }
+                        auto evaluate = [&](const Metric& mt, float dmax, float tau) {
+                            CellGeom<float> cg;
+                            cell_geom<N, float>(cx, cy, cz, mt, cg);
+                            bool ill = false;
+                            const float cb = cell_min_d2<N, float>(cq, cg, mt, dmax, kInf, ill);
+                            if (ill && cell_gram_ill<N>(cq, ok, mt.kappa, tau))
+                                atomicOr(&W.fixm, 1u << own);                  // k_tail_fix redoes it
+                            else
+                                atomicMin(&W.best[own], __float_as_uint(cb + 0.f));   // -0 -> +0
+                        };
+                        if constexpr (BATCH) {
+                            // the owner's pair's metric: three 16-byte loads
+                            const float4* m4 = bd->metric4 + 3 * (int)V.pair[own];
+                            const float4 a = __ldg(m4), b = __ldg(m4 + 1), c = __ldg(m4 + 2);
+                            Metric mt;
+                            mt.hn2[0] = a.x; mt.hn2[1] = a.y; mt.hn2[2] = a.z;
+                            mt.kappa[0] = 0.f;
+                            mt.kappa[1] = b.x; mt.kappa[2] = b.y; mt.kappa[3] = b.z; mt.kappa[4] = b.w;
+                            mt.kappa[5] = c.x; mt.kappa[6] = c.y; mt.kappa[7] = c.z;
+                            evaluate(mt, a.w > 0.f ? 0.99f * rsqrtf(a.w) : kInf, a.w);   // bound as ill_dmax
+                        } else {
+                            evaluate(P0.mt, ill_dmax(P0), P0.tau);
+                        }
+                    }
+                    head2 += n;
+                    cnt2 -= n;
+                    if (stats && lane == 0) atomicAdd(&s_stat[0], (unsigned long long)n);
+                    __syncwarp();
+                    continue;
+                }
+                if (cnt1 >= 32u || (rest && cnt1 > 0u)) {
+                    // ---- tier 2: plane_bound of the oldest cells past the dose gap ----
+                    const unsigned n = min(cnt1, 32u);
+                    bool cand = false;
+                    unsigned w = 0;
+                    if ((unsigned)lane < n) {
+                        w = V.ring[0][(head1 + (unsigned)lane) & (kCqRing - 1)];
+                        const int own = (int)(w & 31u);
+                        const Problem& O = BATCH ? bd->probs[V.pair[own]] : P0;
+                        const WalkEntry oe = O.walk[w >> 5];
+                        const int onx = O.nx, osz = onx * O.ny;
+                        const float* q = O.ev + ((int)V.vox[own] + oe.lin);
+                        float d[8];
+#pragma unroll
+                        for (int u = 0; u < (1 << N); ++u)
+                            d[u] = __ldg(q + (u & 1) + ((u & 2) ? onx : 0) + ((u & 4) ? osz : 0));
+                        const float c[3] = {(float)unpack10(oe.off, 0), (float)unpack10(oe.off, 10),
+                                            (float)unpack10(oe.off, 20)};
+                        float hn2[3], kap[3];
+                        if constexpr (BATCH) {
+                            const float4* m4 = bd->metric4 + 3 * (int)V.pair[own];
+                            const float4 ma = __ldg(m4), mb = __ldg(m4 + 1);
+                            hn2[0] = ma.x; hn2[1] = ma.y; hn2[2] = ma.z;
+                            kap[0] = mb.x; kap[1] = mb.y; kap[2] = mb.w;
+                        } else {
+                            hn2[0] = P0.mt.hn2[0]; hn2[1] = P0.mt.hn2[1]; hn2[2] = P0.mt.hn2[2];
+                            kap[0] = P0.mt.kappa[1]; kap[1] = P0.mt.kappa[2]; kap[2] = P0.mt.kappa[4];
+                        }
+                        const float ob = __uint_as_float(V.best[own]);
+                        cand = oe.off != V.skip[own] &&
+                               !(plane_bound<N>(d, c, V.dr[own], V.inv[own], hn2, kap) >= ob * kPlaneSlack);
+                    }
+                    head1 += n;
+                    cnt1 -= n;
+                    const unsigned cm = __ballot_sync(kFull, cand);
+                    if (cand) V.ring[1][(head2 + cnt2 + (unsigned)__popc(cm & lt_mask)) & (kCqRing - 1)] = w;
+                    cnt2 += (unsigned)__popc(cm);
+                    if (stats && lane == 0) atomicAdd(&s_stat[1], (unsigned long long)(n - (unsigned)__popc(cm)));
+                    __syncwarp();
+                    continue;
+                }
+                if (t < 0) {
+                    if (r0 >= nlive) break;                    // the batch is done
+                    slot = (int)r0 + lane / g;                 // the next round: nv voxels, g lanes each
+                    r0 += nv;
+                    t = gl;
+                }
+                // the lane's voxel (from shared memory after every pass of
+                // the other tiers, which so need not keep it in registers)
+                const bool live = (unsigned)slot < nlive;
+                const int sl = live ? slot : 0;
+                const Problem& Q = BATCH ? bd->probs[V.pair[sl]] : P0;
+                const int x = V.xyz[0][sl], y = V.xyz[1][sl], z = V.xyz[2][sl];
+                const int nx = Q.nx, sz = nx * Q.ny;
+                int reach = min(min(x, nx - 1 - x), min(y, Q.ny - 1 - y));   // cells of this margin lie in the grid
+                if (N == 3) reach = min(reach, min(z, Q.nz - 1 - z));
+                const float* const ev = Q.ev + V.vox[sl];
+                const WalkEntry* const tab = Q.walk;
+                const float dr = V.dr[sl], inv = V.inv[sl];
+                const float best = live ? __uint_as_float(V.best[sl]) : -1.f;   // < 0: nothing is below it
+                WalkEntry en = tab[t];
+                // ---- tier 1: one table entry per lane and step ----
+                do {
+                    const WalkEntry e = en;
+                    const bool keyed = e.key * e.key < best;
+                    if (!__any_sync(kFull, keyed)) {
+                        t = -1;
+                        break;
+                    }
+                    const unsigned ent = (unsigned)t;
+                    t += g;
+                    en = tab[t];                       // the table is padded with unreachable keys
+                    bool cand = false, edge = false;   // edge: a cell with vertices outside the grid
+                    if (keyed) {
+                        const float* q = ev + e.lin;
+                        float dlo, dhi;
+                        bool in = true;
+                        if (e.margin <= reach) {
+                            float d[8];
+#pragma unroll
+                            for (int u = 0; u < (1 << N); ++u)
+                                d[u] = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
+                            if constexpr (N == 3) {
+                                dlo = fminf(min3(min3(d[0], d[1], d[2]), d[3], d[4]), min3(d[5], d[6], d[7]));
+                                dhi = fmaxf(max3(max3(d[0], d[1], d[2]), d[3], d[4]), max3(d[5], d[6], d[7]));
+                            } else {
+                                dlo = fminf(min3(d[0], d[1], d[2]), d[3]);
+                                dhi = fmaxf(max3(d[0], d[1], d[2]), d[3]);
+                            }
+                        } else {
+                            // near the grid's faces: a cell outside it does not exist, one with
+                            // vertices outside keeps the faces that lie inside
+                            const int px = x + unpack10(e.off, 0), py = y + unpack10(e.off, 10), pz = z + unpack10(e.off, 20);
+                            in = (unsigned)px < (unsigned)nx && (unsigned)py < (unsigned)Q.ny &&
+                                 (N == 2 || (unsigned)pz < (unsigned)Q.nz);
+                            const bool ex = px + 1 < nx, ey = py + 1 < Q.ny, ez = N == 3 && pz + 1 < Q.nz;
+                            edge = !(ex && ey && (N == 2 || ez));
+                            dlo = kInf;
+                            dhi = -kInf;
+                            if (in) {
+#pragma unroll
+                                for (int u = 0; u < (1 << N); ++u) {
+                                    if ((!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
+                                        const float f = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
+                                        dlo = fminf(dlo, f);
+                                        dhi = fmaxf(dhi, f);
+                                    }
+                                }
+                            }
+                        }
+                        const float gap = max3(dlo - dr, dr - dhi, 0.f) * inv;
+                        cand = in && fmaf(gap, gap, e.key * e.key) < best;
+                    }
+                    // a whole cell goes to tier 2, one at the grid's edge to tier 3
+                    const unsigned cm = __ballot_sync(kFull, cand && !edge);
+                    if (cand && !edge)
+                        V.ring[0][(head1 + cnt1 + (unsigned)__popc(cm & lt_mask)) & (kCqRing - 1)] = ent << 5 | (unsigned)slot;
+                    cnt1 += (unsigned)__popc(cm);
+                    const unsigned em = __ballot_sync(kFull, cand && edge);
+                    if (em) {
+                        if (cand && edge)
+                            V.ring[1][(head2 + cnt2 + (unsigned)__popc(em & lt_mask)) & (kCqRing - 1)] = ent << 5 | (unsigned)slot;
+                        cnt2 += (unsigned)__popc(em);
+                    }
+                    if (stats) {
+                        const unsigned km = __ballot_sync(kFull, keyed), pm = __ballot_sync(kFull, keyed && !cand);
+                        if (lane == 0) {
+                            atomicAdd(&s_stat[1], (unsigned long long)__popc(pm));
+                            atomicAdd(&s_stat[2], (unsigned long long)__popc(km));
+                            atomicAdd(&s_stat[3], 32ull);
+                        }
+                    }
+                } while (max(cnt1, cnt2) < 32u);
+                __syncwarp();
+            }
+            // ---- final values, one voxel per lane ----
+            const unsigned fixm = V.fixm;
+            bool pass = false, fin = false;
+            int pr = 0;
+            if ((unsigned)lane < nlive) {
+                if (BATCH) pr = V.pair[lane];
+                const Problem& Q = BATCH ? bd->probs[pr] : P0;
+                const unsigned v = V.vox[lane];
+                const float b = __uint_as_float(V.best[lane]);
+                if (((fixm >> lane) & 1u) || b > Q.r_cover * Q.r_cover) {
+                    Q.out[v] = b;                              // squared gamma: k_tail_fix completes it
                     if constexpr (BATCH) {
                         const unsigned k = atomicAdd(bd->fix_count, 1u);
                         bd->fix_v[k] = v;
-                        bd->fix_p[k] = V.pair[ds];
+                        bd->fix_p[k] = (unsigned short)pr;
                     } else {
                         Q.fix_list[atomicAdd(&Q.ctr->fix_count, 1u)] = v;
                     }
                 } else {
-                    const float gam = sqrtf(best);
+                    const float gam = sqrtf(b);
                     Q.out[v] = gam;
-                    if constexpr (BATCH) {
-                        if (V.cpair[ld] != (int)V.pair[ds]) {
-                            cq_flush_counts(bd, V, ld);
-                            V.cpair[ld] = V.pair[ds];
-                        }
-                    }
-                    ++V.cnt[0][ld];
-                    if (gam <= 1.f) ++V.cnt[1][ld];
-                }
-                sta &= ~kCqDBusy;
-            }
-            // 2. an ended walk becomes the drain slot; the walker takes a new voxel
-            if ((sta & kCqEnded) && !(sta & kCqDBusy)) {
-                const int ws = ld + ((sta & kCqSlot) ? 32 : 0);
-                unsigned d = kCqDBusy;
-                if (sta & kCqWPend) d |= kCqDPend;
-                if (V.t[ld] >= (BATCH ? VD.dim[3][ld] : P0.ntable)) d |= kCqDOver;
-                V.dseq[ld] = V.wseq[ld];
-                sta = d | ((sta & kCqSlot) ^ kCqSlot);
-            }
-        }
-        // 3. refill the empty walkers from the current part of the queue
-        const bool empty = leader && !(sta & (kCqWalk | kCqEnded));
-        const unsigned need = __ballot_sync(kFull, empty);
-        if (need && !queue_done) {
-            const unsigned lo = part ? s_end[part - 1] : 0u, hi = s_end[part];
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(&heads[part], (unsigned)__popc(need));
-            base = __shfl_sync(kFull, base, 0) + lo;
-            if (base + (unsigned)__popc(need) >= hi) queue_done = true;
-            if (empty) {
-                const unsigned item = base + (unsigned)__popc(need & lt_mask);
-                if (item < hi) {
-                    const int ws = ld + ((sta & kCqSlot) ? 32 : 0);
-                    unsigned v;
-                    if constexpr (BATCH) {
-                        v = bd->items_v[item];
-                        V.pair[ws] = bd->items_p[item];
-                    } else {
-                        v = P0.sort_tail ? P0.tail_sorted[item] : P0.tail_raw[item];
-                    }
-                    const Problem& Q = cq_prob<BATCH>(P0, bd, V, ws);
-                    V.xyz[0][ld] = (int)(v % (unsigned)Q.nx);
-                    const unsigned r1 = v / (unsigned)Q.nx;
-                    V.xyz[1][ld] = (int)(r1 % (unsigned)Q.ny);
-                    V.xyz[2][ld] = (int)(r1 / (unsigned)Q.ny);
-                    const float dr = __ldg(Q.ref + v);
-                    V.dr[ws] = dr;
-                    V.inv[ws] = 1.0f / (Q.dd_frac * (Q.local ? dr : (BATCH ? resolve_dnorm(Q) : s_dnorm)));
-                    V.best[ws] = __float_as_uint(Q.out[v]);  // gamma^2 over the faces through v
-                    V.vox[ws] = v;
-                    if constexpr (BATCH) {
-                        VD.dim[0][ld] = Q.nx;
-                        VD.dim[1][ld] = Q.ny;
-                        VD.dim[2][ld] = Q.nz;
-                        VD.dim[3][ld] = Q.ntable;
-                        VD.tab[ld] = Q.table;
-                        VD.ev[ld] = Q.ev;
-                    }
-                    atomicAnd(&W.fixm[ws >> 5], ~(1u << (ws & 31)));
-                    V.t[ld] = 0;
-                    sta = (sta & ~kCqWPend) | kCqWalk;
+                    fin = true;
+                    pass = gam <= 1.f;
                 }
             }
-        }
-        if (leader) V.state[ld] = sta;
-        __syncwarp();
-        sta = V.state[ld];                 // the group's lanes follow their walker
-        if (queue_done && !__any_sync(kFull, (sta & (kCqWalk | kCqEnded | kCqDBusy)) != 0)) {
-            if (part == kCqParts - 1) break;
-            ++part;                        // this part is done: the next, with fewer lanes per voxel
-            g = cq_part_lanes(part);
-            queue_done = false;
-            V.state[lane] = 0;
+            const unsigned fm = __ballot_sync(kFull, fin), pm = __ballot_sync(kFull, pass);
+            if constexpr (BATCH) {
+                if (fin) {                         // one atomic per pair of the batch (almost always one)
+                    const unsigned peers = __match_any_sync(fm, pr);
+                    if (lane == __ffs(peers) - 1) {
+                        Counters* c = bd->probs[pr].ctr;
+                        atomicAdd(&c->n_eval, (unsigned long long)__popc(peers));
+                        if (pm & peers) atomicAdd(&c->n_pass, (unsigned long long)__popc(pm & peers));
+                    }
+                }
+            } else if (lane == 0) {
+                atomicAdd(&s_cnt[0], (unsigned)__popc(fm));
+                atomicAdd(&s_cnt[1], (unsigned)__popc(pm));
+            }
             __syncwarp();
-            continue;
+            if (lane == 0 && fixm) W.fixm = 0;
+            __syncwarp();
         }
-
-        // 4. one table step of every walking group: entries t .. t + g - 1
-        const bool walking = (sta & kCqWalk) != 0;
-        const int ws = ld + ((sta & kCqSlot) ? 32 : 0);
-        // the walking voxel's grid and table (batched: cached at its refill)
-        const int qnx = BATCH ? VD.dim[0][ld] : P0.nx, qny = BATCH ? VD.dim[1][ld] : P0.ny;
-        const int qnz = BATCH ? VD.dim[2][ld] : P0.nz, qnt = BATCH ? VD.dim[3][ld] : P0.ntable;
-        const TableEntry* qtab = BATCH ? VD.tab[ld] : P0.table;
-        const float* qev = BATCH ? VD.ev[ld] : P0.ev;
-        const bool qstats = !BATCH && P0.stats;
-        const int t0 = walking ? V.t[ld] : 0;
-        float key = kInf;
-        uint32_t off = 0;
-        if (walking && t0 + gl < qnt) {
-            const TableEntry e = qtab[t0 + gl];
-            key = e.key;
-            off = e.off;
-        }
-        const float k0 = __shfl_sync(kFull, key, ld);
-        bool cand = false, ended = false;
-        float q[8];
-        uint32_t ok = 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) q[u] = 0.f;
-        if (walking) {
-            const float bst = __uint_as_float(V.best[ws]);
-            ended = t0 >= qnt || k0 * k0 >= bst;              // A1 step 4b-ii, exact
-            if (!ended && key * key < bst) {
-                if (qstats) ++V.stat[2][lane];
-                const int px = V.xyz[0][ld] + unpack10(off, 0);
-                const int py = V.xyz[1][ld] + unpack10(off, 10);
-                const int pz = V.xyz[2][ld] + unpack10(off, 20);
-                if ((unsigned)px < (unsigned)qnx && (unsigned)py < (unsigned)qny &&
-                    (N == 2 || (unsigned)pz < (unsigned)qnz)) {
-                    const long long sy = qnx, sz = (long long)qnx * qny;
-                    const bool ex = px + 1 < qnx, ey = py + 1 < qny, ez = N == 3 && pz + 1 < qnz;
-                    const long long p = (long long)pz * sz + (long long)py * sy + px;
-                    const float dr = V.dr[ws], inv = V.inv[ws];
-                    float qmin = kInf, qmax = -kInf;
-#pragma unroll
-                    for (int u = 0; u < (1 << N); ++u) {
-                        const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
-                        if (present) {
-                            const long long o = p + ((u & 1) ? 1 : 0) + ((u & 2) ? sy : 0) +
-                                                ((u & 4) ? sz : 0);
-                            q[u] = (__ldg(qev + o) - dr) * inv;
-                            qmin = fminf(qmin, q[u]);
-                            qmax = fmaxf(qmax, q[u]);
-                            ok |= 1u << u;
-                        }
-                    }
-                    const float gap = qmin > 0.f ? qmin : (qmax < 0.f ? -qmax : 0.f);
-                    if (fmaf(gap, gap, key * key) >= bst) {
-                        if (qstats) ++V.stat[1][lane];
-                    } else {
-                        cand = true;
-                    }
-                }
-            }
-        }
-        // 5. append the surviving cells to the ring
-        const unsigned cm = __ballot_sync(kFull, cand);
-        if (cand) {
-            const unsigned seq = head + count + (unsigned)__popc(cm & lt_mask);
-            const int slot = (int)(seq & (kCqRing - 1));
-#pragma unroll
-            for (int u = 0; u < (1 << N); ++u) V.q[u][slot] = q[u];
-            V.off[slot] = off;
-            V.meta[slot] = (unsigned)ws | (ok << 8);
-        }
-        if (leader && walking) {
-            if (ended) {
-                sta = (sta & ~kCqWalk) | kCqEnded;
-            } else {
-                V.t[ld] = t0 + g;
-                const unsigned gm = cm & gmask;
-                if (gm) {                   // the group's last appended cell
-                    const int hl = 31 - __clz(gm);
-                    V.wseq[ld] = head + count + (unsigned)__popc(cm & ((1u << hl) - 1u));
-                    sta |= kCqWPend;
-                }
-            }
-            V.state[ld] = sta;
-        }
-        count += (unsigned)__popc(cm);
-        const int nwalk = g * __popc(__ballot_sync(kFull, leader && (sta & kCqWalk) && !ended));
-        __syncwarp();
-        // 6. evaluate the oldest 32 pending cells (or fewer, when few lanes walk)
-        if (count >= 32u || (count > 0u && nwalk < kCqMinWalking)) {
-            const unsigned n = min(count, 32u);
-            if ((unsigned)lane < n) {
-                const int slot = (int)((head + (unsigned)lane) & (kCqRing - 1));
-                const unsigned meta = V.meta[slot];
-                const int owner = (int)(meta & 63u);
-                const unsigned cok = meta >> 8;
-                const unsigned coff = V.off[slot];
-                float cq[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) cq[u] = u < (1 << N) ? V.q[u][slot] : 0.f;
-                auto evaluate = [&](const Metric& mt, float dmax, float tau) {
-                    CellGeom<float> cg;
-                    cell_geom<N, float>(unpack10(coff, 0), unpack10(coff, 10), unpack10(coff, 20), mt, cg);
-                    bool ill = false;
-                    const float cb = cell_min_d2<N, float>(cq, cok, cg, mt, dmax, kInf, ill);
-                    if (ill && cell_gram_ill<N>(cq, cok, mt.kappa, tau))
-                        atomicOr(&W.fixm[owner >> 5], 1u << (owner & 31));   // k_tail_fix redoes it
-                    else
-                        atomicMin(&W.best[owner], __float_as_uint(cb + 0.f));   // -0 -> +0
-                };
-                if constexpr (BATCH) {
-                    // the owner's pair's metric: three 16-byte loads
-                    const float4* m4 = bd->metric4 + 3 * (int)V.pair[owner];
-                    const float4 a = m4[0], b = m4[1], c = m4[2];
-                    Metric mt;
-                    mt.hn2[0] = a.x; mt.hn2[1] = a.y; mt.hn2[2] = a.z;
-                    mt.kappa[0] = 0.f;
-                    mt.kappa[1] = b.x; mt.kappa[2] = b.y; mt.kappa[3] = b.z; mt.kappa[4] = b.w;
-                    mt.kappa[5] = c.x; mt.kappa[6] = c.y; mt.kappa[7] = c.z;
-                    evaluate(mt, a.w > 0.f ? 0.99f * rsqrtf(a.w) : kInf, a.w);   // bound as ill_dmax
-                } else {
-                    evaluate(P0.mt, ill_dmax(P0), P0.tau);
-                }
-                if (!BATCH && P0.stats) ++V.stat[0][lane];
-            }
-            head += n;
-            count -= n;
-        }
-        __syncwarp();
     }
-    if constexpr (BATCH) {
-        cq_flush_counts(bd, V, lane);          // per-pair counts of every walker
-    } else {
-        // per-warp totals
-        const Problem& P = P0;
-        unsigned c0 = W.cnt[0][lane], c1 = W.cnt[1][lane];
-        unsigned long long s0 = W.stat[0][lane], s1 = W.stat[1][lane], s2 = W.stat[2][lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            c0 += __shfl_xor_sync(kFull, c0, o);
-            c1 += __shfl_xor_sync(kFull, c1, o);
-            s0 += __shfl_xor_sync(kFull, s0, o);
-            s1 += __shfl_xor_sync(kFull, s1, o);
-            s2 += __shfl_xor_sync(kFull, s2, o);
-        }
-        if (lane == 0) {
-            if (c0) atomicAdd(&P.ctr->n_eval, (unsigned long long)c0);
-            if (c1) atomicAdd(&P.ctr->n_pass, (unsigned long long)c1);
-            if (P.stats) {
-                atomicAdd(&P.ctr->cells_visited, s0);
-                atomicAdd(&P.ctr->cells_pruned, s1);
-                atomicAdd(&P.ctr->cells_keyed, s2);
-                atomicAdd(&P.ctr->lane_steps, 32ull * steps);
+    if constexpr (!BATCH) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (s_cnt[0]) atomicAdd(&P0.ctr->n_eval, (unsigned long long)s_cnt[0]);
+            if (s_cnt[1]) atomicAdd(&P0.ctr->n_pass, (unsigned long long)s_cnt[1]);
+            if (stats) {
+                atomicAdd(&P0.ctr->cells_visited, s_stat[0]);
+                atomicAdd(&P0.ctr->cells_pruned, s_stat[1]);
+                atomicAdd(&P0.ctr->cells_keyed, s_stat[2]);
+                atomicAdd(&P0.ctr->lane_steps, s_stat[3]);
             }
         }
     }
@@ -1759,7 +2007,7 @@ __device__ __forceinline__ float visit_cell_box(const Problem& P, const float* _
     float qmin = kInf, qmax = -kInf;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.f;
+        q[u] = kNaN;
         if (u < (1 << N)) {
             const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
             if (present) {
@@ -2534,6 +2782,15 @@ cudaError_t launch_patch_host(const Problem& P, float* host_out_mapped, Counters
     return cudaGetLastError();
 }
 
+cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s)
+{
+    if (!P.plane_raw) return cudaSuccess;
+    const int grid = grid_for(P.nvox, 256, device_sm_count() * 8);
+    if (P.ndim == 3) k_plane_seed<3, false><<<grid, 256, 0, s>>>(P, nullptr);
+    else k_plane_seed<2, false><<<grid, 256, 0, s>>>(P, nullptr);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_order_tail(const Problem& P, cudaStream_t s)
 {
     if (!P.sort_tail) return cudaSuccess;
@@ -2579,16 +2836,16 @@ template <int N, bool BATCH>
 static void launch_tail_cq_n(const Problem& P, const BatchDesc* bd, int per_sm, cudaStream_t s)
 {
     const int grid = device_sm_count() * per_sm;      // persistent: one wave of resident blocks
-    if (per_sm >= 4) k_tail_cq<N, 4, BATCH><<<grid, 256, 0, s>>>(P, bd);
-    else if (per_sm == 3) k_tail_cq<N, 3, BATCH><<<grid, 256, 0, s>>>(P, bd);
-    else if (per_sm == 2) k_tail_cq<N, 2, BATCH><<<grid, 256, 0, s>>>(P, bd);
-    else k_tail_cq<N, 1, BATCH><<<grid, 256, 0, s>>>(P, bd);
+    if (per_sm >= 4) k_tail_cq<N, 4, BATCH><<<grid, cq_threads(4), 0, s>>>(P, bd);
+    else if (per_sm == 3) k_tail_cq<N, 3, BATCH><<<grid, cq_threads(3), 0, s>>>(P, bd);
+    else if (per_sm == 2) k_tail_cq<N, 2, BATCH><<<grid, cq_threads(2), 0, s>>>(P, bd);
+    else k_tail_cq<N, 1, BATCH><<<grid, cq_threads(1), 0, s>>>(P, bd);
     k_tail_fix<N, BATCH><<<device_sm_count() * 2, 256, 0, s>>>(P, bd);
 }
 
 cudaError_t launch_tail_cq(const Problem& P, int tail_minblocks, cudaStream_t s)
 {
-    if (!P.fix_list) return cudaErrorInvalidValue;
+    if (!P.fix_list || !P.plane_raw) return cudaErrorInvalidValue;
     const int per_sm = std::min(4, std::max(1, tail_minblocks));
     if (P.ndim == 3) launch_tail_cq_n<3, false>(P, nullptr, per_sm, s);
     else launch_tail_cq_n<2, false>(P, nullptr, per_sm, s);
@@ -2695,6 +2952,16 @@ cudaError_t launch_batch_shell(const BatchGroup& g, int shell_minblocks, cudaStr
                                           SlabGate{nullptr, 0u, 0}, g.desc);
     else launch_shell_w_k<2, true>(per_sm, grid, s, dummy, map, 0, 0, g.total_tiles, g.shell_next,
                                           SlabGate{nullptr, 0u, 0}, g.desc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s)
+{
+    if (g.npairs <= 0) return cudaSuccess;
+    Problem dummy{};
+    const dim3 grid((unsigned)grid_for(g.max_nvox, 256, device_sm_count() * 4), (unsigned)g.npairs);
+    if (g.ndim == 3) k_plane_seed<3, true><<<grid, 256, 0, s>>>(dummy, g.desc);
+    else k_plane_seed<2, true><<<grid, 256, 0, s>>>(dummy, g.desc);
     return cudaGetLastError();
 }
 

@@ -152,7 +152,7 @@ __device__ __forceinline__ bool load_cell(const Problem& P, int x, int y, int z,
     ok = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.f;
+        q[u] = kNaN;
         if (u < (1 << N)) {
             const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
             if (present) {
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ Problem 
             CellGeom<float> g;
             cell_geom<N, float>(cx, cy, cz, P.mt, g);
             const float before = best;
-            cell_argmin<N, float>(q, ok, g, P.mt, best, foot);
+            cell_argmin<N, float>(q, g, P.mt, best, foot);
             if (best < before) {
                 fv[0] = cx + foot[0];
                 fv[1] = cy + foot[1];
@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(256) k_seed_apply(const __grid_constant__ Prob
                 CellGeom<float> gg;
                 cell_geom<N, float>(cx, cy, cz, P.mt, gg);
                 bool ill = false;
-                const float cb = cell_min_d2<N, float>(q, okc, gg, P.mt,
+                const float cb = cell_min_d2<N, float>(q, gg, P.mt,
                                                        P.tau > 0.f ? 0.99f * rsqrtf(P.tau) : kInf,
                                                        kInf, ill);
                 if (ill) ill = cell_gram_ill<N>(q, okc, P.mt.kappa, P.tau);

@@ -171,7 +171,7 @@ __device__ __forceinline__ float paper_cell(const Problem& P, int x, int y, int 
     uint32_t ok = 0;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        q[u] = 0.f;
+        q[u] = kNaN;
         if (u < (1 << N)) {
             const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
             if (present) {
