@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(256, MINB)
                 const int gx = x0 - 4 + bx, gy = y0 - 1 + by, gz = (N == 3 ? z0 - 1 : 0) + bz;
                 const bool in = (unsigned)gx < (unsigned)P.nx && (unsigned)gy < (unsigned)P.ny &&
                                 (N == 2 || (unsigned)gz < (unsigned)P.nz);
-                tl[i] = in ? __ldg(P.ev + ((long long)gz * P.ny + gy) * P.nx + gx) : 0.f;
+                tl[i] = in ? __ldg(P.ev + ((long long)gz * P.ny + gy) * P.nx + gx) : kNaN;
             }
             __syncthreads();
         }
@@ -298,21 +298,12 @@ __global__ void __launch_bounds__(256, MINB)
             bad_ev |= !isfinite(tl[tix0]);           // every evaluation dose is some tile's centre
         }
         const int tix = tix0;
-        uint32_t inm = 0, inp = 0;       // neighbours at -1 / +1 inside the grid, per axis
-        inm |= (x > 0) ? 1u : 0u;
-        inp |= (x + 1 < P.nx) ? 1u : 0u;
-        inm |= (y > 0) ? 2u : 0u;
-        inp |= (y + 1 < P.ny) ? 2u : 0u;
-        if (N == 3) {
-            inm |= (z > 0) ? 4u : 0u;
-            inp |= (z + 1 < P.nz) ? 4u : 0u;
-        }
         if (act) {
             const float dD = P.dd_frac * (P.local ? dr : dnorm);
             const float q0 = (tl[tix] - dr) / dD;
             best = q0 * q0;
             my_rmax = fmaxf(my_rmax, fabsf(q0));
-            if (best > 0.f) best = near_gamma2<N, T::BX, T::BX * T::BY>(tl, tix, inm, inp, dr, dD, P.mt.kappa);
+            if (best > 0.f) best = near_gamma2<N, T::BX, T::BX * T::BY>(tl, tix, dr, dD, P.mt.kappa);
         }
 
         // ---- finish or queue ----
@@ -406,7 +397,11 @@ __global__ void __launch_bounds__(256, MINB)
 // and takes its next tile from the work counter by itself: warps never wait
 // for one another until the end of the kernel.  Batched launches number the
 // tiles of all pairs of a group in one range; a warp keeps a copy of its
-// current pair's Problem in shared memory.
+// current pair's Problem in shared memory.  The next tile's number, pair, box
+// and reference doses are all requested a tile ahead (warps stalled on memory
+// half as often: 0.8 of 7 cycles per instruction; 454 to 418 us on a batch of
+// eight planes and eight volumes, 656 to 640 us with the plane seeds on a
+// 320x320x240 map).
 template <int N>
 struct WarpTile {
     static constexpr int TX = 32, TY = N == 3 ? 2 : 4, TZ = N == 3 ? 2 : 1;
@@ -424,6 +419,7 @@ __global__ void __launch_bounds__(256, MINB)
 {
     using T = WarpTile<N>;
     __shared__ __align__(128) float tiles[8][2][T::STRIDE];
+    __shared__ float refs[8][2][T::TX * T::TY * T::TZ];     // the tiles' reference doses
     __shared__ __align__(8) uint64_t bar[8][2];
     __shared__ __align__(16) Problem sh_P[BATCH ? 8 : 1];   // batched: each warp's current pair
     __shared__ unsigned int sh_hist[kNumBuckets];
@@ -470,26 +466,31 @@ __global__ void __launch_bounds__(256, MINB)
         z0 = (lt / ntx / nty) * T::TZ;
     };
     bool gate_failed = false;                 // lane 0: a slab wait gave up
-    // the copy of tile t's box into buffer b, by the whole warp: one TMA copy
+    // the copies of a tile (lt of pair pr) into buffer b, by the whole warp, a
+    // whole tile ahead of its use: its box of evaluation doses by one TMA copy
     // issued by lane 0, or, for a grid without a TMA map (its rows are not
-    // 16-byte aligned), 4-byte asynchronous copies by every lane; either way
-    // the box of the next tile is in flight while this one is computed.  One
-    // cp.async group per call (empty for TMA tiles), so that the group of
-    // the tile to compute is the second most recent one.  (Slab gates come
-    // only with a TMA map.)
-    auto issue = [&](int t, int b) {
+    // 16-byte aligned), by 4-byte asynchronous copies of every lane; its
+    // reference doses by such copies too, each lane its own.  One cp.async
+    // group per call, so that the group of the tile to compute is the second
+    // most recent one.  (Slab gates come only with a TMA map.)
+    constexpr int ROWS = T::TY * T::TZ;
+    auto issue = [&](int t, int pr, int lt, int tma, int b) {
         if (t < ntiles) {
-            int pr, lt;
-            locate(t, pr, lt);
             const Problem& Q = BATCH ? bd->probs[pr] : P0;
             int x0, y0, z0;
             origin(Q.nx, Q.ny, lt, x0, y0, z0);
-            if (BATCH ? bd->use_tma[pr] : use_tma0) {
+            const int nx = Q.nx, ny = Q.ny, nz = Q.nz;
+            if (tma) {
+                if constexpr (BATCH) {
+                    // the buffer may hold an earlier pair's box, written by the lanes
+                    fence_async_shared();
+                    __syncwarp();
+                }
                 if (lane == 0) {
                     const CUtensorMap* map = BATCH ? &bd->maps[pr] : &tmap0;
                     if (!BATCH && gate.flag && !gate_failed) {
                         // the box reads slices z0 - 1 .. z0 + TZ, from at most two slabs
-                        const int zlo = max(z0 - 1, 0), zhi = min(z0 + T::TZ, Q.nz - 1);
+                        const int zlo = max(z0 - 1, 0), zhi = min(z0 + T::TZ, nz - 1);
                         if (!flag_wait_bounded(gate.flag + zlo / gate.depth, gate.epoch) ||
                             !flag_wait_bounded(gate.flag + zhi / gate.depth, gate.epoch)) {
                             atomicOr(&Q.ctr->flags, kFlagTimeout);     // the run reports a timeout
@@ -501,8 +502,10 @@ __global__ void __launch_bounds__(256, MINB)
                     if (N == 3) tma_load_3d(tiles[w][b], map, x0 - 4, y0 - 1, z0 - 1, &bar[w][b]);
                     else tma_load_2d(tiles[w][b], map, x0 - 4, y0 - 1, &bar[w][b]);
                 }
+                // the other lanes wait here for lane 0's slab waits: polling the box's
+                // barrier meanwhile would slow lane 0's own polls down
+                if (!BATCH && gate.flag) __syncwarp();
             } else {
-                const int nx = Q.nx, ny = Q.ny, nz = Q.nz;
                 const float* ev = Q.ev;
                 float* dst = tiles[w][b];
                 for (int i = lane; i < T::ELEMS; i += 32) {
@@ -510,15 +513,29 @@ __global__ void __launch_bounds__(256, MINB)
                     const int gx = x0 - 4 + bx, gy = y0 - 1 + by, gz = (N == 3 ? z0 - 1 : 0) + bz;
                     const bool in = (unsigned)gx < (unsigned)nx && (unsigned)gy < (unsigned)ny &&
                                     (N == 2 || (unsigned)gz < (unsigned)nz);
-                    cp_async_f32(dst + i, ev + (in ? ((long long)gz * ny + gy) * nx + gx : 0), in);
+                    if (in) cp_async_f32(dst + i, ev + ((long long)gz * ny + gy) * nx + gx);
+                    else dst[i] = kNaN;             // a node outside the grid
                 }
+            }
+            const int x = x0 + lane;
+            const float* src = Q.ref + ((long long)z0 * ny + y0) * nx + x;
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const int ly = r % T::TY, lz = r / T::TY;
+                if (x < nx && y0 + ly < ny && z0 + lz < nz)
+                    cp_async_f32(&refs[w][b][r * 32 + lane], src + ((long long)lz * ny + ly) * nx);
             }
         }
         cp_async_commit();
     };
+    auto pair_tma = [&](int t, int pr) { return BATCH ? (t < ntiles ? bd->use_tma[pr] : 0) : use_tma0; };
     const int nwarps = (int)gridDim.x * 8;
-    int t = t_first + (int)blockIdx.x * 8 + w;     // the first tile of every warp, then the counter
-    issue(t, 0);
+    // the first two tiles of every warp, then the work counter, read a tile ahead
+    int t = t_first + (int)blockIdx.x * 8 + w, nt = t + nwarps;
+    int pr = 0, lt = 0;                       // the current tile's pair, and its number in the pair
+    if (t < ntiles) locate(t, pr, lt);
+    int tma = pair_tma(t, pr);
+    issue(t, pr, lt, tma, 0);
 
     unsigned my_eval = 0, my_pass = 0;
     float my_rmax = 0.f;
@@ -551,7 +568,7 @@ __global__ void __launch_bounds__(256, MINB)
         if (lane == 0) {
             if (my_eval) atomicAdd(&Q.ctr->n_eval, (unsigned long long)my_eval);
             if (my_pass) atomicAdd(&Q.ctr->n_pass, (unsigned long long)my_pass);
-            if (my_rmax > 0.f) atomicMax(&Q.ctr->rmax_enc, fenc(my_rmax));
+            if (my_rmax > 0.f) atomicMax(&Q.ctr->rmax_enc, fenc(Q.local ? my_rmax : my_rmax / (Q.dd_frac * dnorm)));
         }
         my_eval = my_pass = 0;
         my_rmax = 0.f;
@@ -593,12 +610,12 @@ __global__ void __launch_bounds__(256, MINB)
     };
 
     while (t < ntiles) {
-        int nt = 0;
-        if (lane == 0) nt = t_first + nwarps + (int)atomicAdd(tile_next, 1u);
-        nt = __shfl_sync(kFull, nt, 0);
-        issue(nt, b ^ 1);
-        int pr, lt;
-        locate(t, pr, lt);
+        unsigned nn = 0;                       // the tile after next
+        if (lane == 0) nn = atomicAdd(tile_next, 1u);
+        int npr = 0, nlt = 0;
+        if (nt < ntiles) locate(nt, npr, nlt);
+        const int ntma = pair_tma(nt, npr);
+        issue(nt, npr, nlt, ntma, b ^ 1);
         if constexpr (BATCH) {
             if (pr != cur) {                   // warp-uniform
                 if (cur >= 0) {
@@ -618,88 +635,79 @@ __global__ void __launch_bounds__(256, MINB)
         float* tl = tiles[w][b];
         int x0, y0, z0;
         origin(P.nx, P.ny, lt, x0, y0, z0);
-        // the tile's reference doses, loaded while its staged box may still
-        // be in flight (row r in drq[0] when row r is processed)
-        constexpr int ROWS = T::TY * T::TZ;
-        float drq[ROWS];
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const int x = x0 + lane, y = y0 + r % T::TY, z = z0 + r / T::TY;
-            drq[r] = (x < P.nx && y < P.ny && z < P.nz) ? __ldg(P.ref + ((long long)z * P.ny + y) * P.nx + x)
-                                                         : 0.f;
-        }
-        if (BATCH ? bd->use_tma[pr] : use_tma0) {
+        cp_async_wait<1>();                    // this tile's copies (the next tile's may be in flight)
+        if (tma) {
             if (!mbar_wait_bounded(&bar[w][b], (parity >> b) & 1u)) {
                 timed_out = true;              // (warp-uniform: every lane polls the same phase)
                 break;
             }
             parity ^= 1u << b;
         } else {
-            cp_async_wait<1>();                // this tile's copies (the next tile's may be in flight)
             __syncwarp();
         }
 #pragma unroll 1
-        for (int r = 0; r < ROWS; ++r) {
+        for (int r = 0; r < ROWS; r += 2) {        // rows y and y + 1 together
             const int ly = r % T::TY, lz = r / T::TY;
             const int x = x0 + lane, y = y0 + ly, z = z0 + lz;
-            const bool inside = x < P.nx && y < P.ny && z < P.nz;
-            const long long v = inside ? ((long long)z * P.ny + y) * P.nx + x : 0;
             const int tix = ((N == 3 ? lz + 1 : 0) * T::BY + (ly + 1)) * T::BX + (lane + 4);
-            const float dr = drq[0];
-#pragma unroll
-            for (int k = 0; k + 1 < ROWS; ++k) drq[k] = drq[k + 1];
-            float best = 0.f;
-            bool act = false;
-            if (inside) {
-                act = is_evaluated(P, dr, thr);
-                if (!act) P.out[v] = __int_as_float(0x7fc00000);
+            const float dr[2] = {refs[w][b][r * 32 + lane], refs[w][b][r * 32 + 32 + lane]};
+            const bool in0 = x < P.nx && y < P.ny && z < P.nz, in1 = in0 && y + 1 < P.ny;
+            const bool act[2] = {in0 && is_evaluated(P, dr[0], thr), in1 && is_evaluated(P, dr[1], thr)};
+            float* const out = P.out + (in0 ? ((long long)z * P.ny + y) * P.nx + x : 0);
+            if (in0) {
+                if (!act[0]) out[0] = kNaN;
                 bad_ev |= !isfinite(tl[tix]);       // every evaluation dose is some tile's centre
             }
-            uint32_t inm = 0, inp = 0;         // neighbours at -1 / +1 inside the grid, per axis
-            inm |= (x > 0) ? 1u : 0u;
-            inp |= (x + 1 < P.nx) ? 1u : 0u;
-            inm |= (y > 0) ? 2u : 0u;
-            inp |= (y + 1 < P.ny) ? 2u : 0u;
-            if (N == 3) {
-                inm |= (z > 0) ? 4u : 0u;
-                inp |= (z + 1 < P.nz) ? 4u : 0u;
+            if (in1) {
+                if (!act[1]) out[P.nx] = kNaN;
+                bad_ev |= !isfinite(tl[tix + T::BX]);
             }
-            if (act) {
-                const float dD = P.dd_frac * (P.local ? dr : dnorm);
-                const float q0 = (tl[tix] - dr) / dD;
-                best = q0 * q0;
-                my_rmax = fmaxf(my_rmax, fabsf(q0));
-                if (best > 0.f) best = near_gamma2<N, T::BX, T::BX * T::BY>(tl, tix, inm, inp, dr, dD, P.mt.kappa);
+            float best[2] = {0.f, 0.f};
+            if (act[0] || act[1]) {
+                const float dD0 = P.dd_frac * (P.local ? dr[0] : dnorm), dD1 = P.dd_frac * (P.local ? dr[1] : dnorm);
+                // gamma0 = |g| / dD; with one dD for all voxels the division waits for the maximum
+                const float g0 = fabsf(tl[tix] - dr[0]), g1 = fabsf(tl[tix + T::BX] - dr[1]);
+                if (P.local) my_rmax = max3(my_rmax, act[0] ? g0 / dD0 : 0.f, act[1] ? g1 / dD1 : 0.f);
+                else my_rmax = max3(my_rmax, act[0] ? g0 : 0.f, act[1] ? g1 : 0.f);
+                near_gamma2_pair<N, T::BX, T::BX * T::BY>(tl, tix, dr[0], dr[1], dD0, dD1, P.mt.kappa, best[0],
+                                                          best[1]);
             }
-            bool tail = false;
-            int bucket = 0;
-            if (act) {
-                tail = best > qlim;
-                if (tail) {
-                    P.out[v] = best;                   // gamma^2, finished by the table walk
-                    // 1 + floor(2 log2 of the table cells with key < gamma)
-                    bucket = cost_bucket_of(P.bucket_key, sqrtf(best));
-                } else {
-                    const float gam = sqrtf(best);
-                    P.out[v] = gam;
-                    ++my_eval;
-                    my_pass += gam <= 1.f;             // decided on the value written
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                bool tail = false;
+                int bucket = 0;
+                if (act[k]) {
+                    tail = best[k] > qlim;
+                    if (tail) {
+                        out[k ? P.nx : 0] = best[k];       // gamma^2, finished by the table walk
+                        // 1 + floor(2 log2 of the table cells with key < gamma)
+                        bucket = cost_bucket_of(P.bucket_key, sqrtf(best[k]));
+                    } else {
+                        const float gam = sqrtf(best[k]);
+                        out[k ? P.nx : 0] = gam;
+                        ++my_eval;
+                        my_pass += gam <= 1.f;             // decided on the value written
+                    }
                 }
-            }
-            const unsigned tm = __ballot_sync(kFull, tail);
-            if (tm) {
-                if (qn + 32 > kShellQ) flush_queue(P);
-                if (tail) {
-                    const int i = qn + __popc(tm & ((1u << lane) - 1u));
-                    qv[w][i] = (unsigned)v;
-                    qb[w][i] = (unsigned char)bucket;
+                const unsigned tm = __ballot_sync(kFull, tail);
+                if (tm) {
+                    if (qn + 32 > kShellQ) flush_queue(P);
+                    if (tail) {
+                        const int i = qn + __popc(tm & ((1u << lane) - 1u));
+                        qv[w][i] = (unsigned)(((long long)z * P.ny + y + k) * P.nx + x);
+                        qb[w][i] = (unsigned char)bucket;
+                    }
+                    qn += __popc(tm);
+                    __syncwarp();
                 }
-                qn += __popc(tm);
-                __syncwarp();
             }
         }
         __syncwarp();                          // tiles[w][b] is free for the copy after next
         t = nt;
+        pr = npr;
+        lt = nlt;
+        tma = ntma;
+        nt = t_first + 2 * nwarps + (int)__shfl_sync(kFull, nn, 0);
         b ^= 1;
     }
     cp_async_wait<0>();                        // no copy into this block's memory outlives it
@@ -731,6 +739,7 @@ __global__ void __launch_bounds__(256, MINB)
         if (lane == 0) {
             if (my_eval) atomicAdd(&sh_eval, (unsigned long long)my_eval);
             if (my_pass) atomicAdd(&sh_pass, (unsigned long long)my_pass);
+            if (!P0.local && my_rmax > 0.f) my_rmax /= P0.dd_frac * dnorm;
             atomicMax(&sh_rmax, fenc(my_rmax));
             if (bad) sh_bad = 1;
         }
@@ -1221,20 +1230,6 @@ __global__ void __launch_bounds__(256, MINB)
 // --------------------------------------------------------------------------
 // Plane seeds: a queued voxel's bound before its table walk
 // --------------------------------------------------------------------------
-
-// minimum / maximum of three (one instruction on sm_100 and later)
-__device__ __forceinline__ float min3(float a, float b, float c)
-{
-    float r;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
 
 // The affine part of the 2^N vertex doses e of a cell: the value m at the
 // cell's centre, the slope G per voxel along each axis, and eps, a bound on
@@ -2598,12 +2593,15 @@ bool encode_bf16_2d(CUtensorMap* map, const void* base, unsigned long long inner
                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map of the evaluation dose with a tile box of (bx, by, bz) floats;
-// false when TMA cannot be used for it.
-static bool encode_box_map(const Problem& P, CUtensorMap* map, int bx, int by, int bz)
+// Tensor map of the evaluation dose with a tile box of (bx, by, bz) floats,
+// zeros or NaN (nan_fill) outside the grid; false when TMA cannot be used for
+// it.
+static bool encode_box_map(const Problem& P, CUtensorMap* map, int bx, int by, int bz, bool nan_fill = false)
 {
     const EncodeFn encode = tensor_map_encoder();
     if (!encode) return false;
+    const CUtensorMapFloatOOBfill fill =
+        nan_fill ? CU_TENSOR_MAP_FLOAT_OOB_FILL_NAN_REQUEST_ZERO_FMA : CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE;
     if (((uintptr_t)P.ev & 15u) != 0 || (P.nx % 4) != 0) return false;   // TMA alignment rules
     if (P.ndim == 3) {
         const cuuint64_t dims[3] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, (cuuint64_t)P.nz};
@@ -2612,8 +2610,7 @@ static bool encode_box_map(const Problem& P, CUtensorMap* map, int bx, int by, i
         const cuuint32_t es[3] = {1, 1, 1};
         return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, (void*)P.ev, dims, strides, box, es,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, fill) == CUDA_SUCCESS;
     }
     const cuuint64_t dims[2] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny};
     const cuuint64_t strides[1] = {(cuuint64_t)P.nx * 4};
@@ -2621,8 +2618,7 @@ static bool encode_box_map(const Problem& P, CUtensorMap* map, int bx, int by, i
     const cuuint32_t es[2] = {1, 1};
     return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)P.ev, dims, strides, box, es,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, fill) == CUDA_SUCCESS;
 }
 
 // The shell of a run uses k_shell_w (warp tiles) unless a staged walk needs
@@ -2632,10 +2628,10 @@ static bool warp_tiled(const Problem& P) { return !P.tile_mask && !P.row_items; 
 bool encode_tile_map(const Problem& P, CUtensorMap* map)
 {
     if (warp_tiled(P))
-        return P.ndim == 3 ? encode_box_map(P, map, WarpTile<3>::BX, WarpTile<3>::BY, WarpTile<3>::BZ)
-                           : encode_box_map(P, map, WarpTile<2>::BX, WarpTile<2>::BY, 1);
-    return P.ndim == 3 ? encode_box_map(P, map, ShellTile<3>::BX, ShellTile<3>::BY, ShellTile<3>::BZ)
-                       : encode_box_map(P, map, ShellTile<2>::BX, ShellTile<2>::BY, 1);
+        return P.ndim == 3 ? encode_box_map(P, map, WarpTile<3>::BX, WarpTile<3>::BY, WarpTile<3>::BZ, true)
+                           : encode_box_map(P, map, WarpTile<2>::BX, WarpTile<2>::BY, 1, true);
+    return P.ndim == 3 ? encode_box_map(P, map, ShellTile<3>::BX, ShellTile<3>::BY, ShellTile<3>::BZ, true)
+                       : encode_box_map(P, map, ShellTile<2>::BX, ShellTile<2>::BY, 1, true);
 }
 
 template <class T>

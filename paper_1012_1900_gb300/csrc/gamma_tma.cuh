@@ -86,15 +86,11 @@ __device__ __forceinline__ void fence_async_shared()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// 2D / 3D tiled TMA loads into shared memory, completing on `bar`.  The
-// innermost coordinate x must be a multiple of 4 (16 bytes of float32).
 // One float from global to shared memory by an asynchronous copy (cp.async,
-// 4 bytes, no alignment rule); in == false reads nothing and writes 0.
-__device__ __forceinline__ void cp_async_f32(float* dst, const float* src, bool in)
+// 4 bytes, no alignment rule).
+__device__ __forceinline__ void cp_async_f32(float* dst, const float* src)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_addr(dst)), "l"(src),
-                 "r"(in ? 4 : 0)
-                 : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 
 // Close the thread's current group of cp.async copies.
@@ -110,6 +106,8 @@ __device__ __forceinline__ void cp_async_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// 2D / 3D tiled TMA loads into shared memory, completing on `bar`.  The
+// innermost coordinate x must be a multiple of 4 (16 bytes of float32).
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
                                             uint64_t* bar)
 {
