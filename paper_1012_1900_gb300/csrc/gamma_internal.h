@@ -340,8 +340,10 @@ bool model_weights(const gamma_model_s* m, MlpWeights* w);
 // on the tensor cores (P.seed_Y) and the exact seeds from the proposals.
 cudaError_t launch_seeding(const Problem& P, const MlpWeights& W, int min_bucket, cudaStream_t s);
 // Network outputs for M feature rows (row-major [M][384] BF16, 16-byte aligned).
+// host_flags: device address of a page-locked host word that gets kFlagTimeout
+// if a bounded wait gave up.
 cudaError_t launch_mlp_infer(const MlpWeights& W, const __nv_bfloat16* X, long long M, float* Y,
-                             unsigned* flags, cudaStream_t s);
+                             unsigned* host_flags, cudaStream_t s);
 
 // Reference and evaluation doses on different grids (gamma_grids.cu).
 // Positions and spacings are in DTA units, axes (x, y, z).
@@ -401,11 +403,12 @@ cudaError_t launch_batch_order(const BatchGroup& g, cudaStream_t s);
 cudaError_t launch_batch_tail(const BatchGroup& g, int walk, int lanes_per_voxel, int tail_minblocks,
                               cudaStream_t s);
 // Tensor map of a row-major bf16 matrix (inner elements x rows, row stride in
-// bytes) with boxes of box_inner x box_rows elements; false when the driver's
-// encoder is missing or the alignment rules fail.
+// bytes) with boxes of box_inner x box_rows elements (swizzle: boxes of 64
+// columns with the 128-byte swizzle); false when the driver's encoder is
+// missing or the alignment rules fail.
 bool encode_bf16_2d(CUtensorMap* map, const void* base, unsigned long long inner,
                     unsigned long long rows, unsigned long long row_stride_bytes,
-                    unsigned box_inner, unsigned box_rows);
+                    unsigned box_inner, unsigned box_rows, bool swizzle = false);
 // C (+)= A B^T on the tensor cores (gamma_gemm_tc.cu): A [M][K] and B [N][K]
 // bf16 with K contiguous (row strides lda, ldb: multiples of 8 elements, bases
 // 16-byte aligned), C fp32 [M][ldc].  With splits > 1 the K range is split over

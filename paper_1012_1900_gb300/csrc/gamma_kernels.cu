@@ -2579,7 +2579,7 @@ static EncodeFn tensor_map_encoder()
 
 bool encode_bf16_2d(CUtensorMap* map, const void* base, unsigned long long inner,
                     unsigned long long rows, unsigned long long row_stride_bytes,
-                    unsigned box_inner, unsigned box_rows)
+                    unsigned box_inner, unsigned box_rows, bool swizzle)
 {
     const EncodeFn encode = tensor_map_encoder();
     if (!encode || ((uintptr_t)base & 15u) || (row_stride_bytes & 15u) || (box_inner * 2) % 16) return false;
@@ -2589,8 +2589,10 @@ bool encode_bf16_2d(CUtensorMap* map, const void* base, unsigned long long inner
     const cuuint32_t es[2] = {1, 1};
     std::memset(map, 0, sizeof(*map));
     return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+                  es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  swizzle ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Tensor map of the evaluation dose with a tile box of (bx, by, bz) floats,

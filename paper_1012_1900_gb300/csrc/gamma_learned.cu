@@ -378,41 +378,52 @@ __global__ void k_cast_weights(const float* __restrict__ W1, const float* __rest
 // --------------------------------------------------------------------------
 // Network inference on the fifth-generation tensor cores (tcgen05)
 //
-// One block of 256 threads per SM keeps the three weight matrices resident in
-// shared memory in the no-swizzle K-major core-matrix layout (8 rows x 16
-// bytes per core matrix; core matrices adjacent in K are LBO = rows/8 * 128
-// bytes apart, adjacent 8-row groups SBO = 128 bytes apart) and runs 128
-// feature rows at a time.  The rows arrive by TMA: each 64-column chunk is
-// eight boxes of 8 columns x 128 rows, which land in exactly that layout,
-// through three stages (one "full" and one "empty" mbarrier each).  One thread
-// issues the copies and the MMAs: layer 1 accumulates X W1^T over the six
-// chunks in TMEM columns 0..127, and as soon as its last MMAs are committed
-// the first three chunks of the block's next tile are copied in, overlapping
-// the rest of this tile.  The epilogues read TMEM with tcgen05.ld (warp w
-// reads lanes 32 (w % 4) .. +31), add the bias, apply the ReLU and write the
-// next layer's BF16 operand: H1 W2^T goes to columns 128..255, then H2 (over
-// H1, whose MMAs have completed) times W3^T (N padded to 16) to columns
-// 0..15.  Every wait is bounded.
+// One block per SM keeps the three weight matrices resident in shared memory
+// and runs 128 feature rows at a time, each of its warps in one role:
+//   warp 8   copies the rows: 64-column panels of 128 rows x 128 bytes by TMA
+//            (128-byte swizzle) through three stages, always three ahead;
+//   warp 9   issues layer 1, X W1^T over the six panels, into two accumulators
+//            in turn (TMEM columns 0..127, 128..255), so that the rows keep
+//            arriving while the tile before is finished;
+//   warp 10  issues layers 2 and 3: H1 W2^T in columns 256..383, H2 W3^T (N
+//            padded to 16) in 384..399;
+//   warps 0-7 the epilogues: TMEM to registers (warp w reads lanes 32 (w % 4)
+//            .. +31), bias and ReLU, and the next layer's BF16 operand into
+//            shared memory (H2 over H1, whose MMAs have completed), no-swizzle
+//            K-major core-matrix layout (8 rows x 16 bytes per core matrix).
+// Everything between the roles is an mbarrier; every wait is bounded.
+//
+// What bounds it: reading the rows (768 bytes each).  A panel used to arrive
+// as eight boxes of 16-byte rows, and one thread took copies, MMAs and
+// epilogues in turn: 204 us for 262,144 rows (0.99 TB/s).  With whole 128-byte
+// rows per box and the roles apart it takes 61 us with one thread issuing all
+// three layers, and 50 us with layer 1 apart (4.0 TB/s); three panels (48 KB)
+// in flight per SM is what the weights leave room for.
 // --------------------------------------------------------------------------
 
 constexpr int kRows = 128;                 // rows per tile (MMA M)
-constexpr int kKc = 64;                    // K chunk of the streamed features
+constexpr int kKc = 64;                    // columns of a panel of streamed features
 constexpr int kNChunks = kInPad / kKc;     // 6
-constexpr int kXStages = 3;                // chunk stages in flight (divides kNChunks)
-static_assert(kNChunks % kXStages == 0, "chunk c of every tile must use stage c % kXStages");
+constexpr int kXStages = 3;                // panels in flight
 constexpr int kN3 = 16;                    // layer-3 N (4 outputs, padded)
-constexpr int kTmemCols = 256;
+constexpr int kTmemCols = 512;             // 400 used; allocations are powers of two
+constexpr int kMlpThreads = 352;
+constexpr int kEpiWarps = 8;
+constexpr int kStagers = kMlpThreads - 32; // threads that stage the weights: all but the copying warp's
+constexpr int kPanel = kRows * kKc;        // elements of a panel (rows 128)
 
 struct __align__(1024) TcSmem {
-    bf16 W1[kH * kInPad];                  // rows 128, K 384 (core-matrix layout)
-    bf16 W2[kH * kH];                      // rows 128, K 128
-    bf16 H[kRows * kH];                    // H1, then H2 (rows 128, K 128)
-    bf16 Xc[kXStages][kRows * kKc];        // feature chunks (TMA destinations)
+    bf16 W1[kNChunks][kPanel];             // rows 128, 64-column panels (128-byte swizzle)
+    bf16 Xc[kXStages][kPanel];             // feature panels (TMA destinations, 128-byte swizzle)
+    bf16 W2[kH * kH];                      // rows 128, K 128 (core-matrix layout)
+    bf16 H[kRows * kH];                    // H1, then H2 (rows 128, K 128; core-matrix layout)
     bf16 W3[kN3 * kH];                     // rows 16, K 128 (rows >= kOut zero)
     float b1[kH], b2[kH], b3[kOutPad];
-    uint64_t xfull[kXStages], xempty[kXStages], mma;
+    uint64_t xfull[kXStages], xempty[kXStages];
+    uint64_t d1[2], d2, d3;                // a layer's accumulator is complete
+    uint64_t e1[2];                        // layer 1's accumulator is read (one arrival per epilogue warp)
+    uint64_t h1, h2;                       // a layer's operand is written (likewise)
     uint32_t tmem;
-    int ok;
 };
 
 // Element index of (row, k) in a core-matrix tile with `rows` rows.
@@ -428,12 +439,18 @@ __device__ __forceinline__ uint64_t tile_desc(const bf16* base, int rows, int k0
     return smem_desc(smem_addr(base) + (uint32_t)(k0 >> 3) * lbo, lbo, 128u);
 }
 
+// Index of a weight-staging thread (every warp but the copying one).
+__device__ __forceinline__ int stager()
+{
+    return (int)threadIdx.x - ((int)threadIdx.x >= kEpiWarps * 32 ? 32 : 0);
+}
+
 // Row-major [rows][K] BF16 weights (global) -> core-matrix tile (shared).
 __device__ __forceinline__ void stage_weights(bf16* dst, const bf16* __restrict__ src, int rows,
                                               int src_rows, int K)
 {
     const int n = rows * (K / 8);
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    for (int e = stager(); e < n; e += kStagers) {
         const int r = e / (K / 8), j = e % (K / 8);
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (r < src_rows) v = *reinterpret_cast<const uint4*>(src + (long long)r * K + j * 8);
@@ -441,19 +458,30 @@ __device__ __forceinline__ void stage_weights(bf16* dst, const bf16* __restrict_
     }
 }
 
+// Row-major [128][384] BF16 weights (global) -> swizzled 64-column panels.
+__device__ __forceinline__ void stage_panels(bf16 (*dst)[kPanel], const bf16* __restrict__ src)
+{
+#pragma unroll 8
+    for (int e = stager(); e < kH * (kInPad / 8); e += kStagers) {
+        const int r = e / (kInPad / 8), j = e % (kInPad / 8);
+        *reinterpret_cast<uint4*>(dst[j >> 3] + r * kKc + (((j & 7) ^ (r & 7)) << 3)) =
+            *reinterpret_cast<const uint4*>(src + (long long)r * kInPad + j * 8);
+    }
+}
+
 // D (TMEM, 128 lanes x 128 columns from column `col`) + bias, ReLU -> BF16
-// core-matrix tile `dst` (rows 128, K 128).
+// core-matrix tile `dst` (rows 128, K 128); warps 0-7, half the columns each.
 __device__ __forceinline__ void epilogue_relu(uint32_t tmem, uint32_t col, const float* bias, bf16* dst)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = warp & 3, half = warp >> 2, row = 32 * q + lane;
 #pragma unroll 1
-    for (int j = 0; j < 4; ++j) {
-        const int c0 = half * 64 + j * 16;
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + col + (uint32_t)c0, v);
+    for (int j = 0; j < 2; ++j) {
+        const int c0 = half * 64 + j * 32;
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + col + (uint32_t)c0, v);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < 4; ++h) {
             uint32_t w[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -475,10 +503,13 @@ static_assert(sizeof(TcSmem) + 1024 <= kTcSmemBytes, "tensor-core tile does not 
 
 // Network outputs Y [rows][4] of the feature rows X [rows][384] (bf16, read by
 // the tensor map xmap), for rows < (*count_dev if given, capped at M, else M).
-__global__ void __launch_bounds__(256, 1) k_mlp_rows(const __grid_constant__ MlpWeights W,
-                                                     const __grid_constant__ CUtensorMap xmap,
-                                                     long long M, const unsigned* count_dev,
-                                                     float* __restrict__ Y, unsigned* flags)
+// A timed-out wait sets kFlagTimeout in *flags (host_flags: page-locked host
+// memory, written by a plain store).
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_rows(const __grid_constant__ MlpWeights W,
+                                                             const __grid_constant__ CUtensorMap xmap,
+                                                             long long M, const unsigned* count_dev,
+                                                             float* __restrict__ Y, unsigned* flags,
+                                                             int host_flags)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -487,130 +518,146 @@ __global__ void __launch_bounds__(256, 1) k_mlp_rows(const __grid_constant__ Mlp
     const long long nrows = count_dev ? min((long long)*count_dev, M) : M;
     const long long ntiles = (nrows + kRows - 1) / kRows;
     if ((long long)blockIdx.x >= ntiles) return;                  // block-uniform
-    stage_weights(S.W1, W.W1, kH, kH, kInPad);
-    stage_weights(S.W2, W.W2, kH, kH, kH);
-    stage_weights(S.W3, W.W3, kN3, kOutPad, kH);
-    for (int i = tid; i < kH; i += blockDim.x) {
-        S.b1[i] = W.b1[i];
-        S.b2[i] = W.b2[i];
-    }
-    if (tid < kOutPad) S.b3[tid] = W.b3[tid];
     if (tid == 0) {
         for (int b = 0; b < kXStages; ++b) {
             mbar_init(&S.xfull[b], 1);
             mbar_init(&S.xempty[b], 1);
         }
-        mbar_init(&S.mma, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&S.d1[b], 1);
+            mbar_init(&S.e1[b], kEpiWarps);
+        }
+        mbar_init(&S.d2, 1);
+        mbar_init(&S.d3, 1);
+        mbar_init(&S.h1, kEpiWarps);
+        mbar_init(&S.h2, kEpiWarps);
         mbar_fence_init();
-        S.ok = 1;
     }
     if (warp == 0) {
         tmem_alloc(&S.tmem, kTmemCols);
         tmem_relinquish();
     }
-    fence_async_shared();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    if (warp != kEpiWarps) {             // (the rows' copies start meanwhile)
+        stage_panels(S.W1, W.W1);
+        stage_weights(S.W2, W.W2, kH, kH, kH);
+        stage_weights(S.W3, W.W3, kN3, kOutPad, kH);
+        const int i = warp < kEpiWarps ? tid : tid - 32;
+        for (int k = i; k < kH; k += kStagers) {
+            S.b1[k] = W.b1[k];
+            S.b2[k] = W.b2[k];
+        }
+        if (i < kOutPad) S.b3[i] = W.b3[i];
+        fence_async_shared();
+        asm volatile("bar.sync 1, %0;" ::"n"(kStagers) : "memory");
+    }
     const uint32_t tm = S.tmem;
-    constexpr uint32_t kId128 = idesc_bf16_f32(kRows, kH), kId16 = idesc_bf16_f32(kRows, kN3);
-    constexpr uint32_t kChunkBytes = kRows * kKc * 2;
-    // thread 0's bookkeeping: loads issued into / consumed from each stage
-    uint32_t loads[kXStages] = {}, used[kXStages] = {};
-    bool t0ok = true;
-    auto issue = [&](long long tile, int c) {           // thread 0: chunk c of a tile
-        const int s = c % kXStages;
-        if (loads[s] > 0 && t0ok)                        // the MMAs of the stage's last chunk
-            t0ok = mbar_wait_bounded(&S.xempty[s], (loads[s] - 1) & 1u);
-        if (!t0ok) return;
-        mbar_arrive_expect_tx(&S.xfull[s], kChunkBytes);
-#pragma unroll
-        for (int j = 0; j < kKc / 8; ++j)
-            tma_load_2d(&S.Xc[s][j * kRows * 8], &xmap, c * kKc + 8 * j, (int)(tile * kRows), &S.xfull[s]);
-        ++loads[s];
-    };
-    uint32_t nmma = 0;                                   // phases of S.mma waited so far
-    if (tid == 0)
-        for (int c = 0; c < kXStages; ++c) issue(blockIdx.x, c);
     bool ok = true;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const long long row0 = t * kRows;
-        if (tid == 0) {
-            // ---- layer 1: D1 = X W1^T over six chunks ----
-            for (int c = 0; c < kNChunks && t0ok; ++c) {
-                const int s = c % kXStages;
-                if (c >= kXStages) issue(t, c);
-                if (!t0ok) break;
-                t0ok = mbar_wait_bounded(&S.xfull[s], used[s] & 1u);
-                if (!t0ok) break;
-                ++used[s];
+    if (warp == kEpiWarps) {
+        // ---- the copies ----
+        if (lane == 0) {
+            uint32_t n = 0;                                       // panels requested
+            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x)
+                for (int c = 0; c < kNChunks && ok; ++c, ++n) {
+                    const uint32_t s = n % kXStages;
+                    if (n >= kXStages) ok = mbar_wait_bounded(&S.xempty[s], (n / kXStages - 1) & 1u);
+                    if (!ok) break;
+                    mbar_arrive_expect_tx(&S.xfull[s], kPanel * 2);
+                    tma_load_2d(S.Xc[s], &xmap, c * kKc, (int)(t * kRows), &S.xfull[s]);
+                }
+            // the copies still in flight land before the block leaves
+            for (uint32_t k = n > kXStages ? n - kXStages : 0; k < n; ++k)
+                mbar_wait_bounded(&S.xfull[k % kXStages], (k / kXStages) & 1u);
+        }
+    } else if (warp == kEpiWarps + 1) {
+        // ---- layer 1 ----
+        if (lane == 0) {
+            constexpr uint32_t kId = idesc_bf16_f32(kRows, kH);
+            uint32_t n = 0, i = 0;                                // panels consumed, tiles begun
+            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+                const uint32_t b = i & 1u;
+                if (i >= 2) ok = mbar_wait_bounded(&S.e1[b], (i / 2 - 1) & 1u);
+                for (int c = 0; c < kNChunks && ok; ++c, ++n) {
+                    const uint32_t s = n % kXStages;
+                    ok = mbar_wait_bounded(&S.xfull[s], (n / kXStages) & 1u);
+                    if (!ok) break;
+                    tc_fence_after_sync();
+                    const uint32_t xa = smem_addr(S.Xc[s]), wa = smem_addr(S.W1[c]);
+#pragma unroll
+                    for (int kk = 0; kk < kKc; kk += 16)
+                        tc_mma_bf16(tm + b * kH, smem_desc_sw128(xa, kk * 2), smem_desc_sw128(wa, kk * 2), kId,
+                                    (c | kk) != 0);
+                    tc_commit(&S.xempty[s]);
+                }
+                tc_commit(&S.d1[b]);
+            }
+        }
+    } else if (warp == kEpiWarps + 2) {
+        // ---- layers 2 and 3 ----
+        if (lane == 0) {
+            constexpr uint32_t kId128 = idesc_bf16_f32(kRows, kH), kId16 = idesc_bf16_f32(kRows, kN3);
+            uint32_t i = 0;
+            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+                ok = mbar_wait_bounded(&S.h1, i & 1u);
+                if (!ok) break;
                 tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < kKc; kk += 16)
-                    tc_mma_bf16(tm, tile_desc(S.Xc[s], kRows, kk), tile_desc(S.W1, kH, c * kKc + kk),
-                                kId128, (c | kk) != 0);
-                tc_commit(&S.xempty[s]);
+                for (int kk = 0; kk < kH; kk += 16)
+                    tc_mma_bf16(tm + 2 * kH, tile_desc(S.H, kRows, kk), tile_desc(S.W2, kH, kk), kId128, kk != 0);
+                tc_commit(&S.d2);
+                ok = mbar_wait_bounded(&S.h2, i & 1u);
+                if (!ok) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int kk = 0; kk < kH; kk += 16)
+                    tc_mma_bf16(tm + 3 * kH, tile_desc(S.H, kRows, kk), tile_desc(S.W3, kN3, kk), kId16, kk != 0);
+                tc_commit(&S.d3);
             }
-            tc_commit(&S.mma);
-            // the next tile's first chunks, while this tile finishes
-            if (t + gridDim.x < ntiles)
-                for (int c = 0; c < kXStages; ++c) issue(t + gridDim.x, c);
-            if (!t0ok) S.ok = 0;
         }
-        ok = mbar_wait_bounded(&S.mma, nmma & 1u) && ok;
-        ++nmma;
-        tc_fence_after_sync();
-        epilogue_relu(tm, 0u, S.b1, S.H);
-        fence_async_shared();
-        tc_fence_before_sync();
-        __syncthreads();
-        // ---- layer 2: D2 (columns 128..255) = H1 W2^T ----
-        if (tid == 0) {
+    } else {
+        // ---- the epilogues ----
+        uint32_t i = 0;
+        for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&S.d1[i & 1u], (i / 2) & 1u));
+            if (!ok) break;
             tc_fence_after_sync();
-#pragma unroll
-            for (int kk = 0; kk < kH; kk += 16)
-                tc_mma_bf16(tm + kH, tile_desc(S.H, kRows, kk), tile_desc(S.W2, kH, kk), kId128, kk != 0);
-            tc_commit(&S.mma);
-        }
-        ok = mbar_wait_bounded(&S.mma, nmma & 1u) && ok;
-        ++nmma;
-        tc_fence_after_sync();
-        __syncthreads();                                 // every read of H1 is done (MMAs completed)
-        epilogue_relu(tm, (uint32_t)kH, S.b2, S.H);      // H2 over H1
-        fence_async_shared();
-        tc_fence_before_sync();
-        __syncthreads();
-        // ---- layer 3: D3 (columns 0..15) = H2 W3^T ----
-        if (tid == 0) {
+            epilogue_relu(tm, (i & 1u) * kH, S.b1, S.H);
+            fence_async_shared();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&S.e1[i & 1u]);
+                mbar_arrive(&S.h1);
+            }
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&S.d2, i & 1u));
+            if (!ok) break;
             tc_fence_after_sync();
+            epilogue_relu(tm, 2u * kH, S.b2, S.H);                // H2 over H1 (its MMAs have completed)
+            fence_async_shared();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.h2);
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&S.d3, i & 1u));
+            if (!ok) break;
+            tc_fence_after_sync();
+            if (warp < 4) {
+                float v[16];
+                tmem_ld16(tm + ((uint32_t)(32 * warp) << 16) + 3 * kH, v);
+                const long long row = t * kRows + 32 * warp + lane;
+                if (row < nrows) {
+                    float* y = Y + row * kOut;
 #pragma unroll
-            for (int kk = 0; kk < kH; kk += 16)
-                tc_mma_bf16(tm, tile_desc(S.H, kRows, kk), tile_desc(S.W3, kN3, kk), kId16, kk != 0);
-            tc_commit(&S.mma);
-        }
-        ok = mbar_wait_bounded(&S.mma, nmma & 1u) && ok;
-        ++nmma;
-        tc_fence_after_sync();
-        if (warp < 4) {
-            float v[16];
-            tmem_ld16(tm + ((uint32_t)(32 * warp) << 16), v);
-            const long long row = row0 + 32 * warp + lane;
-            if (row < nrows)
-#pragma unroll
-                for (int o = 0; o < kOut; ++o) Y[row * kOut + o] = v[o] + S.b3[o];
-        }
-        tc_fence_before_sync();
-        const bool all_ok = __syncthreads_and(ok && S.ok) != 0;
-        tc_fence_after_sync();
-        if (!all_ok) {
-            ok = false;
-            break;
+                    for (int o = 0; o < kOut; ++o) y[o] = v[o] + S.b3[o];
+                }
+            }
+            tc_fence_before_sync();
         }
     }
-    if (tid == 0 && (!ok || !t0ok)) {
-        atomicOr(flags, kFlagTimeout);
-        for (int b = 0; b < kXStages; ++b)               // copies still in flight land first
-            if (loads[b] > used[b]) mbar_wait_bounded(&S.xfull[b], used[b] & 1u);
+    if (!ok && lane == 0) {
+        if (host_flags) *(volatile unsigned*)flags = kFlagTimeout;
+        else atomicOr(flags, kFlagTimeout);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -619,25 +666,25 @@ __global__ void __launch_bounds__(256, 1) k_mlp_rows(const __grid_constant__ Mlp
 }
 
 cudaError_t launch_mlp_rows(const MlpWeights& W, const bf16* X, long long M, const unsigned* count_dev,
-                            float* Y, unsigned* flags, cudaStream_t s)
+                            float* Y, unsigned* flags, int host_flags, cudaStream_t s)
 {
     if (M <= 0) return cudaSuccess;
     CUtensorMap xmap;
-    if (!encode_bf16_2d(&xmap, X, kInPad, (unsigned long long)M, kInPad * 2, 8, kRows))
+    if (!encode_bf16_2d(&xmap, X, kInPad, (unsigned long long)M, kInPad * 2, kKc, kRows, true))
         return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kTcSmemBytes);
     if (e != cudaSuccess) return e;
     const long long tiles = (M + kRows - 1) / kRows;
     const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, device_sm_count()));
-    k_mlp_rows<<<grid, 256, kTcSmemBytes, s>>>(W, xmap, M, count_dev, Y, flags);
+    k_mlp_rows<<<grid, kMlpThreads, kTcSmemBytes, s>>>(W, xmap, M, count_dev, Y, flags, host_flags);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_infer(const MlpWeights& W, const bf16* X, long long M, float* Y,
-                             unsigned* flags, cudaStream_t s)
+                             unsigned* host_flags, cudaStream_t s)
 {
-    return launch_mlp_rows(W, X, M, nullptr, Y, flags, s);
+    return launch_mlp_rows(W, X, M, nullptr, Y, host_flags, 1, s);
 }
 
 // --------------------------------------------------------------------------
@@ -898,7 +945,7 @@ static cudaError_t launch_seeding_n(const Problem& P, const BatchDesc* bd, const
     k_seed_features<N, BATCH><<<sms * 16, 256, 0, s>>>(P, bd);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if ((e = launch_mlp_rows(W, X, cap, count, Y, flags, s)) != cudaSuccess) return e;
+    if ((e = launch_mlp_rows(W, X, cap, count, Y, flags, 0, s)) != cudaSuccess) return e;
     k_seed_apply<N, BATCH><<<sms * 8, 256, 0, s>>>(P, bd);
     return cudaGetLastError();
 }
@@ -976,7 +1023,9 @@ struct gamma_model_s {
     // row stride wsMp = wsM rounded up to 8 (16-byte rows for TMA)
     bf16 *XT = nullptr, *H1T = nullptr, *dZ1T = nullptr, *dZ2T = nullptr;
     long long wsMp = 0;
-    unsigned* dflags = nullptr;   // error flags of the tensor-core kernels
+    unsigned* dflags = nullptr;   // error flags of the training kernels
+    unsigned* hflags = nullptr;   // ... of gamma_model_infer: page-locked, mapped host memory
+    unsigned* hflags_dev = nullptr;   // its device address
 };
 
 namespace {
@@ -1168,6 +1217,8 @@ int gamma_model_create(gamma_model* out, uint64_t seed)
     if ((rc = cuda_rc(cudaMalloc(&m->W3h, sizeof(bf16) * gk::kOutPad * gk::kH)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->dflags, sizeof(unsigned))))) return fail(rc);
     if ((rc = cuda_rc(cudaMemset(m->dflags, 0, sizeof(unsigned))))) return fail(rc);
+    if ((rc = cuda_rc(cudaHostAlloc(&m->hflags, sizeof(unsigned), cudaHostAllocMapped)))) return fail(rc);
+    if ((rc = cuda_rc(cudaHostGetDevicePointer((void**)&m->hflags_dev, m->hflags, 0)))) return fail(rc);
     std::vector<float> h;
     init_params(h, seed);
     m->seed = seed;
@@ -1188,6 +1239,7 @@ void gamma_model_destroy(gamma_model m)
     cudaFree(m->p); cudaFree(m->gr); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->mask);
     cudaFree(m->W1h); cudaFree(m->W2h); cudaFree(m->W2Th); cudaFree(m->W3h);
     cudaFree(m->dflags);
+    if (m->hflags) cudaFreeHost(m->hflags);
     free_ws(m);
     delete m;
 }
@@ -1234,12 +1286,13 @@ int gamma_model_infer(gamma_model m, const void* X_bf16_dev, int64_t M, float* Y
     cudaStream_t s = (cudaStream_t)cuda_stream;
     gk::MlpWeights W;
     gk::model_weights(m, &W);
-    MCK(cudaMemsetAsync(m->dflags, 0, sizeof(unsigned), s));
-    MCK(gk::launch_mlp_infer(W, (const bf16*)X_bf16_dev, M, Y_dev, m->dflags, s));
-    unsigned flags = 0;
-    MCK(cudaMemcpyAsync(&flags, m->dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    // the kernel reports a timeout in mapped host memory: no reset or copy
+    // around it (the call ends with the stream's synchronisation anyway)
+    volatile unsigned* flag = m->hflags;
+    *flag = 0;
+    MCK(gk::launch_mlp_infer(W, (const bf16*)X_bf16_dev, M, Y_dev, m->hflags_dev, s));
     MCK(cudaStreamSynchronize(s));
-    return (flags & gk::kFlagTimeout) ? GAMMA_ERR_TIMEOUT : GAMMA_OK;
+    return (*flag & gk::kFlagTimeout) ? GAMMA_ERR_TIMEOUT : GAMMA_OK;
 }
 
 int gamma_model_backward(gamma_model m, const void* X_bf16_dev, const float* T_dev, int64_t M,

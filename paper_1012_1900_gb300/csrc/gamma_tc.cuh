@@ -7,6 +7,10 @@
 // the core matrix of row group g and k-chunk c sits at
 //     base + c * LBO + g * SBO,
 // with LBO the byte step between k-chunks and SBO the step between row groups.
+// Operands that arrive by TMA take the 128-byte swizzle instead: a panel of 64
+// columns is one box of R rows x 128 bytes (R * 128 bytes, aligned to 1 KB),
+// in which 16-byte chunk j of row r sits at chunk j ^ (r % 8) of its row; row
+// groups are 1 KB apart, and a K = 16 step moves the start by 32 bytes.
 #pragma once
 #include <cstdint>
 
@@ -54,6 +58,18 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
     return d;                                    // base offset 0, no swizzle
 }
 
+// Descriptor of the K = 16 slice starting at byte `k0_bytes` of a 64-column
+// panel with the 128-byte swizzle (K-major).
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t panel, uint32_t k0_bytes)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)(((panel + k0_bytes) >> 4) & 0x3FFFu);
+    d |= (uint64_t)(1024u >> 4) << 32;           // step between 8-row groups
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;                      // 128-byte swizzle
+    return d;
+}
+
 // Instruction descriptor, kind::f16: D FP32, A and B BF16, both K-major.
 constexpr uint32_t idesc_bf16_f32(int M, int N)
 {
@@ -96,6 +112,25 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// 32 consecutive columns, one wait.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
+{
+    uint32_t r[32];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+            "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+            : "=r"(r[16 * h]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]),
+              "=r"(r[16 * h + 4]), "=r"(r[16 * h + 5]), "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]),
+              "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]), "=r"(r[16 * h + 10]), "=r"(r[16 * h + 11]),
+              "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]), "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+            : "r"(taddr + 16u * h));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Byte offset of element (row, k) of a K-major bf16 tile in the core-matrix
