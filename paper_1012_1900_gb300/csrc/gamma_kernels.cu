@@ -797,12 +797,15 @@ __device__ __forceinline__ void auto_part_buckets(unsigned count, unsigned lanes
 __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem P)
 {
     __shared__ unsigned start[kNumBuckets], cnt[kNumBuckets], base[kNumBuckets];
-    if (threadIdx.x == 0) {
-        unsigned acc = 0;
-        for (int b = kNumBuckets - 1; b >= 0; --b) {
-            start[b] = acc;
-            acc += P.ctr->hist[b];
+    if (threadIdx.x < kNumBuckets) {
+        const unsigned own = P.ctr->hist[threadIdx.x];
+        unsigned sum = own;                    // of this bucket and the costlier ones
+#pragma unroll
+        for (int o = 1; o < kNumBuckets; o <<= 1) {
+            const unsigned u = __shfl_down_sync(kFull, sum, o);
+            if (threadIdx.x + o < kNumBuckets) sum += u;
         }
+        start[threadIdx.x] = sum - own;
     }
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     for (unsigned c0 = blockIdx.x * blockDim.x; c0 < total; c0 += gridDim.x * blockDim.x) {
@@ -1490,21 +1493,24 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
     for (int part = 0; part < kCqParts; ++part) {
         const unsigned lo = part ? s_end[part - 1] : 0u, hi = s_end[part];
         if (lo >= hi) continue;
-        const int g = cq_part_lanes(part);         // lanes per voxel
+        // lanes per voxel: the part's, and more where it is too short to fill
+        // the warps (the walk is then bound by its steps' latency)
+        int g = cq_part_lanes(part);
+        while (g < 32 && (unsigned long long)(hi - lo) * (unsigned)g * 2u <= 32ull * nwarps) g *= 2;
         const unsigned nv = 32u / (unsigned)g;     // voxels per round
-        unsigned nb = nv;                          // voxels per batch
-        unsigned at = lo;                          // where the queue stood when this warp last looked
         const int gl = lane & (g - 1);
+        unsigned at = lo;                          // where the queue stood when this warp last looked
         for (;;) {
-            // as many rounds per batch as keep it below an eighth of a warp's
-            // share of the queue's estimated cells, from the cost bucket at
-            // the last known position (costs only fall from there); in a
+            // voxels per batch: as many rounds as keep it below half of a
+            // warp's share of the queue's estimated cells, from the cost bucket
+            // at the last known position (costs only fall from there); in a
             // batch group, whose parts mix pairs and costs, two rounds
+            unsigned nb = nv;
             if constexpr (BATCH) {
                 nb = min(32u, 2u * nv);
             } else if (P0.sort_tail) {
                 const unsigned m = __ballot_sync(kFull, s_start[lane] <= at && (lane == 0 || s_start[lane - 1] > at));
-                const float share = s_cells / (8.f * (float)nwarps * bucket_cells(m ? 31 - __clz(m) : 0));
+                const float share = s_cells / (2.f * (float)nwarps * bucket_cells(m ? 31 - __clz(m) : 0));
                 nb = min(32u, max(nv, (unsigned)fminf(share, 32.f) / nv * nv));
             }
             unsigned base = 0;
@@ -2715,8 +2721,7 @@ cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s)
 cudaError_t launch_order_tail(const Problem& P, cudaStream_t s)
 {
     if (!P.sort_tail) return cudaSuccess;
-    const int sms = device_sm_count();
-    k_scatter<<<sms * 8, 256, 0, s>>>(P);
+    k_scatter<<<grid_for(P.nvox, 256, device_sm_count() * 8), 256, 0, s>>>(P);
     return cudaGetLastError();
 }
 
@@ -2756,12 +2761,16 @@ cudaError_t launch_tail(const Problem& P, int lanes_per_voxel, int tail_minblock
 template <int N, bool BATCH>
 static void launch_tail_cq_n(const Problem& P, const BatchDesc* bd, int per_sm, cudaStream_t s)
 {
-    const int grid = device_sm_count() * per_sm;      // persistent: one wave of resident blocks
+    const int sms = device_sm_count();
+    // persistent: one wave of resident blocks (fewer where even a voxel per
+    // lane group would leave blocks without work)
+    const int grid = BATCH ? sms * per_sm : grid_for(P.nvox, cq_threads(per_sm) / 32, sms * per_sm);
     if (per_sm >= 4) k_tail_cq<N, 4, BATCH><<<grid, cq_threads(4), 0, s>>>(P, bd);
     else if (per_sm == 3) k_tail_cq<N, 3, BATCH><<<grid, cq_threads(3), 0, s>>>(P, bd);
     else if (per_sm == 2) k_tail_cq<N, 2, BATCH><<<grid, cq_threads(2), 0, s>>>(P, bd);
     else k_tail_cq<N, 1, BATCH><<<grid, cq_threads(1), 0, s>>>(P, bd);
-    k_tail_fix<N, BATCH><<<device_sm_count() * 2, 256, 0, s>>>(P, bd);
+    // (a warp per listed voxel; most often there is none)
+    k_tail_fix<N, BATCH><<<BATCH ? device_sm_count() * 2 : grid_for(P.nvox, 8, device_sm_count() * 2), 256, 0, s>>>(P, bd);
 }
 
 cudaError_t launch_tail_cq(const Problem& P, int tail_minblocks, cudaStream_t s)
