@@ -73,7 +73,8 @@ void free_batch(BatchState* b);
 struct GridState {
     gk::GridProblem G{};
     TableEntry* table_dev = nullptr;
-    unsigned* walk_list = nullptr;     // voxels the warp-evaluated walk leaves to k_grid_walk
+    unsigned* walk_list = nullptr;     // voxels the walk leaves to k_grid_walk; then its queue and
+                                       // the cells of the queue's seeds (nref entries each)
 };
 
 // Evaluation-dose z slabs of a host-buffer run: the shell starts on a slab
@@ -830,7 +831,7 @@ int gamma_create_grids(gamma_handle* out, const float* ref_dev, const float* eva
     auto fail = [&](int code) { free_ctx(h); return code; };
     h->grids = new (std::nothrow) GridState();
     if (!h->grids) return fail(GAMMA_ERR_OOM);
-    h->walk = 0;       // the lane walk: the warp-evaluated one measured slower on two grids
+    h->walk = 0;       // lanes_per_voxel lanes per reference voxel
     if (cudaGetDevice(&h->device) != cudaSuccess) return fail(GAMMA_ERR_CUDA);
     h->ndim = ndim;
     h->nz = ndim == 3 ? ref_shape[0] : 1;
@@ -854,6 +855,8 @@ int gamma_create_grids(gamma_handle* out, const float* ref_dev, const float* eva
         G.ro[a] = used ? ref_origin_mm[src] / dta : 0.0;
         G.eh[a] = used ? eval_spacing_mm[src] / dta : 1.0;
         G.eo[a] = used ? eval_origin_mm[src] / dta : 0.0;
+        G.ua[a] = (G.ro[a] - G.eo[a]) / G.eh[a];
+        G.ub[a] = G.rh[a] / G.eh[a];
         G.mt.hn2[a] = (float)(G.eh[a] * G.eh[a]);
         G.mtd.hn2[a] = G.eh[a] * G.eh[a];
     }
@@ -872,7 +875,7 @@ int gamma_create_grids(gamma_handle* out, const float* ref_dev, const float* eva
     G.local = crit->mode == GAMMA_LOCAL;
     if (int rc = upload_grid_tables(h, h->table_cap)) return fail(rc);
     cudaError_t e;
-    if ((e = cudaMalloc(&h->grids->walk_list, sizeof(unsigned) * (size_t)nref)) != cudaSuccess)
+    if ((e = cudaMalloc(&h->grids->walk_list, 3 * sizeof(unsigned) * (size_t)nref)) != cudaSuccess)
         return fail(cuda_fail(e));
     for (auto& te : h->tev)
         if ((e = cudaEventCreate(&te)) != cudaSuccess) return fail(cuda_fail(e));
@@ -938,10 +941,10 @@ int gamma_run(gamma_handle h, float* gamma_out_dev, void* cuda_stream)
         G.out = gamma_out_dev;
         G.ctr = h->ctr;
         G.tau = (float)h->tau;
-        G.lanes = h->lanes;
-        G.walk = h->walk;
+        G.lanes = h->walk == 3 ? gk::kDefaultLanesPerVoxel : h->lanes;
         G.walk_list = h->grids->walk_list;
-        G.from_list = 0;
+        G.queue = G.walk_list + h->nvox;
+        G.skip = G.queue + h->nvox;
         if (tm) {
             CK(cudaEventRecord(h->tev[0], s));
             CK(cudaEventRecord(h->tev[1], s));

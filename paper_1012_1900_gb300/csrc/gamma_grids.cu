@@ -6,15 +6,17 @@
 //
 //   k_grid_prepare  max of the reference dose (the global dose norm) and a
 //                   finite check of both grids
-//   k_grid_walk     a group of lanes per reference voxel (eight by default)
-//                   walks the cell table in key order, a cell per lane and
-//                   round, from the evaluation cell
-//                   that holds the voxel (clamped to the grid), with the exact
-//                   stop of A1 step 4b-ii; a cell is skipped when the distance
-//                   from the reference point to its box, with its dose gap,
-//                   already reaches the running gamma, else every face of it
-//                   is evaluated (real-valued cell offsets; FP64 redo when a
-//                   Gram matrix is near singular)
+//   k_grid_seed     the evaluated reference voxels, each with a bound from the
+//                   affine parts of a few cells around it
+//   k_grid_cq       the walk of the cell table in key order from the evaluation
+//                   cell that holds the voxel (clamped to the grid), with the
+//                   exact stop of A1 step 4b-ii; a cell is skipped when the
+//                   distance from the reference point to its box, with its
+//                   dose gap, or its affine part already keeps it at the
+//                   running gamma, else every face of it is evaluated
+//                   (real-valued cell offsets)
+//   k_grid_walk     the voxels with a near-singular cell (FP64 redo) or a walk
+//                   past a truncated table (box scan), a warp each
 //
 // The table is keyed by the distance between the box of the voxel's cell and
 // the box of the other cell, divided by the DTA: a lower bound on the distance
@@ -32,6 +34,7 @@
 #include "../../include/gamma.h"
 #include "gamma_cell.cuh"
 #include "gamma_internal.h"
+#include "gamma_plane.cuh"
 
 namespace gk {
 
@@ -142,8 +145,9 @@ __device__ __forceinline__ float grid_cell(const GridProblem& G, const int (&p)[
     return fminf(best, cb);
 }
 
-// GL lanes per reference voxel (GL-aligned groups of a warp; 2 .. 32).  The
-// table starts with the voxel's own cell (offset 0), so the first round of G
+// GL lanes per reference voxel (GL-aligned groups of a warp) over the voxels
+// that k_grid_cq left in walk_list, each from an infinite bound.  The table
+// starts with the voxel's own cell (offset 0), so the first round of G
 // cells gives a finite bound; later cells are skipped when the distance from
 // the point itself to the cell's box, with the dose gap, already reaches the
 // running gamma.  The exact stop (A1 step 4b-ii) takes the table's key.
@@ -153,19 +157,13 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
     const int lane = threadIdx.x & 31, gl = lane & (GL - 1), gbase = lane & ~(GL - 1);
     const unsigned gmask = GL == 32 ? kFull : (((1u << GL) - 1u) << gbase);
     const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
-    const float thr = cutoff_threshold(G.local, G.cutoff_frac, dnorm);
     unsigned my_eval = 0, my_pass = 0, my_over = 0;
     const long long ngroups = ((long long)gridDim.x * blockDim.x) / GL;
-    // every reference voxel, or (from_list) those k_grid_cq left in walk_list
-    const long long nwork = G.from_list ? (long long)G.ctr->fix_count : G.nref;
+    const long long nwork = (long long)G.ctr->fix_count;
     for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / GL; i < nwork;
          i += ngroups) {                                     // group-uniform
-        const long long v = G.from_list ? (long long)G.walk_list[i] : i;
+        const long long v = (long long)G.walk_list[i];
         const float dr = __ldg(G.ref + v);
-        if (!(dr >= thr && (!G.local || dr > 0.f))) {
-            if (gl == 0) G.out[v] = __int_as_float(0x7fc00000);
-            continue;
-        }
         const long long ix[3] = {v % G.rn[0], (v / G.rn[0]) % G.rn[1], v / ((long long)G.rn[0] * G.rn[1])};
         // the point in evaluation voxel units: its cell c0 (clamped to the
         // grid) and its position fr in that cell (outside [0, 1) beyond the
@@ -290,288 +288,381 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
 }
 
 // --------------------------------------------------------------------------
-// The warp-evaluated walk (default): cells collected per warp, evaluated 32
-// at a time
+// Plane seeds and the tiered walk
 // --------------------------------------------------------------------------
 
-// As for coincident grids (k_tail_cq), the face evaluation of a cell is not
-// done by the lane that reached it: a cell that passes the box and dose-gap
-// bounds is appended, with its vertex doses and its offset from the point, to
-// a ring of the warp, and the whole warp evaluates 32 such cells at once, one
-// per lane, lowering each owner's running bound in shared memory (atomicMin
-// on the bits of a non-negative float).  GL lanes walk one reference voxel's
-// table together (GL entries per step); a walker keeps two voxel slots so that
-// it starts its next voxel while the cells of its last one wait.  Every stop
-// and prune stays exact with a lagging bound, and each cell is evaluated with
-// the arithmetic of grid_cell, so the map is k_grid_walk's.  A voxel with a
-// near-singular cell, or whose walk runs past a truncated table, goes to
-// walk_list; k_grid_walk then searches it again from scratch (FP64 redo, box
-// scan), so that this kernel keeps the registers of the FP32 evaluation.
+// A reference voxel's place on the evaluation grid: its cell c0 (clamped to
+// the grid) and its position fr in that cell (outside [0, 1) beyond the grid).
+template <int N>
+struct GridPlace {
+    int c0[3];
+    float fr[3];
+};
+
+template <int N>
+__device__ __forceinline__ GridPlace<N> grid_place(const GridProblem& G, unsigned v)
+{
+    GridPlace<N> p;
+    const unsigned r1 = v / (unsigned)G.rn[0];
+    const unsigned ix[3] = {v % (unsigned)G.rn[0], r1 % (unsigned)G.rn[1], r1 / (unsigned)G.rn[1]};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        p.c0[a] = 0;
+        p.fr[a] = 0.f;
+        if (a < N) {
+            const double u = fma((double)ix[a], G.ub[a], G.ua[a]);
+            const double f = fmin(fmax(floor(u), 0.0), (double)(G.en[a] - 2));
+            p.c0[a] = (int)f;
+            p.fr[a] = (float)(u - f);
+        }
+    }
+    return p;
+}
+
+// The evaluated reference voxels, in order, with a bound on each one's gamma
+// (squared, in out) as k_plane_seed finds it: kGridSteps steps along the affine
+// part of one cell, from the cell that holds the point, then every face of the
+// last cell (none when it is near singular: an infinite bound).
+constexpr int kGridSteps = 3;
+
+template <int N>
+__global__ void __launch_bounds__(256) k_grid_seed(const __grid_constant__ GridProblem G)
+{
+    const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
+    const float thr = cutoff_threshold(G.local, G.cutoff_frac, dnorm);
+    const int sy = G.en[0], sz = G.en[0] * G.en[1], lane = threadIdx.x & 31;
+    const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
+    for (long long b = (long long)blockIdx.x * blockDim.x; b < G.nref; b += (long long)gridDim.x * blockDim.x) {
+        const long long i = b + threadIdx.x;
+        float dr = 0.f;
+        bool take = false;
+        if (i < G.nref) {
+            dr = __ldg(G.ref + i);
+            take = dr >= thr && (!G.local || dr > 0.f);
+            if (!take) G.out[i] = kNaN;
+        }
+        const unsigned tk = __ballot_sync(kFull, take);
+        unsigned pos = 0;
+        if (tk && lane == 0) pos = atomicAdd(&G.ctr->tail_count, (unsigned)__popc(tk));
+        pos = __shfl_sync(kFull, pos, 0) + (unsigned)__popc(tk & ((1u << lane) - 1u));
+        if (!take) continue;
+        const unsigned v = (unsigned)i;
+        const GridPlace<N> at = grid_place<N>(G, v);
+        const float inv = 1.0f / (G.dd_frac * (G.local ? dr : dnorm)), inv2 = inv * inv;
+        int c[3] = {at.c0[0], at.c0[1], at.c0[2]};            // grid coordinates, every vertex inside
+        float e[8];
+#pragma unroll 1
+        for (int it = 0;; ++it) {
+            const float* q = G.ev + ((long long)c[2] * sz + (long long)c[1] * sy + c[0]);
+#pragma unroll
+            for (int u = 0; u < (1 << N); ++u)
+                e[u] = __ldg(q + (u & 1) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0));
+            if (it == kGridSteps) break;
+            const CellPlane<N> p = cell_plane<N>(e);
+            float L = p.m - dr, D = 0.f, gk[3];
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                L = fmaf(-p.G[a], (float)(c[a] - at.c0[a]) - at.fr[a] + 0.5f, L);
+                gk[a] = p.G[a] * G.mt.kappa[1 << a];
+                D = fmaf(p.G[a], gk[a], D);
+            }
+            const float r = __fdividef(L * inv2, fmaf(D, inv2, 1.f));
+            bool same = true;
+#pragma unroll
+            for (int a = 0; a < N; ++a) {
+                // at most 500 cells away: the packed offset's range
+                const float s = fminf(fmaxf(at.fr[a] - r * gk[a], -500.f), 500.f);
+                const int t = max(0, min(G.en[a] - 2, at.c0[a] + __float2int_rd(s)));
+                same = same && t == c[a];
+                c[a] = t;
+            }
+            if (same) break;
+        }
+        float q[8], cf[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int u = 0; u < 8; ++u) q[u] = u < (1 << N) ? rel_dose(e[u], dr, inv) : kNaN;
+#pragma unroll
+        for (int a = 0; a < N; ++a) cf[a] = (float)(c[a] - at.c0[a]) - at.fr[a];
+        CellGeom<float> g;
+        cell_geom<N, float>(cf[0], cf[1], cf[2], G.mt, g);
+        bool ill = false;
+        const float cb = cell_min_d2<N, float>(q, g, G.mt, dmax, kInf, ill);
+        if (ill) ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, G.mt.kappa, G.tau);
+        bool near = true;                                     // the offset fits its packed form
+#pragma unroll
+        for (int a = 0; a < N; ++a) near = near && abs(c[a] - at.c0[a]) <= 510;
+        G.out[v] = ill ? kInf : cb + 0.f;
+        G.queue[pos] = v;
+        G.skip[pos] = ill || !near ? 0xffffffffu
+                                   : pack10(c[0] - at.c0[0], c[1] - at.c0[1], N == 3 ? c[2] - at.c0[2] : 0);
+    }
+}
+
+// The table walk in three tiers, as k_tail_cq's: a warp takes a batch of up to
+// 32 queued voxels and walks 32 / gl of them at a time, gl lanes each.  A cell
+// below the bound is tested by the distance from the point itself to its box
+// and its dose gap (tier 1), by plane_bound (tier 2) and by its faces (tier 3),
+// tiers 2 and 3 on full warps of cells from ring buffers.  Each cell is
+// evaluated with the arithmetic of grid_cell.  A voxel with a near-singular
+// cell, or whose bound lies past a truncated table, goes to walk_list;
+// k_grid_walk searches it from scratch (FP64 redo, box scan).
+//
+// What bounds it: issue (68 %, the ALU pipe at 62 %): 0.56 ms, and 0.09 ms for
+// the seeds, for 1.21 M voxels of a 160x160x120 reference against a 320x320x240
+// evaluation dose.  The lane walk before it (k_grid_walk for every voxel: from
+// an infinite bound, each lane evaluating its own cells, the rest of the warp
+// waiting) took 1.91 ms there.
 constexpr int kGqRing = 64;
 
 struct GqWarp {
-    float q[8][kGqRing];       // vertex doses of a pending cell (relative, normalised)
-    float cf[3][kGqRing];      // its lower corner relative to the point (evaluation voxels)
-    unsigned meta[kGqRing];    // owner slot (bits 0-5), vertices inside the grid (bits 8-15)
-    unsigned best[64];         // running squared gamma per voxel slot (float bits)
-    unsigned vox[64];          // reference voxel per slot
-    float dr[32], inv[32];     // the walking voxel's reference dose and 1 / Delta D, per walker
-    float fr[3][32];           // its position in its evaluation cell
-    int c0[3][32];             // that cell
-    int t[32];                 // its next table entry
-    unsigned wseq[32], dseq[32], state[32];
-    unsigned fixm[2];          // slots whose voxel is searched again by k_grid_walk
-    unsigned cnt[2][32];       // voxels finished and passed
-    unsigned pend[64];         // evaluated reference voxels not yet taken by a walker
-    int tv[64];                // table variant of each slot's voxel
+    unsigned ring[2][kGqRing]; // pending cells of tiers 2 and 3: table entry << 5 | slot of the voxel
+    unsigned best[32];         // per slot: running squared gamma (float bits),
+    unsigned vox[32], skip[32];    // voxel, its seed's cell,
+    float dr[32], inv[32], fr[3][32];   // reference dose, 1 / Delta D, place in its cell,
+    int c0[3][32], tv[32];     // that cell, and its table variant
+    unsigned fixm;             // slots whose voxel is searched again by k_grid_walk
 };
-constexpr unsigned kGqWalk = 1u, kGqEnded = 2u, kGqWPend = 4u, kGqDBusy = 8u, kGqDPend = 16u,
-                   kGqDOver = 32u, kGqSlot = 64u;     // slot bit: the walking slot is walker + 32
 
-template <int N, int GL>
-__global__ void __launch_bounds__(256, 2) k_grid_cq(const __grid_constant__ GridProblem G)
+template <int N>
+__global__ void __launch_bounds__(384, 2) k_grid_cq(const __grid_constant__ GridProblem G)
 {
-    __shared__ GqWarp gqw[8];
+    __shared__ GqWarp gqw[12];
     GqWarp& W = gqw[threadIdx.x >> 5];
     volatile GqWarp& V = gqw[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31, gl = lane & (GL - 1), ld = lane - gl;
-    const bool leader = gl == 0;
+    const int lane = threadIdx.x & 31, g = G.lanes, gl = lane & (g - 1);
     const unsigned lt_mask = (1u << lane) - 1u;
-    const unsigned gmask = GL == 32 ? kFull : ((1u << GL) - 1u) << ld;
     const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
-    const float thr = cutoff_threshold(G.local, G.cutoff_frac, dnorm);
-    const float ehf[3] = {(float)G.eh[0], (float)G.eh[1], (float)G.eh[2]};
-    W.state[lane] = 0;
-    W.wseq[lane] = W.dseq[lane] = 0;
-    W.cnt[0][lane] = W.cnt[1][lane] = 0;
-    W.tv[lane] = W.tv[lane + 32] = 8;
-    if (lane < 2) W.fixm[lane] = 0;
+    const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
+    const float eh[3] = {(float)G.eh[0], (float)G.eh[1], (float)G.eh[2]};
+    const int sy = G.en[0], sz = G.en[0] * G.en[1];
+    const unsigned total = G.ctr->tail_count, nwarps = gridDim.x * (blockDim.x >> 5);
+    const unsigned nv = 32u / (unsigned)g;         // voxels per round
+    const unsigned nb = min(32u, max(nv, total / (8u * nwarps) / nv * nv));
+    unsigned my_eval = 0, my_pass = 0;
+    if (lane == 0) W.fixm = 0;
     __syncwarp();
-
-    unsigned head = 0, count = 0;      // the ring: pending cells are [head, head + count)
-    unsigned pend_n = 0;               // entries of W.pend (warp-uniform)
-    bool queue_done = false;           // warp-uniform
     for (;;) {
-        unsigned sta = V.state[ld];
-        if (leader) {
-            // 1. a drained voxel whose cells are all evaluated is final
-            if ((sta & kGqDBusy) && (!(sta & kGqDPend) || (int)(head - V.dseq[ld]) > 0)) {
-                const int ds = ld + ((sta & kGqSlot) ? 0 : 32);
-                const float best = __uint_as_float(V.best[ds]);
-                const unsigned v = V.vox[ds];
-                const float rc = G.tcover[V.tv[ds]];
-                if (((V.fixm[ds >> 5] >> (ds & 31)) & 1u) || ((sta & kGqDOver) && best > rc * rc)) {
-                    G.walk_list[atomicAdd(&G.ctr->fix_count, 1u)] = v;   // k_grid_walk finishes it
-                } else {
-                    const float gam = sqrtf(best);
-                    G.out[v] = gam;
-                    ++V.cnt[0][ld];
-                    if (gam <= 1.f) ++V.cnt[1][ld];
-                }
-                sta &= ~kGqDBusy;
-            }
-            // 2. an ended walk becomes the drain slot; the walker takes a new voxel
-            if ((sta & kGqEnded) && !(sta & kGqDBusy)) {
-                unsigned d = kGqDBusy;
-                if (sta & kGqWPend) d |= kGqDPend;
-                if (V.t[ld] >= G.tlen[V.tv[ld + ((sta & kGqSlot) ? 32 : 0)]]) d |= kGqDOver;
-                V.dseq[ld] = V.wseq[ld];
-                sta = d | ((sta & kGqSlot) ^ kGqSlot);
-            }
-        }
-        // 3. refill the empty walkers, from a per-warp list of evaluated voxels
-        //    that the warp fills 32 grid voxels at a time (one atomic each)
-        const bool empty = leader && !(sta & (kGqWalk | kGqEnded));
-        const unsigned need = __ballot_sync(kFull, empty);
-        while (__popc(need) > (int)pend_n && !queue_done) {      // warp-uniform
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(&G.ctr->head, 32u);
-            base = __shfl_sync(kFull, base, 0);
-            const long long v = (long long)base + lane;
-            bool take = false;
-            if (v < G.nref) {
-                const float r = __ldg(G.ref + v);
-                take = r >= thr && (!G.local || r > 0.f);
-                if (!take) G.out[v] = __int_as_float(0x7fc00000);
-            }
-            const unsigned tk = __ballot_sync(kFull, take);
-            if (take) V.pend[pend_n + __popc(tk & lt_mask)] = (unsigned)v;
-            pend_n += __popc(tk);
-            if ((long long)base + 32 >= G.nref) queue_done = true;
-            __syncwarp();
-        }
-        if (empty) {
-            const int k = __popc(need & lt_mask);
-            if (k < (int)pend_n) {
-                const unsigned v = V.pend[pend_n - 1 - k];
-                const int ws = ld + ((sta & kGqSlot) ? 32 : 0);
-                const long long ix[3] = {v % G.rn[0], (v / G.rn[0]) % G.rn[1], v / ((long long)G.rn[0] * G.rn[1])};
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(&G.ctr->head, nb);
+        base = __shfl_sync(kFull, base, 0);
+        if (base >= total) break;                  // warp-uniform
+        const unsigned nlive = min(nb, total - base);
+        if ((unsigned)lane < nlive) {
+            const unsigned v = G.queue[base + lane];
+            const GridPlace<N> at = grid_place<N>(G, v);
+            const float dr = __ldg(G.ref + v);
 #pragma unroll
-                for (int a = 0; a < N; ++a) {
-                    // the point in evaluation voxel units: its cell (clamped to
-                    // the grid) and its position in that cell (FP64, once)
-                    const double ua = (G.ro[a] + (double)ix[a] * G.rh[a] - G.eo[a]) / G.eh[a];
-                    const double f = fmin(fmax(floor(ua), 0.0), (double)(G.en[a] - 2));
-                    V.c0[a][ld] = (int)f;
-                    V.fr[a][ld] = (float)(ua - f);
-                }
-                for (int a = N; a < 3; ++a) {
-                    V.c0[a][ld] = 0;
-                    V.fr[a][ld] = 0.f;
-                }
-                {
-                    float frr[3];
-                    for (int a = 0; a < 3; ++a) frr[a] = V.fr[a][ld];
-                    V.tv[ws] = grid_variant(frr, N);
-                }
-                const float dr = __ldg(G.ref + v);
-                V.dr[ld] = dr;
-                V.inv[ld] = 1.0f / (G.dd_frac * (G.local ? dr : dnorm));
-                V.best[ws] = __float_as_uint(kInf);
-                V.vox[ws] = v;
-                atomicAnd(&W.fixm[ws >> 5], ~(1u << (ws & 31)));
-                V.t[ld] = 0;
-                sta = (sta & ~kGqWPend) | kGqWalk;
+            for (int a = 0; a < 3; ++a) {
+                V.c0[a][lane] = at.c0[a];
+                V.fr[a][lane] = at.fr[a];
             }
+            V.tv[lane] = grid_variant(at.fr, N);
+            V.dr[lane] = dr;
+            V.inv[lane] = 1.0f / (G.dd_frac * (G.local ? dr : dnorm));
+            V.best[lane] = __float_as_uint(G.out[v]);
+            V.vox[lane] = v;
+            V.skip[lane] = G.skip[base + lane];
         }
-        pend_n -= min((unsigned)__popc(need), pend_n);
-        if (leader) V.state[ld] = sta;
         __syncwarp();
-        sta = V.state[ld];                 // the group's lanes follow their walker
-        if (queue_done && pend_n == 0 &&
-            !__any_sync(kFull, (sta & (kGqWalk | kGqEnded | kGqDBusy)) != 0))
-            break;
-
-        // 4. one table step of every walking group: entries t .. t + GL - 1
-        const bool walking = (sta & kGqWalk) != 0;
-        const int ws = ld + ((sta & kGqSlot) ? 32 : 0);
-        const int t0 = walking ? V.t[ld] : 0;
-        float key = kInf;
-        uint32_t off = 0;
-        const int var = V.tv[ws];
-        const int ntable = G.tlen[var];
-        if (walking && t0 + gl < ntable) {
-            const TableEntry e = G.table[G.toff[var] + t0 + gl];
-            key = e.key;
-            off = e.off;
-        }
-        const float k0 = __shfl_sync(kFull, key, ld);
-        bool cand = false, ended = false;
-        float q[8], cf[3] = {0.f, 0.f, 0.f};
-        uint32_t ok = 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) q[u] = kNaN;
-        if (walking) {
-            const float bst = __uint_as_float(V.best[ws]);
-            ended = t0 >= ntable || k0 * k0 >= bst;           // A1 step 4b-ii, exact
-            if (!ended && key * key < bst) {
-                const int d[3] = {unpack10(off, 0), unpack10(off, 10), N == 3 ? unpack10(off, 20) : 0};
-                int p[3];
-                bool in = true;
-                // the distance from the point to the cell's box: a lower bound
-                // in FP32 from the integer offset and the point's fraction,
-                // each axis lowered by its rounding and the sum by 1e-5
-                float k2 = 0.f;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    p[a] = V.c0[a][ld] + d[a];
-                    const float fr = V.fr[a][ld];
-                    cf[a] = (float)d[a] - fr;
-                    if (a < N) {
-                        in = in && p[a] >= 0 && p[a] < G.en[a];
-                        const float lo = (float)d[a] - fr, hi = fr - (float)(d[a] + 1);
-                        const float slack = 4.8e-7f * (fabsf(fr) + fabsf((float)d[a]) + 2.f);
-                        const float gap = fmaxf(fmaxf(lo, hi) - slack, 0.f) * ehf[a];
-                        k2 = fmaf(gap, gap, k2);
-                    }
-                }
-                k2 *= 0.99999f;
-                if (in && k2 < bst) {
-                    const long long sy = G.en[0], sz = (long long)G.en[0] * G.en[1];
-                    const long long pidx = (long long)p[2] * sz + (long long)p[1] * sy + p[0];
+        unsigned head1 = 0, cnt1 = 0, head2 = 0, cnt2 = 0;   // the rings: [head, head + cnt)
+        unsigned r0 = 0;                           // first slot of the next round
+        int slot = 0, t = -1;                      // this lane's voxel and table entry (t < 0: no round)
+        for (;;) {
+            const bool rest = t < 0 && r0 >= nlive;            // every round is done: empty the rings
+            if (cnt2 >= 32u || (rest && cnt1 == 0u && cnt2 > 0u)) {
+                // ---- tier 3: the faces of the oldest pending cells ----
+                const unsigned n = min(cnt2, 32u);
+                if ((unsigned)lane < n) {
+                    const unsigned w = V.ring[1][(head2 + (unsigned)lane) & (kGqRing - 1)];
+                    const int own = (int)(w & 31u);
+                    const uint32_t off = G.table[G.toff[V.tv[own]] + (int)(w >> 5)].off;
+                    const int d[3] = {unpack10(off, 0), unpack10(off, 10), N == 3 ? unpack10(off, 20) : 0};
+                    const int p[3] = {V.c0[0][own] + d[0], V.c0[1][own] + d[1], V.c0[2][own] + d[2]};
                     const bool ex = p[0] + 1 < G.en[0], ey = p[1] + 1 < G.en[1], ez = N == 3 && p[2] + 1 < G.en[2];
-                    const float dr = V.dr[ld], inv = V.inv[ld];
-                    float qmin = kInf, qmax = -kInf;
+                    const float* q = G.ev + ((long long)p[2] * sz + (long long)p[1] * sy + p[0]);
+                    const float odr = V.dr[own], oinv = V.inv[own];
+                    float cq[8];
+                    uint32_t ok = 0;
 #pragma unroll
-                    for (int u = 0; u < (1 << N); ++u) {
-                        const bool present = (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez);
-                        if (present) {
-                            const long long o = pidx + ((u & 1) ? 1 : 0) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0);
-                            q[u] = (__ldg(G.ev + o) - dr) * inv;
-                            qmin = fminf(qmin, q[u]);
-                            qmax = fmaxf(qmax, q[u]);
+                    for (int u = 0; u < 8; ++u) {
+                        cq[u] = kNaN;
+                        if (u < (1 << N) && (!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
+                            cq[u] = rel_dose(__ldg(q + (u & 1) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0)), odr, oinv);
                             ok |= 1u << u;
                         }
                     }
-                    const float gap = qmin > 0.f ? qmin : (qmax < 0.f ? -qmax : 0.f);
-                    const float kb = sqrtf(fmaxf(k2, key * key));
-                    cand = fmaf(gap, gap, kb * kb) < bst;
+                    CellGeom<float> cg;
+                    cell_geom<N, float>((float)d[0] - V.fr[0][own], (float)d[1] - V.fr[1][own],
+                                        N == 3 ? (float)d[2] - V.fr[2][own] : 0.f, G.mt, cg);
+                    bool ill = false;
+                    const float cb = cell_min_d2<N, float>(cq, cg, G.mt, dmax, kInf, ill);
+                    if (ill && cell_gram_ill<N>(cq, ok, G.mt.kappa, G.tau))
+                        atomicOr(&W.fixm, 1u << own);                  // searched again
+                    else
+                        atomicMin(&W.best[own], __float_as_uint(cb + 0.f));   // -0 -> +0
                 }
+                head2 += n;
+                cnt2 -= n;
+                __syncwarp();
+                continue;
             }
-        }
-        // 5. append the surviving cells to the ring
-        const unsigned cm = __ballot_sync(kFull, cand);
-        if (cand) {
-            const unsigned seq = head + count + (unsigned)__popc(cm & lt_mask);
-            const int slot = (int)(seq & (kGqRing - 1));
+            if (cnt1 >= 32u || (rest && cnt1 > 0u)) {
+                // ---- tier 2: plane_bound of the oldest cells past tier 1 ----
+                const unsigned n = min(cnt1, 32u);
+                bool cand = false;
+                unsigned w = 0;
+                if ((unsigned)lane < n) {
+                    w = V.ring[0][(head1 + (unsigned)lane) & (kGqRing - 1)];
+                    const int own = (int)(w & 31u);
+                    const uint32_t off = G.table[G.toff[V.tv[own]] + (int)(w >> 5)].off;
+                    const int d[3] = {unpack10(off, 0), unpack10(off, 10), N == 3 ? unpack10(off, 20) : 0};
+                    const float* q = G.ev + ((long long)(V.c0[2][own] + d[2]) * sz +
+                                             (long long)(V.c0[1][own] + d[1]) * sy + (V.c0[0][own] + d[0]));
+                    float dose[8], c[3] = {0.f, 0.f, 0.f}, hn2[3], kap[3];
 #pragma unroll
-            for (int u = 0; u < (1 << N); ++u) V.q[u][slot] = q[u];
+                    for (int u = 0; u < (1 << N); ++u)
+                        dose[u] = __ldg(q + (u & 1) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0));
 #pragma unroll
-            for (int a = 0; a < 3; ++a) V.cf[a][slot] = cf[a];
-            V.meta[slot] = (unsigned)ws | (ok << 8);
+                    for (int a = 0; a < N; ++a) {
+                        c[a] = (float)d[a] - V.fr[a][own];
+                        hn2[a] = G.mt.hn2[a];
+                        kap[a] = G.mt.kappa[1 << a];
+                    }
+                    cand = off != V.skip[own] &&
+                           !(plane_bound<N>(dose, c, V.dr[own], V.inv[own], hn2, kap) >=
+                             __uint_as_float(V.best[own]) * kPlaneSlack);
+                }
+                head1 += n;
+                cnt1 -= n;
+                const unsigned cm = __ballot_sync(kFull, cand);
+                if (cand) V.ring[1][(head2 + cnt2 + (unsigned)__popc(cm & lt_mask)) & (kGqRing - 1)] = w;
+                cnt2 += (unsigned)__popc(cm);
+                __syncwarp();
+                continue;
+            }
+            if (t < 0) {
+                if (r0 >= nlive) break;                        // the batch is done
+                slot = (int)r0 + lane / g;                     // the next round
+                r0 += nv;
+                t = gl;
+            }
+            // the lane's voxel (from shared memory after every pass of the other tiers)
+            const bool live = (unsigned)slot < nlive;
+            const int sl = live ? slot : 0;
+            int c0[3];
+            float fr[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                c0[a] = V.c0[a][sl];
+                fr[a] = V.fr[a][sl];
+            }
+            const float dr = V.dr[sl], inv = V.inv[sl];
+            const float best = live ? __uint_as_float(V.best[sl]) : -1.f;   // < 0: nothing is below it
+            const TableEntry* const tab = G.table + G.toff[V.tv[sl]];
+            const int ntable = G.tlen[V.tv[sl]];
+            do {
+                // ---- tier 1: one table entry per lane and step ----
+                TableEntry e{0u, kInf};
+                if (t < ntable) e = tab[t];
+                const float key2 = e.key * e.key;
+                const bool keyed = key2 < best;
+                if (!__any_sync(kFull, keyed)) {               // A1 step 4b-ii, exact
+                    t = -1;
+                    break;
+                }
+                const unsigned ent = (unsigned)t;
+                t += g;
+                bool cand = false, edge = false;               // edge: a cell with vertices outside the grid
+                if (keyed) {
+                    const int d[3] = {unpack10(e.off, 0), unpack10(e.off, 10), N == 3 ? unpack10(e.off, 20) : 0};
+                    int p[3];
+                    bool in = true;
+                    // the distance from the point to the cell's box: a lower bound
+                    // in FP32 from the integer offset and the point's fraction,
+                    // each axis lowered by its rounding (4 ulp of its operands) and
+                    // the sum by 1e-5
+                    float k2 = 0.f;
+#pragma unroll
+                    for (int a = 0; a < N; ++a) {
+                        p[a] = c0[a] + d[a];
+                        in = in && (unsigned)p[a] < (unsigned)G.en[a];
+                        edge = edge || p[a] + 1 >= G.en[a];
+                        const float lo = (float)d[a] - fr[a];
+                        const float slack = 4.8e-7f * (fabsf(fr[a]) + fabsf((float)d[a]) + 2.f);
+                        const float gap = fmaxf(fmaxf(lo, -1.f - lo) - slack, 0.f) * eh[a];
+                        k2 = fmaf(gap, gap, k2);
+                    }
+                    k2 = fmaxf(k2 * 0.99999f, key2);
+                    if (in && k2 < best) {
+                        const float* q = G.ev + ((long long)(N == 3 ? p[2] : 0) * sz + (long long)p[1] * sy + p[0]);
+                        float dlo = kInf, dhi = -kInf;
+                        if (!edge) {
+                            float f[8];
+#pragma unroll
+                            for (int u = 0; u < (1 << N); ++u)
+                                f[u] = __ldg(q + (u & 1) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0));
+                            dlo = fminf(min3(f[0], f[1], f[2]), f[3]);
+                            dhi = fmaxf(max3(f[0], f[1], f[2]), f[3]);
+                            if constexpr (N == 3) {
+                                dlo = min3(min3(dlo, f[4], f[5]), f[6], f[7]);
+                                dhi = max3(max3(dhi, f[4], f[5]), f[6], f[7]);
+                            }
+                        } else {
+                            const bool ex = p[0] + 1 < G.en[0], ey = p[1] + 1 < G.en[1],
+                                       ez = N == 3 && p[2] + 1 < G.en[2];
+#pragma unroll
+                            for (int u = 0; u < (1 << N); ++u) {
+                                if ((!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
+                                    const float f = __ldg(q + (u & 1) + ((u & 2) ? sy : 0) + ((u & 4) ? sz : 0));
+                                    dlo = fminf(dlo, f);
+                                    dhi = fmaxf(dhi, f);
+                                }
+                            }
+                        }
+                        const float gap = max3(dlo - dr, dr - dhi, 0.f) * inv;
+                        cand = fmaf(gap, gap, k2) < best;
+                    }
+                }
+                // a whole cell goes to tier 2, one at the grid's edge to tier 3
+                const unsigned cm = __ballot_sync(kFull, cand && !edge);
+                if (cand && !edge)
+                    V.ring[0][(head1 + cnt1 + (unsigned)__popc(cm & lt_mask)) & (kGqRing - 1)] = ent << 5 | (unsigned)slot;
+                cnt1 += (unsigned)__popc(cm);
+                const unsigned em = __ballot_sync(kFull, cand && edge);
+                if (em) {
+                    if (cand && edge)
+                        V.ring[1][(head2 + cnt2 + (unsigned)__popc(em & lt_mask)) & (kGqRing - 1)] = ent << 5 | (unsigned)slot;
+                    cnt2 += (unsigned)__popc(em);
+                }
+            } while (max(cnt1, cnt2) < 32u);
+            __syncwarp();
         }
-        if (leader && walking) {
-            if (ended) {
-                sta = (sta & ~kGqWalk) | kGqEnded;
+        // ---- final values, one voxel per lane ----
+        const unsigned fixm = V.fixm;
+        if ((unsigned)lane < nlive) {
+            const float b = __uint_as_float(V.best[lane]), rc = G.tcover[V.tv[lane]];
+            const unsigned v = V.vox[lane];
+            if (((fixm >> lane) & 1u) || !(b <= rc * rc)) {
+                G.walk_list[atomicAdd(&G.ctr->fix_count, 1u)] = v;     // k_grid_walk finishes it
             } else {
-                V.t[ld] = t0 + GL;
-                const unsigned gm = cm & gmask;
-                if (gm) {                   // the group's last appended cell
-                    const int hl = 31 - __clz(gm);
-                    V.wseq[ld] = head + count + (unsigned)__popc(cm & ((1u << hl) - 1u));
-                    sta |= kGqWPend;
-                }
+                const float gam = sqrtf(b);
+                G.out[v] = gam;
+                ++my_eval;
+                my_pass += gam <= 1.f;
             }
-            V.state[ld] = sta;
         }
-        count += (unsigned)__popc(cm);
-        const int nwalk = GL * __popc(__ballot_sync(kFull, leader && (sta & kGqWalk) && !ended));
         __syncwarp();
-        // 6. evaluate the oldest 32 pending cells (or fewer, when few lanes walk)
-        if (count >= 32u || (count > 0u && nwalk < 16)) {
-            const unsigned n = min(count, 32u);
-            if ((unsigned)lane < n) {
-                const int slot = (int)((head + (unsigned)lane) & (kGqRing - 1));
-                const unsigned meta = V.meta[slot];
-                const int owner = (int)(meta & 63u);
-                const unsigned cok = meta >> 8;
-                float cq[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) cq[u] = u < (1 << N) ? V.q[u][slot] : 0.f;
-                CellGeom<float> cg;
-                cell_geom<N, float>(V.cf[0][slot], V.cf[1][slot], N == 3 ? V.cf[2][slot] : 0.f, G.mt, cg);
-                bool ill = false;
-                const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
-                const float cb = cell_min_d2<N, float>(cq, cg, G.mt, dmax, kInf, ill);
-                if (ill && cell_gram_ill<N>(cq, cok, G.mt.kappa, G.tau))
-                    atomicOr(&W.fixm[owner >> 5], 1u << (owner & 31));   // searched again
-                else
-                    atomicMin(&W.best[owner], __float_as_uint(cb + 0.f));   // -0 -> +0
-            }
-            head += n;
-            count -= n;
-        }
+        if (lane == 0 && fixm) W.fixm = 0;
         __syncwarp();
     }
-    unsigned c0 = W.cnt[0][lane], c1 = W.cnt[1][lane];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        c0 += __shfl_xor_sync(kFull, c0, o);
-        c1 += __shfl_xor_sync(kFull, c1, o);
+        my_eval += __shfl_xor_sync(kFull, my_eval, o);
+        my_pass += __shfl_xor_sync(kFull, my_pass, o);
     }
     if (lane == 0) {
-        if (c0) atomicAdd(&G.ctr->n_eval, (unsigned long long)c0);
-        if (c1) atomicAdd(&G.ctr->n_pass, (unsigned long long)c1);
+        if (my_eval) atomicAdd(&G.ctr->n_eval, (unsigned long long)my_eval);
+        if (my_pass) atomicAdd(&G.ctr->n_pass, (unsigned long long)my_pass);
     }
 }
 
@@ -649,39 +740,24 @@ int build_grid_table(int nd, const double hn[3], const int en[3], long long cap,
     return GAMMA_OK;
 }
 
-template <int N>
-static void launch_grid_walk_n(const GridProblem& G, int gl, int grid, cudaStream_t s)
-{
-    switch (gl) {
-    case 2: k_grid_walk<N, 2><<<grid, 256, 0, s>>>(G); break;
-    case 4: k_grid_walk<N, 4><<<grid, 256, 0, s>>>(G); break;
-    case 16: k_grid_walk<N, 16><<<grid, 256, 0, s>>>(G); break;
-    case 32: k_grid_walk<N, 32><<<grid, 256, 0, s>>>(G); break;
-    default: k_grid_walk<N, 8><<<grid, 256, 0, s>>>(G); break;
-    }
-}
-
 cudaError_t launch_grids(const GridProblem& G, cudaStream_t s)
 {
     const int sms = device_sm_count();
     const long long nmax = std::max(G.nref, G.neval);
     const int gp = (int)std::max<long long>(1, std::min<long long>((nmax + 255) / 256, (long long)sms * 8));
     k_grid_prepare<<<gp, 256, 0, s>>>(G);
-    if (G.walk == 3 && G.walk_list) {
-        // the warp-evaluated walk, then a 32-lane search of the voxels it left
-        if (G.ndim == 3) k_grid_cq<3, 8><<<sms * 2, 256, 0, s>>>(G);
-        else k_grid_cq<2, 8><<<sms * 2, 256, 0, s>>>(G);
-        GridProblem F = G;
-        F.from_list = 1;
-        if (G.ndim == 3) launch_grid_walk_n<3>(F, 32, sms * 2, s);
-        else launch_grid_walk_n<2>(F, 32, sms * 2, s);
-        return cudaGetLastError();
+    // bounds from plane seeds, the tiered walk, then a 32-lane search of the
+    // voxels it left
+    const int gs = (int)std::max<long long>(1, std::min<long long>((G.nref + 255) / 256, (long long)sms * 8));
+    if (G.ndim == 3) {
+        k_grid_seed<3><<<gs, 256, 0, s>>>(G);
+        k_grid_cq<3><<<sms * 2, 384, 0, s>>>(G);
+        k_grid_walk<3, 32><<<sms * 2, 256, 0, s>>>(G);
+    } else {
+        k_grid_seed<2><<<gs, 256, 0, s>>>(G);
+        k_grid_cq<2><<<sms * 2, 384, 0, s>>>(G);
+        k_grid_walk<2, 32><<<sms * 2, 256, 0, s>>>(G);
     }
-    const int gl = G.lanes;
-    const int gw = (int)std::max<long long>(1, std::min<long long>((G.nref * gl + 255) / 256,
-                                                                   (long long)sms * 16));
-    if (G.ndim == 3) launch_grid_walk_n<3>(G, gl, gw, s);
-    else launch_grid_walk_n<2>(G, gl, gw, s);
     return cudaGetLastError();
 }
 

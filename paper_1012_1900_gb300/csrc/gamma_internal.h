@@ -371,9 +371,10 @@ struct GridProblem {
     float tcover[9];
     Counters* ctr;
     int lanes;                   // lanes per reference voxel (2 .. 32)
-    int walk;                    // 3: the warp-evaluated walk (k_grid_cq), else k_grid_walk
+    double ua[3], ub[3];         // evaluation voxel units of reference index i: ua + i ub
+    unsigned* queue;             // evaluated voxels (nref entries), and the packed offset of the cell
+    unsigned* skip;              // each one's plane seed evaluated
     unsigned* walk_list;         // voxels k_grid_cq leaves to k_grid_walk (nref entries)
-    int from_list;               // k_grid_walk: walk only walk_list[0 .. ctr->fix_count)
 };
 int build_grid_table(int nd, const double hn[3], const int en[3], long long cap, int variant,
                      std::vector<TableEntry>& table, double& r_cover);
