@@ -1,24 +1,23 @@
-// BF16 GEMM with FP32 accumulation on the fifth-generation tensor cores, for
-// the training passes of the proposal network:
+// The weight gradients of the proposal network on the fifth-generation tensor
+// cores, both in one launch:
 //
-//     C[m][n] (+)= sum_k A[m][k] B[n][k]        (A: M x K, B: N x K, both K-major)
+//     dW1 += dZ1^T X   (128 x 384),     dW2 += dZ2^T H1   (128 x 128)
 //
-// One block of 128 threads computes a 128 x BN tile of C (BN 128, or 64 when
-// that gives the SMs more blocks, or 16 for the output layer).  Thread 0
-// streams the K dimension in chunks of 64 through three shared-memory stages,
-// each chunk's copy issued two chunks ahead of its MMAs: each chunk of A
-// and B arrives by TMA as eight 16-byte-wide column slices (one box of 8 x 128
-// or 8 x BN elements each), which is exactly the no-swizzle K-major core-matrix
-// layout the MMA descriptors expect (adjacent 8-row groups 128 bytes apart,
-// adjacent 8-column slices rows * 16 bytes apart).  It issues four
-// tcgen05.mma (K = 16) per chunk into one TMEM accumulator and commits them to
-// the stage's mbarrier, which frees the stage for the copy three chunks later.
-// A product split over K runs about two blocks per SM, which add their tiles.
-// After the last commit the four warps read their 32 TMEM lanes and store (or,
-// split over K, atomically add) the FP32 tile.  Rows and columns past the
-// matrices' ends are filled with zeros by the copies and never stored.  Every
-// wait is bounded: a wait that gives up raises the caller's error flag and the
-// block leaves without storing.
+// with the batch as K.  The operands come transposed from the rows' kernel
+// (dZ1T, dZ2T: [128][rows]; XT: [384][rows]; H1T: [128][rows]; BF16, K-major).
+// A block of 128 threads takes one 128 x 64 tile of dW1 (six) or dW2 (two) and
+// a part of the rows, so that the batch is split over about two blocks per SM.
+// Thread 0 streams the rows in chunks of 64 through four stages: a chunk of A
+// (128 x 128 bytes) and of B (64 x 128 bytes) is one TMA box each, with the
+// 128-byte swizzle the MMA descriptors name.  Four tcgen05.mma (K = 16) per
+// chunk go into one TMEM accumulator, whose FP32 tile the four warps then add
+// into the gradient, four columns per reduction.  Rows past the batch are
+// filled with zeros by the copies.  Every wait is bounded: a wait that gives up
+// raises the caller's error flag and the block leaves without adding.
+//
+// Bound by latency (a block has four chunks of a batch of 8,192 rows).  As two
+// GEMMs with boxes of 16-byte rows, after four transposes through memory, this
+// took 63 us of a training step of 8,192 rows.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -34,36 +33,39 @@ using bf16 = __nv_bfloat16;
 
 namespace {
 
-constexpr int kGemmBM = 128;             // rows per tile (MMA M)
-constexpr int kGemmBK = 64;              // K per stage
-constexpr int kGemmStages = 3;           // stages in flight
+constexpr int kGemmBM = 128;             // rows of a tile (MMA M: the output features)
+constexpr int kGemmBN = 64;              // columns of a tile
+constexpr int kGemmBK = 64;              // batch rows per stage
+constexpr int kGemmStages = 4;           // stages in flight
+constexpr int kTiles1 = kInPad / kGemmBN, kTiles2 = kH / kGemmBN;
 
-template <int BN>
-struct GemmSmem {
-    bf16 A[kGemmStages][kGemmBM * kGemmBK];   // per stage: 8 slices of 128 rows x 16 bytes
-    bf16 B[kGemmStages][BN * kGemmBK];        // per stage: 8 slices of BN rows x 16 bytes
+struct __align__(1024) GemmSmem {
+    bf16 A[kGemmStages][kGemmBM * kGemmBK];   // 128 rows x 128 bytes per stage (128-byte swizzle)
+    bf16 B[kGemmStages][kGemmBN * kGemmBK];   // 64 rows x 128 bytes
     uint64_t full[kGemmStages], empty[kGemmStages], done;
     uint32_t tmem;
     int ok;
 };
 
-template <int BN, bool ATOMIC>
-__global__ void __launch_bounds__(128, 1)
-    k_gemm_tc(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
-              int M, int N, int nchunks, int chunks_per_split, float* __restrict__ C, int ldc,
-              unsigned* flags)
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d)
 {
-    static_assert(BN == 16 || BN == 64 || BN == 128, "tile width");
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(128, 1)
+    k_wgrad(const __grid_constant__ WgradMaps maps, int nchunks, int chunks_per_split, float* __restrict__ gW1,
+            float* __restrict__ gW2, unsigned* flags)
+{
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // the stages start on a 1 KB boundary (TMA destinations: 128 bytes)
     unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-    GemmSmem<BN>& S = *reinterpret_cast<GemmSmem<BN>*>(base);
+    GemmSmem& S = *reinterpret_cast<GemmSmem*>(base);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * kGemmBM, n0 = blockIdx.x * BN;
-    const int c0 = blockIdx.z * chunks_per_split;
-    const int c1 = min(nchunks, c0 + chunks_per_split);
-    if (c0 >= c1) return;                                 // block-uniform: an empty K split
-    constexpr uint32_t kTmemCols = BN < 32 ? 32 : BN;
+    const bool first = blockIdx.x < kTiles1;                  // a tile of dW1, else of dW2
+    const int n0 = (first ? (int)blockIdx.x : (int)blockIdx.x - kTiles1) * kGemmBN;
+    const int c0 = blockIdx.y * chunks_per_split;
+    const int nloc = min(nchunks, c0 + chunks_per_split) - c0;
+    if (nloc <= 0) return;                                    // block-uniform: an empty part
     if (tid == 0) {
         for (int b = 0; b < kGemmStages; ++b) {
             mbar_init(&S.full[b], 1);
@@ -74,7 +76,7 @@ __global__ void __launch_bounds__(128, 1)
         S.ok = 1;
     }
     if (warp == 0) {
-        tmem_alloc(&S.tmem, kTmemCols);
+        tmem_alloc(&S.tmem, kGemmBN);
         tmem_relinquish();
     }
     tc_fence_before_sync();
@@ -82,77 +84,57 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_after_sync();
     const uint32_t tm = S.tmem;
     if (tid == 0) {
-        constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, BN);
-        constexpr uint32_t kBytes = (kGemmBM + BN) * kGemmBK * 2;
-        uint32_t nfull[kGemmStages] = {}, nempty[kGemmStages] = {};
-        bool pending[kGemmStages] = {};                   // a copy issued but not yet seen landed
+        constexpr uint32_t kId = idesc_bf16_f32(kGemmBM, kGemmBN);
+        constexpr uint32_t kBytes = (kGemmBM + kGemmBN) * kGemmBK * 2;
+        const CUtensorMap* am = first ? &maps.dz1 : &maps.dz2;
+        const CUtensorMap* bm = first ? &maps.x : &maps.h1;
         bool ok = true;
-        // chunk i (from c0) goes to stage i % kGemmStages; its copy is issued
-        // kGemmStages - 1 chunks ahead of its MMAs
+        int loaded = 0, used = 0;                             // chunks requested, chunks seen landed
         auto load = [&](int i) {
             const int s = i % kGemmStages;
-            if (i >= kGemmStages) {                       // the MMAs of chunk i - kGemmStages read it
-                ok = mbar_wait_bounded(&S.empty[s], nempty[s] & 1u);
-                ++nempty[s];
-                if (!ok) return;
-            }
+            if (i >= kGemmStages) ok = mbar_wait_bounded(&S.empty[s], (i / kGemmStages - 1) & 1u);
+            if (!ok) return;
             mbar_arrive_expect_tx(&S.full[s], kBytes);
-            pending[s] = true;
             const int k0 = (c0 + i) * kGemmBK;
-#pragma unroll
-            for (int j = 0; j < kGemmBK / 8; ++j) {
-                tma_load_2d(&S.A[s][j * kGemmBM * 8], &amap, k0 + 8 * j, m0, &S.full[s]);
-                tma_load_2d(&S.B[s][j * BN * 8], &bmap, k0 + 8 * j, n0, &S.full[s]);
-            }
+            tma_load_2d(S.A[s], am, k0, 0, &S.full[s]);
+            tma_load_2d(S.B[s], bm, k0, n0, &S.full[s]);
+            ++loaded;
         };
-        const int nloc = c1 - c0;
         for (int i = 0; i < kGemmStages - 1 && i < nloc && ok; ++i) load(i);
-        for (int c = c0; c < c1 && ok; ++c) {
-            const int i = c - c0, s = i % kGemmStages;
+        for (int i = 0; i < nloc && ok; ++i) {
             if (i + kGemmStages - 1 < nloc) load(i + kGemmStages - 1);
             if (!ok) break;
-            ok = mbar_wait_bounded(&S.full[s], nfull[s] & 1u);
+            const int s = i % kGemmStages;
+            ok = mbar_wait_bounded(&S.full[s], (i / kGemmStages) & 1u);
             if (!ok) break;
-            pending[s] = false;
-            ++nfull[s];
+            ++used;
             tc_fence_after_sync();
+            const uint32_t aa = smem_addr(S.A[s]), ba = smem_addr(S.B[s]);
 #pragma unroll
-            for (int kk = 0; kk < kGemmBK; kk += 16) {
-                const uint32_t la = kGemmBM * 16u, lb = BN * 16u;    // bytes between 8-column slices
-                const uint64_t ad = smem_desc(smem_addr(&S.A[s][0]) + (uint32_t)(kk >> 3) * la, la, 128u);
-                const uint64_t bd = smem_desc(smem_addr(&S.B[s][0]) + (uint32_t)(kk >> 3) * lb, lb, 128u);
-                tc_mma_bf16(tm, ad, bd, kId, (c > c0 || kk > 0) ? 1u : 0u);
-            }
+            for (int kk = 0; kk < kGemmBK; kk += 16)
+                tc_mma_bf16(tm, smem_desc_sw128(aa, kk * 2), smem_desc_sw128(ba, kk * 2), kId, (i | kk) != 0);
             tc_commit(&S.empty[s]);
         }
         tc_commit(&S.done);
         if (!ok) {
             S.ok = 0;
             // let this block's copies land before it leaves
-            for (int b = 0; b < kGemmStages; ++b)
-                if (pending[b]) mbar_wait_bounded(&S.full[b], nfull[b] & 1u);
+            for (int i = used; i < loaded; ++i) mbar_wait_bounded(&S.full[i % kGemmStages], (i / kGemmStages) & 1u);
         }
     }
     // every thread waits for the accumulator (bounded), then the epilogue
     const bool landed = mbar_wait_bounded(&S.done, 0u);
-    const bool ok = __syncthreads_and(landed) && S.ok;      // block-uniform
+    const bool ok = __syncthreads_and(landed) && S.ok;        // block-uniform
     tc_fence_after_sync();
     if (ok) {
-        const int row = m0 + 32 * warp + lane;
-#pragma unroll 1
-        for (int j = 0; j < BN; j += 16) {
-            float v[16];
-            tmem_ld16(tm + ((uint32_t)(32 * warp) << 16) + (uint32_t)j, v);
-            if (row < M) {
-                float* dst = C + (long long)row * ldc + n0 + j;
+        const int row = 32 * warp + lane;
+        float* dst = first ? gW1 + (long long)row * kInPad + n0 : gW2 + (long long)row * kH + n0;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    if (n0 + j + u < N) {
-                        if (ATOMIC) atomicAdd(dst + u, v[u]);
-                        else dst[u] = v[u];
-                    }
-                }
-            }
+        for (int j = 0; j < kGemmBN; j += 32) {
+            float v[32];
+            tmem_ld32(tm + ((uint32_t)(32 * warp) << 16) + (uint32_t)j, v);
+#pragma unroll
+            for (int u = 0; u < 32; u += 4) red_add4(dst + j + u, v[u], v[u + 1], v[u + 2], v[u + 3]);
         }
     } else if (tid == 0) {
         atomicOr(flags, kFlagTimeout);
@@ -160,93 +142,33 @@ __global__ void __launch_bounds__(128, 1)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    if (warp == 0) tmem_dealloc(tm, kGemmBN);
 }
 
 }  // namespace
 
-template <int BN, bool ATOMIC>
-static cudaError_t launch_gemm_tc_k(const CUtensorMap& am, const CUtensorMap& bm, long long M, int N,
-                                    int nchunks, int per, int splits, float* C, int ldc,
-                                    unsigned* flags, cudaStream_t s)
+bool encode_wgrad_maps(WgradMaps* maps, const bf16* dZ1T, const bf16* XT, const bf16* dZ2T, const bf16* H1T,
+                       long long M, long long Mp)
 {
-    const size_t smem = sizeof(GemmSmem<BN>) + 1024;      // room to align the base to 1 KB
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<BN, ATOMIC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + kGemmBM - 1) / kGemmBM),
-                    (unsigned)splits);
-    k_gemm_tc<BN, ATOMIC><<<grid, 128, smem, s>>>(am, bm, (int)M, N, nchunks, per, C, ldc, flags);
-    return cudaGetLastError();
+    const unsigned long long rows = (unsigned long long)M, stride = (unsigned long long)Mp * 2;
+    return encode_bf16_2d(&maps->dz1, dZ1T, rows, kH, stride, kGemmBK, kGemmBM, true) &&
+           encode_bf16_2d(&maps->x, XT, rows, kInPad, stride, kGemmBK, kGemmBN, true) &&
+           encode_bf16_2d(&maps->dz2, dZ2T, rows, kH, stride, kGemmBK, kGemmBM, true) &&
+           encode_bf16_2d(&maps->h1, H1T, rows, kH, stride, kGemmBK, kGemmBN, true);
 }
 
-cudaError_t launch_gemm_tc(const bf16* A, long long M, long long lda, const bf16* B, int N,
-                           long long ldb, long long K, float* C, int ldc, int splits,
-                           unsigned* flags, cudaStream_t s)
+cudaError_t launch_wgrad(const WgradMaps& maps, long long M, float* gW1, float* gW2, unsigned* flags,
+                         cudaStream_t s)
 {
-    if (M <= 0 || N <= 0 || K <= 0 || splits < 1) return cudaErrorInvalidValue;
-    if ((lda % 8) || (ldb % 8) || (((uintptr_t)A | (uintptr_t)B) & 15u)) return cudaErrorInvalidValue;
-    const long long mtiles = (M + kGemmBM - 1) / kGemmBM;
-    // the widest tile that still gives every SM a block (else 64 columns)
-    const int bn = N <= 16 ? 16 : (mtiles * ((N + 127) / 128) >= device_sm_count() ? 128 : 64);
-    CUtensorMap am, bm;
-    // A: K x M elements (inner, rows), boxes of 8 x 128; B: K x N, boxes of 8 x bn
-    if (!encode_bf16_2d(&am, A, (unsigned long long)K, (unsigned long long)M,
-                        (unsigned long long)lda * 2, 8, kGemmBM) ||
-        !encode_bf16_2d(&bm, B, (unsigned long long)K, (unsigned long long)N,
-                        (unsigned long long)ldb * 2, 8, (unsigned)bn))
-        return cudaErrorInvalidValue;
-    const int nchunks = (int)((K + kGemmBK - 1) / kGemmBK);
-    if (splits > 1) {
-        // a split-K product: about two blocks per SM
-        const long long tiles = mtiles * ((N + bn - 1) / bn);
-        splits = (int)std::max<long long>(splits, (2LL * device_sm_count() + tiles - 1) / tiles);
-        splits = std::min(splits, std::max(1, nchunks / 4));   // at least 4 chunks a block
-    }
-    splits = std::min(splits, nchunks);
+    const size_t smem = sizeof(GemmSmem) + 1024;              // room to align the base to 1 KB
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int nchunks = (int)((M + kGemmBK - 1) / kGemmBK), tiles = kTiles1 + kTiles2;
+    // about two blocks per SM, with at least four chunks each
+    int splits = std::max(1, std::min((2 * device_sm_count() + tiles - 1) / tiles, nchunks / 4));
     const int per = (nchunks + splits - 1) / splits;
     splits = (nchunks + per - 1) / per;
-    const bool atomic = splits > 1;
-    if (bn == 16) {
-        return atomic ? launch_gemm_tc_k<16, true>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s)
-                      : launch_gemm_tc_k<16, false>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s);
-    }
-    if (bn == 64) {
-        return atomic ? launch_gemm_tc_k<64, true>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s)
-                      : launch_gemm_tc_k<64, false>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s);
-    }
-    return atomic ? launch_gemm_tc_k<128, true>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s)
-                  : launch_gemm_tc_k<128, false>(am, bm, M, N, nchunks, per, splits, C, ldc, flags, s);
-}
-
-// Transpose of a bf16 matrix: src [rows][cols] (row stride lds) -> dst
-// [cols][rows] (row stride ldd >= rows; columns rows .. ldd - 1 are zeroed).
-__global__ void __launch_bounds__(256) k_transpose_bf16(const bf16* __restrict__ src, long long rows,
-                                                        int cols, long long lds, bf16* __restrict__ dst,
-                                                        long long ldd)
-{
-    __shared__ bf16 t[32][33];
-    const long long r0 = (long long)blockIdx.x * 32;
-    const int c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
-    for (int j = ty; j < 32; j += 8) {
-        const long long r = r0 + j;
-        const int c = c0 + tx;
-        t[j][tx] = (r < rows && c < cols) ? src[r * lds + c] : __float2bfloat16(0.f);
-    }
-    __syncthreads();
-    for (int j = ty; j < 32; j += 8) {
-        const int c = c0 + j;
-        const long long r = r0 + tx;
-        if (c < cols && r < ldd) dst[(long long)c * ldd + r] = t[tx][j];
-    }
-}
-
-cudaError_t launch_transpose_bf16(const bf16* src, long long rows, int cols, long long lds, bf16* dst,
-                                  long long ldd, cudaStream_t s)
-{
-    const dim3 grid((unsigned)((ldd + 31) / 32), (unsigned)((cols + 31) / 32));
-    k_transpose_bf16<<<grid, 256, 0, s>>>(src, rows, cols, lds, dst, ldd);
+    k_wgrad<<<dim3((unsigned)tiles, (unsigned)splits), 128, smem, s>>>(maps, nchunks, per, gW1, gW2, flags);
     return cudaGetLastError();
 }
 

@@ -410,19 +410,17 @@ cudaError_t launch_batch_tail(const BatchGroup& g, int walk, int lanes_per_voxel
 bool encode_bf16_2d(CUtensorMap* map, const void* base, unsigned long long inner,
                     unsigned long long rows, unsigned long long row_stride_bytes,
                     unsigned box_inner, unsigned box_rows, bool swizzle = false);
-// C (+)= A B^T on the tensor cores (gamma_gemm_tc.cu): A [M][K] and B [N][K]
-// bf16 with K contiguous (row strides lda, ldb: multiples of 8 elements, bases
-// 16-byte aligned), C fp32 [M][ldc].  With splits > 1 the K range is split over
-// that many blocks per tile, which add into C (it must hold the initial value,
-// normally zero); else C is overwritten.  flags receives kFlagTimeout if a
-// bounded wait gave up.
-cudaError_t launch_gemm_tc(const __nv_bfloat16* A, long long M, long long lda, const __nv_bfloat16* B,
-                           int N, long long ldb, long long K, float* C, int ldc, int splits,
-                           unsigned* flags, cudaStream_t s);
-// dst [cols][ldd] = transpose of src [rows][cols] (row stride lds); the
-// columns rows .. ldd - 1 of dst are zeroed.
-cudaError_t launch_transpose_bf16(const __nv_bfloat16* src, long long rows, int cols, long long lds,
-                                  __nv_bfloat16* dst, long long ldd, cudaStream_t s);
+// Weight gradients of a training batch (gamma_gemm_tc.cu): gW1 [kH][kInPad] +=
+// dZ1^T X, gW2 [kH][kH] += dZ2^T H1, from the operands transposed ([column][row]
+// BF16, row stride Mp: a multiple of 8; bases and gradients 16-byte aligned).
+// flags receives kFlagTimeout if a bounded wait gave up.
+struct WgradMaps {
+    CUtensorMap dz1, x, dz2, h1;
+};
+bool encode_wgrad_maps(WgradMaps* maps, const __nv_bfloat16* dZ1T, const __nv_bfloat16* XT,
+                       const __nv_bfloat16* dZ2T, const __nv_bfloat16* H1T, long long M, long long Mp);
+cudaError_t launch_wgrad(const WgradMaps& maps, long long M, float* gW1, float* gW2, unsigned* flags,
+                         cudaStream_t s);
 
 // Learned seeding of a batch group (gamma_learned.cu): the queue items of every
 // pair whose cost bucket is at least min_bucket as (pair, item) rows, then the

@@ -294,149 +294,53 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ Problem 
 }
 
 // --------------------------------------------------------------------------
-// Training passes around the tensor-core GEMMs (gamma_gemm_tc.cu)
+// Optimiser
 // --------------------------------------------------------------------------
 
-// Z (M x N, fp32) += bias; H = bf16(relu(Z)) (or bf16(Z) without relu).
-__global__ void k_bias_act(long long M, int N, float* __restrict__ Z, const float* __restrict__ bias,
-                           bf16* __restrict__ H, int ldh, int relu)
-{
-    const long long total = M * N;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % N);
-        const float z = Z[e] + bias[c];
-        Z[e] = z;
-        if (H) H[(e / N) * ldh + c] = __float2bfloat16(relu ? fmaxf(z, 0.f) : z);
-    }
-}
-
-// Huber loss (delta 1) per output, averaged over the rows with finite
-// targets; dY = dloss / dy.  Y: M x kOutPad, T: M x kOut.
-__global__ void k_huber(long long M, const float* __restrict__ Y, const float* __restrict__ T,
-                        float* __restrict__ dY, float* __restrict__ loss, float inv_count)
-{
-    float acc = 0.f;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < M;
-         i += (long long)gridDim.x * blockDim.x) {
-        const bool valid = isfinite(T[4 * i + 3]);
-#pragma unroll
-        for (int j = 0; j < kOut; ++j) {
-            const float r = valid ? Y[i * kOutPad + j] - T[4 * i + j] : 0.f;
-            const float a = fabsf(r);
-            acc += a <= 1.f ? 0.5f * r * r : a - 0.5f;
-            dY[4 * i + j] = (a <= 1.f ? r : copysignf(1.f, r)) * inv_count;
+// Where parameter i goes among the BF16 copies of the weights (W2 also
+// transposed, for dH1): nothing for the biases.
+struct WeightCopies {
+    bf16 *W1h, *W2h, *W2Th, *W3h;
+    int off_w2, off_w3;                    // first parameters of W2 and W3 (W1 starts at 0)
+    __device__ __forceinline__ void put(int i, float p) const
+    {
+        const bf16 v = __float2bfloat16(p);
+        if (i < kH * kInPad) {
+            W1h[i] = v;
+        } else if (i >= off_w2 && i < off_w2 + kH * kH) {
+            const int k = i - off_w2;
+            W2h[k] = v;
+            W2Th[(k % kH) * kH + k / kH] = v;
+        } else if (i >= off_w3 && i < off_w3 + kOutPad * kH) {
+            W3h[i - off_w3] = v;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc * inv_count);
-}
+};
 
-// Output layer backward on CUDA cores (K = 4 is too thin for the tensor
-// cores): dZ2 = (dY W3) * [Z2 > 0] (bf16), and the partial sums of
-// dW3 = dY^T H2, db3 = sum dY.
-__global__ void k_out_back(long long M, const float* __restrict__ dY, const float* __restrict__ W3,
-                           const float* __restrict__ Z2, const bf16* __restrict__ H2,
-                           bf16* __restrict__ dZ2, float* __restrict__ gW3, float* __restrict__ gb3)
+// Adam on the FP32 master parameters, and their BF16 copies; padded entries
+// (mask == 0) stay zero.
+__global__ void __launch_bounds__(256) k_adam(int n, float* __restrict__ p, const float* __restrict__ g,
+                                              float* __restrict__ m, float* __restrict__ v,
+                                              const unsigned char* __restrict__ mask, WeightCopies copies,
+                                              float lr, float b1, float b2, float eps, float c1, float c2)
 {
-    __shared__ float sW3[kOut * kH];
-    __shared__ float sg[kOut * kH + kOut];
-    for (int i = threadIdx.x; i < kOut * kH; i += blockDim.x) {
-        sW3[i] = W3[i];
-        sg[i] = 0.f;
-    }
-    if (threadIdx.x < kOut) sg[kOut * kH + threadIdx.x] = 0.f;
-    __syncthreads();
-    const int c = threadIdx.x % kH;                  // blockDim.x is a multiple of kH
-    const int rstep = blockDim.x / kH;
-    float gw[kOut] = {0.f, 0.f, 0.f, 0.f}, gb[kOut] = {0.f, 0.f, 0.f, 0.f};
-    for (long long m = (long long)blockIdx.x * rstep + threadIdx.x / kH; m < M;
-         m += (long long)gridDim.x * rstep) {
-        float d = 0.f;
-#pragma unroll
-        for (int j = 0; j < kOut; ++j) d = fmaf(dY[4 * m + j], sW3[j * kH + c], d);
-        dZ2[m * kH + c] = __float2bfloat16(Z2[m * kH + c] > 0.f ? d : 0.f);
-        const float h = __bfloat162float(H2[m * kH + c]);
-#pragma unroll
-        for (int j = 0; j < kOut; ++j) {
-            gw[j] = fmaf(dY[4 * m + j], h, gw[j]);
-            if (c == 0) gb[j] += dY[4 * m + j];
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kOut; ++j) {
-        atomicAdd(&sg[j * kH + c], gw[j]);
-        if (c == 0) atomicAdd(&sg[kOut * kH + j], gb[j]);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kOut * kH; i += blockDim.x) atomicAdd(&gW3[i], sg[i]);
-    if (threadIdx.x < kOut) atomicAdd(&gb3[threadIdx.x], sg[kOut * kH + threadIdx.x]);
-}
-
-// dZ = bf16(dH * [Z > 0]) and the column sums of dZ (bias gradient).
-__global__ void k_relu_back(long long M, int N, const float* __restrict__ dH,
-                            const float* __restrict__ Z, bf16* __restrict__ dZ,
-                            float* __restrict__ gb)
-{
-    const long long total = M * N;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const float d = Z[e] > 0.f ? dH[e] : 0.f;
-        dZ[e] = __float2bfloat16(d);
-    }
-    (void)gb;
-}
-
-// Column sums of a bf16 matrix (M x N) into gb (atomic).
-__global__ void k_colsum(long long M, int N, const bf16* __restrict__ D, float* __restrict__ gb)
-{
-    const int c = blockIdx.y * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    float s = 0.f;
-    for (long long m = blockIdx.x; m < M; m += gridDim.x) s += __bfloat162float(D[m * N + c]);
-    atomicAdd(&gb[c], s);
-}
-
-// Adam on the FP32 master parameters; padded entries (mask == 0) stay zero.
-__global__ void k_adam(long long n, float* __restrict__ p, const float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, const unsigned char* __restrict__ mask,
-                       float lr, float b1, float b2, float eps, float c1, float c2)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         if (!mask[i]) continue;
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
         const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
         m[i] = mi;
         v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        p[i] = pi;
+        copies.put(i, pi);
     }
 }
 
-// bf16 copies of the weights (and W2^T for the backward GEMM).
-__global__ void k_cast_weights(const float* __restrict__ W1, const float* __restrict__ W2,
-                               const float* __restrict__ W3, bf16* __restrict__ W1h,
-                               bf16* __restrict__ W2h, bf16* __restrict__ W2Th,
-                               bf16* __restrict__ W3h)
+// The BF16 copies of all parameters.
+__global__ void __launch_bounds__(256) k_cast_weights(int n, const float* __restrict__ p, WeightCopies copies)
 {
-    const int total = kH * kInPad + 2 * kH * kH + kOutPad * kH;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-        if (e < kH * kInPad) {
-            W1h[e] = __float2bfloat16(W1[e]);
-        } else if (e < kH * kInPad + kH * kH) {
-            const int i = e - kH * kInPad;
-            W2h[i] = __float2bfloat16(W2[i]);
-        } else if (e < kH * kInPad + 2 * kH * kH) {
-            const int i = e - kH * kInPad - kH * kH;
-            const int r = i / kH, c = i % kH;            // W2T[r][c] = W2[c][r]
-            W2Th[i] = __float2bfloat16(W2[c * kH + r]);
-        } else {
-            const int i = e - kH * kInPad - 2 * kH * kH;
-            W3h[i] = __float2bfloat16(W3[i]);
-        }
-    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) copies.put(i, p[i]);
 }
 
 // --------------------------------------------------------------------------
@@ -503,18 +407,14 @@ __device__ __forceinline__ uint64_t tile_desc(const bf16* base, int rows, int k0
     return smem_desc(smem_addr(base) + (uint32_t)(k0 >> 3) * lbo, lbo, 128u);
 }
 
-// Index of a weight-staging thread (every warp but the copying one).
-__device__ __forceinline__ int stager()
-{
-    return (int)threadIdx.x - ((int)threadIdx.x >= kEpiWarps * 32 ? 32 : 0);
-}
-
-// Row-major [rows][K] BF16 weights (global) -> core-matrix tile (shared).
+// Row-major [rows][K] BF16 weights (global) -> core-matrix tile (shared), by
+// thread `first` of `step`.
 __device__ __forceinline__ void stage_weights(bf16* dst, const bf16* __restrict__ src, int rows,
-                                              int src_rows, int K)
+                                              int src_rows, int K, int first, int step)
 {
     const int n = rows * (K / 8);
-    for (int e = stager(); e < n; e += kStagers) {
+#pragma unroll 4
+    for (int e = first; e < n; e += step) {
         const int r = e / (K / 8), j = e % (K / 8);
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (r < src_rows) v = *reinterpret_cast<const uint4*>(src + (long long)r * K + j * 8);
@@ -523,10 +423,11 @@ __device__ __forceinline__ void stage_weights(bf16* dst, const bf16* __restrict_
 }
 
 // Row-major [128][384] BF16 weights (global) -> swizzled 64-column panels.
-__device__ __forceinline__ void stage_panels(bf16 (*dst)[kPanel], const bf16* __restrict__ src)
+__device__ __forceinline__ void stage_panels(bf16 (*dst)[kPanel], const bf16* __restrict__ src, int first,
+                                             int step)
 {
 #pragma unroll 8
-    for (int e = stager(); e < kH * (kInPad / 8); e += kStagers) {
+    for (int e = first; e < kH * (kInPad / 8); e += step) {
         const int r = e / (kInPad / 8), j = e % (kInPad / 8);
         *reinterpret_cast<uint4*>(dst[j >> 3] + r * kKc + (((j & 7) ^ (r & 7)) << 3)) =
             *reinterpret_cast<const uint4*>(src + (long long)r * kInPad + j * 8);
@@ -605,10 +506,10 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_rows(const __grid_consta
     __syncthreads();
     tc_fence_after_sync();
     if (warp != kEpiWarps) {             // (the rows' copies start meanwhile)
-        stage_panels(S.W1, W.W1);
-        stage_weights(S.W2, W.W2, kH, kH, kH);
-        stage_weights(S.W3, W.W3, kN3, kOutPad, kH);
         const int i = warp < kEpiWarps ? tid : tid - 32;
+        stage_panels(S.W1, W.W1, i, kStagers);
+        stage_weights(S.W2, W.W2, kH, kH, kH, i, kStagers);
+        stage_weights(S.W3, W.W3, kN3, kOutPad, kH, i, kStagers);
         for (int k = i; k < kH; k += kStagers) {
             S.b1[k] = W.b1[k];
             S.b2[k] = W.b2[k];
@@ -749,6 +650,371 @@ cudaError_t launch_mlp_infer(const MlpWeights& W, const bf16* X, long long M, fl
                              unsigned* host_flags, cudaStream_t s)
 {
     return launch_mlp_rows(W, X, M, nullptr, Y, host_flags, 1, s);
+}
+
+// --------------------------------------------------------------------------
+// Training: forward, loss and the backward pass of the rows in one kernel
+//
+// A block takes one tile of 128 rows through
+//   Z1 = X W1^T + b1, H1 = relu(Z1),  Z2 = H1 W2^T + b2, H2 = relu(Z2),
+//   Y = H2 W3^T + b3,  the Huber loss and dY,
+//   dZ2 = (dY W3) * [Z2 > 0],  dH1 = dZ2 W2,  dZ1 = dH1 * [Z1 > 0]
+// with the four products on the tensor cores (operands in shared memory,
+// accumulators in TMEM: columns 0..127 Z1 and then dH1, 128..255 Z2, 256..271
+// Y), the element-wise parts in the epilogue warps between them, and the ReLU
+// masks in their registers.  Per tile it adds the column sums (bias gradients,
+// dW3 = dY^T H2) to the gradients, and it writes what the weight-gradient
+// product needs, with the batch as K: X, H1, dZ1 and dZ2 transposed ([column]
+// [row], a lane per row, so that a warp's stores are 64 contiguous bytes).
+// Warp 8 copies the panels of X, warp 9 issues the MMAs.  Every wait is
+// bounded, and every warp passes every block barrier.
+//
+// What bounds it: the latency of one tile's chain (a training batch of 8,192
+// rows is 64 tiles).  Before, the same work took 17 launches: a GEMM per
+// product, bias, activation, loss, mask, column-sum and transpose passes
+// over memory: about 190 us of kernels in a step of 8,192 rows, now 42 us here
+// and 11 us in k_wgrad.
+// --------------------------------------------------------------------------
+
+struct __align__(1024) TrainSmem {
+    bf16 W1[kNChunks][kPanel];             // W1 panels (128-byte swizzle); W2^T (core matrices) once Z1 is done
+    bf16 Xc[kXStages][kPanel];             // X panels (128-byte swizzle); then dZ2 (core matrices)
+    bf16 W2[kH * kH];                      // core matrices, as below
+    bf16 H[kRows * kH];                    // H1, then H2
+    bf16 W3[kN3 * kH];
+    float W3f[kOut * kH];                  // the FP32 master of W3
+    float dY[kRows][kOut];
+    float gW3[kOut * kH], gb1[kH], gb2[kH], gb3[kOut];   // this tile's sums
+    float b1[kH], b2[kH], b3[kOutPad];
+    uint64_t xfull[kXStages], xempty[kXStages];   // (xempty: the MMAs and the eight transposing warps)
+    uint64_t d1, d2, d3, d4, h1, h2, z2;
+    uint32_t tmem;
+};
+static_assert(sizeof(TrainSmem) + 1024 <= kTcSmemBytes, "training tile does not fit in shared memory");
+static_assert(sizeof(bf16) * kXStages * kPanel >= sizeof(bf16) * kRows * kH, "dZ2 takes the X panels' place");
+
+struct TrainArgs {
+    MlpWeights W;
+    const bf16* W2T;                       // [kH][kH], W2 transposed
+    const float* W3f;                      // [kOutPad][kH], FP32 master
+    const float* T;                        // [M][kOut] targets
+    long long M, Mp;                       // rows; row stride of the transposed outputs
+    float inv_count;
+    bf16 *XT, *H1T, *dZ1T, *dZ2T;          // [kInPad or kH][Mp]
+    float *gb1, *gb2, *gW3, *gb3, *loss;
+    unsigned* flags;
+};
+
+// Column sums over a warp's 32 rows: lane l gets the sum of v[l] over the
+// lanes (31 exchanges for 32 columns).
+__device__ __forceinline__ float warp_column_sum(float (&v)[32])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {
+        const bool up = lane & m;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const float send = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+    return v[0];
+}
+
+constexpr int kTrainThreads = 320;
+
+__global__ void __launch_bounds__(kTrainThreads, 1) k_train_rows(const __grid_constant__ TrainArgs A,
+                                                                 const __grid_constant__ CUtensorMap xmap)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(base);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const long long row0 = (long long)blockIdx.x * kRows;
+    if (tid == 0) {
+        for (int b = 0; b < kXStages; ++b) {
+            mbar_init(&S.xfull[b], 1);
+            mbar_init(&S.xempty[b], 1 + kEpiWarps);
+        }
+        mbar_init(&S.d1, 1);
+        mbar_init(&S.d2, 1);
+        mbar_init(&S.d3, 1);
+        mbar_init(&S.d4, 1);
+        mbar_init(&S.h1, kEpiWarps);
+        mbar_init(&S.h2, kEpiWarps);
+        mbar_init(&S.z2, kEpiWarps);
+        mbar_fence_init();
+    }
+    if (warp == 0) {
+        tmem_alloc(&S.tmem, kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tm = S.tmem;
+    bool ok = true;
+    if (warp == kEpiWarps) {
+        // ---- the copies (from here on, while the others stage the weights) ----
+        if (lane == 0) {
+            int c = 0;
+            for (; c < kNChunks; ++c) {
+                const int s = c % kXStages;
+                if (c >= kXStages) ok = mbar_wait_bounded(&S.xempty[s], (c / kXStages - 1) & 1u);
+                if (!ok) break;
+                mbar_arrive_expect_tx(&S.xfull[s], kPanel * 2);
+                tma_load_2d(S.Xc[s], &xmap, c * kKc, (int)row0, &S.xfull[s]);
+            }
+            // the copies still in flight land before the block leaves
+            for (int k = max(0, c - kXStages); k < c; ++k) mbar_wait_bounded(&S.xfull[k % kXStages], (k / kXStages) & 1u);
+        }
+    } else {
+        constexpr int n = kTrainThreads - 32;
+        const int i0 = warp < kEpiWarps ? tid : tid - 32;
+        stage_panels(S.W1, A.W.W1, i0, n);
+        stage_weights(S.W2, A.W.W2, kH, kH, kH, i0, n);
+        stage_weights(S.W3, A.W.W3, kN3, kOutPad, kH, i0, n);
+        for (int k = i0; k < kOut * kH; k += n) {
+            S.W3f[k] = A.W3f[k];
+            S.gW3[k] = 0.f;
+        }
+        for (int k = i0; k < kH; k += n) {
+            S.b1[k] = A.W.b1[k];
+            S.b2[k] = A.W.b2[k];
+            S.gb1[k] = S.gb2[k] = 0.f;
+        }
+        if (i0 < kOutPad) S.b3[i0] = A.W.b3[i0];
+        if (i0 < kOut) S.gb3[i0] = 0.f;
+        fence_async_shared();
+        asm volatile("bar.sync 1, %0;" ::"n"(n) : "memory");
+    }
+    if (warp == kEpiWarps + 1) {
+        // ---- the MMAs ----
+        if (lane == 0) {
+            constexpr uint32_t kId128 = idesc_bf16_f32(kRows, kH), kId16 = idesc_bf16_f32(kRows, kN3);
+            for (int c = 0; c < kNChunks && ok; ++c) {
+                const int s = c % kXStages;
+                ok = mbar_wait_bounded(&S.xfull[s], (c / kXStages) & 1u);
+                if (!ok) break;
+                tc_fence_after_sync();
+                const uint32_t xa = smem_addr(S.Xc[s]), wa = smem_addr(S.W1[c]);
+#pragma unroll
+                for (int kk = 0; kk < kKc; kk += 16)
+                    tc_mma_bf16(tm, smem_desc_sw128(xa, kk * 2), smem_desc_sw128(wa, kk * 2), kId128, (c | kk) != 0);
+                tc_commit(&S.xempty[s]);
+            }
+            tc_commit(&S.d1);
+            auto layer = [&](uint64_t* ready, const bf16* a, const bf16* b, int brows, uint32_t col, uint32_t id,
+                             uint64_t* done) {
+                if (ok) ok = mbar_wait_bounded(ready, 0u);
+                if (!ok) return;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int kk = 0; kk < kH; kk += 16)
+                    tc_mma_bf16(tm + col, tile_desc(a, kRows, kk), tile_desc(b, brows, kk), id, kk != 0);
+                tc_commit(done);
+            };
+            layer(&S.h1, S.H, S.W2, kH, kH, kId128, &S.d2);
+            layer(&S.h2, S.H, S.W3, kN3, 2 * kH, kId16, &S.d3);
+            layer(&S.z2, S.Xc[0], S.W1[0], kH, 0, kId128, &S.d4);
+        }
+    } else if (warp < kEpiWarps) {
+        // ---- the element-wise parts: row 32 q + lane, columns 64 half .. + 63 ----
+        const int q = warp & 3, half = warp >> 2, row = 32 * q + lane;
+        const long long grow = row0 + row;
+        const bool store = grow < A.Mp, live = grow < A.M;
+        const uint32_t tl = tm + ((uint32_t)(32 * q) << 16);
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_bounded(bar, parity));
+            return ok;
+        };
+        // X transposed, while the MMAs take the same panels
+        for (int c = 0; c < kNChunks; ++c) {
+            const int s = c % kXStages;
+            if (!wait(&S.xfull[s], (c / kXStages) & 1u)) break;
+            if (store) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int ch = half * 4 + j;
+                    uint4 v = *reinterpret_cast<const uint4*>(S.Xc[s] + row * kKc + ((ch ^ (row & 7)) << 3));
+                    const bf16* e = reinterpret_cast<const bf16*>(&v);
+                    bf16* dst = A.XT + (long long)(c * kKc + ch * 8) * A.Mp + grow;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) dst[u * A.Mp] = e[u];
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.xempty[s]);
+        }
+        // an activation epilogue: bias, ReLU, BF16 into H, the mask of positive
+        // values, and (H1) the transposed output
+        auto activate = [&](uint32_t col, const float* bias, uint32_t (&mask)[2], bf16* outT) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int c0 = half * 64 + j * 32;
+                float v[32];
+                tmem_ld32(tl + col + (uint32_t)c0, v);
+                mask[j] = 0;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    uint4 w;
+                    bf16* o = reinterpret_cast<bf16*>(&w);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const float z = v[8 * h + u] + bias[c0 + 8 * h + u];
+                        mask[j] |= z > 0.f ? 1u << (8 * h + u) : 0u;
+                        o[u] = __float2bfloat16(fmaxf(z, 0.f));
+                        if (outT && store)
+                            outT[(long long)(c0 + 8 * h + u) * A.Mp + grow] = live ? o[u] : __float2bfloat16(0.f);
+                    }
+                    *reinterpret_cast<uint4*>(S.H + core_idx(row, c0 + 8 * h, kRows)) = w;
+                }
+            }
+            fence_async_shared();
+            tc_fence_before_sync();
+            __syncwarp();
+        };
+        uint32_t m1[2] = {0, 0}, m2[2] = {0, 0};
+        if (wait(&S.d1, 0u)) {
+            tc_fence_after_sync();
+            activate(0u, S.b1, m1, A.H1T);
+            if (lane == 0) mbar_arrive(&S.h1);
+            // W1 has been used: W2^T takes its place (ordered by the arrival on z2)
+            stage_weights(S.W1[0], A.W2T, kH, kH, kH, tid, kEpiWarps * 32);
+        }
+        if (wait(&S.d2, 0u)) {
+            tc_fence_after_sync();
+            activate(kH, S.b2, m2, nullptr);
+            if (lane == 0) mbar_arrive(&S.h2);
+        }
+        if (wait(&S.d3, 0u) && warp < 4) {
+            // loss and dY of this lane's row (Huber, delta 1; rows without a finite
+            // target are passed over)
+            tc_fence_after_sync();
+            float y[16], t[kOut] = {0.f, 0.f, 0.f, 0.f}, acc = 0.f;
+            tmem_ld16(tl + 2 * kH, y);
+            bool valid = false;
+            if (live) {
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) t[j] = A.T[grow * kOut + j];
+                valid = isfinite(t[kOut - 1]);
+            }
+            float d[kOut];
+#pragma unroll
+            for (int j = 0; j < kOut; ++j) {
+                const float r = valid ? y[j] + S.b3[j] - t[j] : 0.f;
+                const float a = fabsf(r);
+                acc += a <= 1.f ? 0.5f * r * r : a - 0.5f;
+                d[j] = live ? (a <= 1.f ? r : copysignf(1.f, r)) * A.inv_count : 0.f;
+                S.dY[row][j] = d[j];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) d[j] += __shfl_xor_sync(0xffffffffu, d[j], o);
+            }
+            if (lane == 0) {
+                atomicAdd(A.loss, acc * A.inv_count);
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) atomicAdd(&S.gb3[j], d[j]);
+            }
+        }
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
+        if (ok) {
+            float dy[kOut];
+#pragma unroll
+            for (int j = 0; j < kOut; ++j) dy[j] = S.dY[row][j];
+            bf16* dz = &S.Xc[0][0];
+#pragma unroll 1
+            for (int j2 = 0; j2 < 2; ++j2) {
+                const int c0 = half * 64 + j2 * 32;
+                const uint32_t mk = j2 ? m2[1] : m2[0];
+                float h[32], v[32];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(S.H + core_idx(row, c0 + 8 * k, kRows));
+                    const bf16* e = reinterpret_cast<const bf16*>(&w);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) h[8 * k + u] = __bfloat162float(e[u]);
+                }
+                // dW3 = dY^T H2
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) v[c] = dy[j] * h[c];
+                    const float s = warp_column_sum(v);
+                    atomicAdd(&S.gW3[j * kH + c0 + lane], s);
+                }
+                // dZ2 = (dY W3) * [Z2 > 0]
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    uint4 w;
+                    bf16* o = reinterpret_cast<bf16*>(&w);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int c = c0 + 8 * k + u;
+                        float d = 0.f;
+#pragma unroll
+                        for (int j = 0; j < kOut; ++j) d = fmaf(dy[j], S.W3f[j * kH + c], d);
+                        o[u] = __float2bfloat16((mk >> (8 * k + u)) & 1u ? d : 0.f);
+                        v[8 * k + u] = __bfloat162float(o[u]);
+                        if (store) A.dZ2T[(long long)c * A.Mp + grow] = o[u];
+                    }
+                    *reinterpret_cast<uint4*>(dz + core_idx(row, c0 + 8 * k, kRows)) = w;
+                }
+                atomicAdd(&S.gb2[c0 + lane], warp_column_sum(v));
+            }
+            fence_async_shared();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.z2);
+        }
+        if (wait(&S.d4, 0u)) {
+            // dZ1 = dH1 * [Z1 > 0]
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int j = 0; j < 2; ++j) {
+                const int c0 = half * 64 + j * 32;
+                const uint32_t mk = j ? m1[1] : m1[0];
+                float v[32];
+                tmem_ld32(tl + (uint32_t)c0, v);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const bf16 o = __float2bfloat16((mk >> c) & 1u ? v[c] : 0.f);
+                    v[c] = __bfloat162float(o);
+                    if (store) A.dZ1T[(long long)(c0 + c) * A.Mp + grow] = o;
+                }
+                atomicAdd(&S.gb1[c0 + lane], warp_column_sum(v));
+            }
+            tc_fence_before_sync();
+        }
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
+        if (ok) {
+            for (int k = tid; k < kOut * kH; k += kEpiWarps * 32) atomicAdd(&A.gW3[k], S.gW3[k]);
+            if (tid < kH) atomicAdd(&A.gb1[tid], S.gb1[tid]);
+            else atomicAdd(&A.gb2[tid - kH], S.gb2[tid - kH]);
+            if (tid < kOut) atomicAdd(&A.gb3[tid], S.gb3[tid]);
+        }
+    }
+    if (!ok && lane == 0) atomicOr(A.flags, kFlagTimeout);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+}
+
+cudaError_t launch_train_rows(const TrainArgs& A, const bf16* X, cudaStream_t s)
+{
+    CUtensorMap xmap;
+    if (!encode_bf16_2d(&xmap, X, kInPad, (unsigned long long)A.M, kInPad * 2, kKc, kRows, true))
+        return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kTcSmemBytes);
+    if (e != cudaSuccess) return e;
+    k_train_rows<<<(unsigned)((A.M + kRows - 1) / kRows), kTrainThreads, kTcSmemBytes, s>>>(A, xmap);
+    return cudaGetLastError();
 }
 
 // --------------------------------------------------------------------------
@@ -1002,14 +1268,14 @@ struct gamma_model_s {
     bf16 *W1h = nullptr, *W2h = nullptr, *W2Th = nullptr, *W3h = nullptr;
     long long step = 0;
     unsigned long long seed = 0;
-    // training workspace
-    long long wsM = 0;
-    float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *dY = nullptr, *dH1 = nullptr, *loss = nullptr;
-    bf16 *H1h = nullptr, *H2h = nullptr, *dZ2h = nullptr, *dZ1h = nullptr;
-    // batch-contiguous (transposed) operands of the weight-gradient GEMMs,
-    // row stride wsMp = wsM rounded up to 8 (16-byte rows for TMA)
+    // training workspace: X, H1, dZ1 and dZ2 of a batch transposed (the
+    // operands of the weight-gradient product), row stride wsMp = wsM rounded
+    // up to 8 (16-byte rows for TMA)
+    long long wsM = 0, wsMp = 0;
     bf16 *XT = nullptr, *H1T = nullptr, *dZ1T = nullptr, *dZ2T = nullptr;
-    long long wsMp = 0;
+    gk::WgradMaps maps{};         // their tensor maps for batches of mapsM rows
+    long long mapsM = 0;
+    float* loss = nullptr;        // behind the gradients (gr), and dflags behind it: one reset, one read
     unsigned* dflags = nullptr;   // error flags of the training kernels
     unsigned* hflags = nullptr;   // ... of gamma_model_infer: page-locked, mapped host memory
     unsigned* hflags_dev = nullptr;   // its device address
@@ -1037,43 +1303,29 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? GAMMA_OK : (e == cudaErro
 
 void free_ws(gamma_model_s* m)
 {
-    cudaFree(m->Z1); cudaFree(m->Z2); cudaFree(m->Y); cudaFree(m->dY); cudaFree(m->dH1);
-    cudaFree(m->loss); cudaFree(m->H1h); cudaFree(m->H2h); cudaFree(m->dZ2h); cudaFree(m->dZ1h);
-    cudaFree(m->XT); cudaFree(m->H1T); cudaFree(m->dZ1T); cudaFree(m->dZ2T);
-    m->Z1 = m->Z2 = m->Y = m->dY = m->dH1 = m->loss = nullptr;
-    m->H1h = m->H2h = m->dZ2h = m->dZ1h = nullptr;
+    cudaFree(m->XT);               // one allocation
     m->XT = m->H1T = m->dZ1T = m->dZ2T = nullptr;
-    m->wsM = m->wsMp = 0;
+    m->wsM = m->wsMp = m->mapsM = 0;
 }
 
 int ensure_ws(gamma_model_s* m, long long M)
 {
-    if (M <= m->wsM) return GAMMA_OK;
-    free_ws(m);
-    MCK(cudaMalloc(&m->Z1, sizeof(float) * M * gk::kH));
-    MCK(cudaMalloc(&m->Z2, sizeof(float) * M * gk::kH));
-    MCK(cudaMalloc(&m->Y, sizeof(float) * M * gk::kOutPad));
-    MCK(cudaMalloc(&m->dY, sizeof(float) * M * gk::kOut));
-    MCK(cudaMalloc(&m->dH1, sizeof(float) * M * gk::kH));
-    MCK(cudaMalloc(&m->loss, sizeof(float)));
-    MCK(cudaMalloc(&m->H1h, sizeof(bf16) * M * gk::kH));
-    MCK(cudaMalloc(&m->H2h, sizeof(bf16) * M * gk::kH));
-    MCK(cudaMalloc(&m->dZ2h, sizeof(bf16) * M * gk::kH));
-    MCK(cudaMalloc(&m->dZ1h, sizeof(bf16) * M * gk::kH));
     const long long Mp = (M + 7) / 8 * 8;
-    MCK(cudaMalloc(&m->XT, sizeof(bf16) * Mp * gk::kInPad));
-    MCK(cudaMalloc(&m->H1T, sizeof(bf16) * Mp * gk::kH));
-    MCK(cudaMalloc(&m->dZ1T, sizeof(bf16) * Mp * gk::kH));
-    MCK(cudaMalloc(&m->dZ2T, sizeof(bf16) * Mp * gk::kH));
-    m->wsM = M;
-    m->wsMp = Mp;
+    if (M > m->wsM) {
+        free_ws(m);
+        MCK(cudaMalloc(&m->XT, sizeof(bf16) * (size_t)Mp * (gk::kInPad + 3 * gk::kH)));
+        m->H1T = m->XT + Mp * gk::kInPad;
+        m->dZ1T = m->H1T + Mp * gk::kH;
+        m->dZ2T = m->dZ1T + Mp * gk::kH;
+        m->wsM = M;
+        m->wsMp = Mp;
+    }
+    if (m->mapsM != M) {
+        m->mapsM = 0;
+        if (!gk::encode_wgrad_maps(&m->maps, m->dZ1T, m->XT, m->dZ2T, m->H1T, M, m->wsMp)) return GAMMA_ERR_CUDA;
+        m->mapsM = M;
+    }
     return GAMMA_OK;
-}
-
-int grid_for_n(long long n, int threads = 256)
-{
-    long long b = (n + threads - 1) / threads;
-    return (int)std::max<long long>(1, std::min<long long>(b, (long long)gk::device_sm_count() * 16));
 }
 
 // Host-side parameter initialisation: He-normal weights from a splitmix64 /
@@ -1109,59 +1361,56 @@ std::vector<unsigned char> param_mask()
     return k;
 }
 
+gk::WeightCopies weight_copies(const gamma_model_s* m)
+{
+    return gk::WeightCopies{m->W1h, m->W2h, m->W2Th, m->W3h, (int)kOffW2, (int)kOffW3};
+}
+
 int refresh_bf16(gamma_model_s* m, cudaStream_t s)
 {
-    gk::k_cast_weights<<<64, 256, 0, s>>>(m->p + kOffW1, m->p + kOffW2, m->p + kOffW3, m->W1h,
-                                          m->W2h, m->W2Th, m->W3h);
+    gk::k_cast_weights<<<(int)(kNParams + 255) / 256, 256, 0, s>>>((int)kNParams, m->p, weight_copies(m));
     return cuda_rc(cudaGetLastError());
 }
 
-// Forward pass of a minibatch through the training kernels (activations
-// kept): the three layers as tensor-core GEMMs (tcgen05, TMEM accumulators,
-// TMA operand loads), bias and ReLU in separate element-wise passes.
-int forward_train(gamma_model_s* m, const bf16* X, long long M, cudaStream_t s)
+// Loss and gradients of a minibatch into m->gr (zeroed first, with the loss and
+// the flags behind it): the rows' passes in one kernel, then both weight
+// gradients in one product with the batch as K, split over several blocks per
+// tile that add into them.
+int backward_train(gamma_model_s* m, const bf16* X, const float* T, long long M, cudaStream_t s)
 {
-    using namespace gk;
-    MCK(launch_gemm_tc(X, M, kInPad, m->W1h, kH, kInPad, kInPad, m->Z1, kH, 1, m->dflags, s));
-    k_bias_act<<<grid_for_n(M * kH), 256, 0, s>>>(M, kH, m->Z1, m->p + kOffB1, m->H1h, kH, 1);
-    MCK(launch_gemm_tc(m->H1h, M, kH, m->W2h, kH, kH, kH, m->Z2, kH, 1, m->dflags, s));
-    k_bias_act<<<grid_for_n(M * kH), 256, 0, s>>>(M, kH, m->Z2, m->p + kOffB2, m->H2h, kH, 1);
-    MCK(launch_gemm_tc(m->H2h, M, kH, m->W3h, kOutPad, kH, kH, m->Y, kOutPad, 1, m->dflags, s));
-    k_bias_act<<<grid_for_n(M * kOutPad), 256, 0, s>>>(M, kOutPad, m->Y, m->p + kOffB3, nullptr, 0, 0);
-    return cuda_rc(cudaGetLastError());
+    MCK(cudaMemsetAsync(m->gr, 0, sizeof(float) * kNParams + 2 * sizeof(unsigned), s));
+    gk::TrainArgs A{};
+    gk::model_weights(m, &A.W);
+    A.W2T = m->W2Th;
+    A.W3f = m->p + kOffW3;
+    A.T = T;
+    A.M = M;
+    A.Mp = m->wsMp;
+    A.inv_count = 1.f / (float)M;
+    A.XT = m->XT;
+    A.H1T = m->H1T;
+    A.dZ1T = m->dZ1T;
+    A.dZ2T = m->dZ2T;
+    A.gb1 = m->gr + kOffB1;
+    A.gb2 = m->gr + kOffB2;
+    A.gW3 = m->gr + kOffW3;
+    A.gb3 = m->gr + kOffB3;
+    A.loss = m->loss;
+    A.flags = m->dflags;
+    MCK(gk::launch_train_rows(A, X, s));
+    MCK(gk::launch_wgrad(m->maps, M, m->gr + kOffW1, m->gr + kOffW2, m->dflags, s));
+    return GAMMA_OK;
 }
 
-// Loss and gradients of a minibatch into m->gr (zeroed first).  The weight
-// gradients sum over the batch, so their GEMMs take the batch as K: the
-// operands are first transposed to batch-contiguous rows, and the K range is
-// split over several blocks per tile that add into the gradient.
-int backward_train(gamma_model_s* m, const bf16* X, const float* T, long long M, long long count,
-                   cudaStream_t s)
+// Loss (optional) of the last backward pass: synchronises.
+int read_loss(gamma_model_s* m, float* loss_out, cudaStream_t s)
 {
-    using namespace gk;
-    MCK(cudaMemsetAsync(m->gr, 0, sizeof(float) * kNParams, s));
-    MCK(cudaMemsetAsync(m->loss, 0, sizeof(float), s));
-    const float invc = count > 0 ? 1.f / (float)count : 0.f;
-    const long long Mp = (M + 7) / 8 * 8;
-    const int splits = (int)std::max<long long>(1, std::min<long long>(32, M / 512));
-    k_huber<<<grid_for_n(M), 256, 0, s>>>(M, m->Y, T, m->dY, m->loss, invc);
-    k_out_back<<<grid_for_n(M * kH, 256), 256, 0, s>>>(M, m->dY, m->p + kOffW3, m->Z2, m->H2h,
-                                                         m->dZ2h, m->gr + kOffW3, m->gr + kOffB3);
-    // dW2 = dZ2^T H1 (K = batch), db2 = colsum dZ2
-    MCK(launch_transpose_bf16(m->dZ2h, M, kH, kH, m->dZ2T, Mp, s));
-    MCK(launch_transpose_bf16(m->H1h, M, kH, kH, m->H1T, Mp, s));
-    MCK(launch_gemm_tc(m->dZ2T, kH, Mp, m->H1T, kH, Mp, M, m->gr + kOffW2, kH, splits, m->dflags, s));
-    k_colsum<<<dim3(256, (kH + 127) / 128), 128, 0, s>>>(M, kH, m->dZ2h, m->gr + kOffB2);
-    // dH1 = dZ2 W2 (B[n][k] = W2^T[n][k] = W2[k][n]), dZ1 = dH1 [Z1 > 0]
-    MCK(launch_gemm_tc(m->dZ2h, M, kH, m->W2Th, kH, kH, kH, m->dH1, kH, 1, m->dflags, s));
-    k_relu_back<<<grid_for_n(M * kH), 256, 0, s>>>(M, kH, m->dH1, m->Z1, m->dZ1h, nullptr);
-    k_colsum<<<dim3(256, (kH + 127) / 128), 128, 0, s>>>(M, kH, m->dZ1h, m->gr + kOffB1);
-    // dW1 = dZ1^T X (K = batch)
-    MCK(launch_transpose_bf16(m->dZ1h, M, kH, kH, m->dZ1T, Mp, s));
-    MCK(launch_transpose_bf16(X, M, kInPad, kInPad, m->XT, Mp, s));
-    MCK(launch_gemm_tc(m->dZ1T, kH, Mp, m->XT, kInPad, Mp, M, m->gr + kOffW1, kInPad, splits,
-                       m->dflags, s));
-    return cuda_rc(cudaGetLastError());
+    if (!loss_out) return GAMMA_OK;
+    unsigned w[2];                                 // loss, flags
+    MCK(cudaMemcpyAsync(w, m->loss, sizeof(w), cudaMemcpyDeviceToHost, s));
+    MCK(cudaStreamSynchronize(s));
+    std::memcpy(loss_out, &w[0], sizeof(float));
+    return (w[1] & gk::kFlagTimeout) ? GAMMA_ERR_TIMEOUT : GAMMA_OK;
 }
 
 }  // namespace
@@ -1194,7 +1443,10 @@ int gamma_model_create(gamma_model* out, uint64_t seed)
     if (cudaGetDevice(&m->device) != cudaSuccess) return fail(GAMMA_ERR_CUDA);
     int rc;
     if ((rc = cuda_rc(cudaMalloc(&m->p, sizeof(float) * kNParams)))) return fail(rc);
-    if ((rc = cuda_rc(cudaMalloc(&m->gr, sizeof(float) * kNParams)))) return fail(rc);
+    if ((rc = cuda_rc(cudaMalloc(&m->gr, sizeof(float) * kNParams + 2 * sizeof(unsigned))))) return fail(rc);
+    m->loss = m->gr + kNParams;
+    m->dflags = reinterpret_cast<unsigned*>(m->loss + 1);
+    if ((rc = cuda_rc(cudaMemset(m->gr, 0, sizeof(float) * kNParams + 2 * sizeof(unsigned))))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->m1, sizeof(float) * kNParams)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->m2, sizeof(float) * kNParams)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->mask, kNParams)))) return fail(rc);
@@ -1202,8 +1454,6 @@ int gamma_model_create(gamma_model* out, uint64_t seed)
     if ((rc = cuda_rc(cudaMalloc(&m->W2h, sizeof(bf16) * gk::kH * gk::kH)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->W2Th, sizeof(bf16) * gk::kH * gk::kH)))) return fail(rc);
     if ((rc = cuda_rc(cudaMalloc(&m->W3h, sizeof(bf16) * gk::kOutPad * gk::kH)))) return fail(rc);
-    if ((rc = cuda_rc(cudaMalloc(&m->dflags, sizeof(unsigned))))) return fail(rc);
-    if ((rc = cuda_rc(cudaMemset(m->dflags, 0, sizeof(unsigned))))) return fail(rc);
     if ((rc = cuda_rc(cudaHostAlloc(&m->hflags, sizeof(unsigned), cudaHostAllocMapped)))) return fail(rc);
     if ((rc = cuda_rc(cudaHostGetDevicePointer((void**)&m->hflags_dev, m->hflags, 0)))) return fail(rc);
     std::vector<float> h;
@@ -1225,7 +1475,6 @@ void gamma_model_destroy(gamma_model m)
     if (!m) return;
     cudaFree(m->p); cudaFree(m->gr); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->mask);
     cudaFree(m->W1h); cudaFree(m->W2h); cudaFree(m->W2Th); cudaFree(m->W3h);
-    cudaFree(m->dflags);
     if (m->hflags) cudaFreeHost(m->hflags);
     free_ws(m);
     delete m;
@@ -1257,11 +1506,9 @@ int gamma_model_forward(gamma_model m, const void* X_bf16_dev, int64_t M, float*
     if (!m || !X_bf16_dev || !Y_dev || M <= 0) return GAMMA_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (reinterpret_cast<uintptr_t>(X_bf16_dev) % 16 != 0) return GAMMA_ERR_INVALID_ARG;
-    if (int rc = ensure_ws(m, M)) return rc;
-    MCK(cudaMemsetAsync(m->dflags, 0, sizeof(unsigned), s));
-    if (int rc = forward_train(m, (const bf16*)X_bf16_dev, M, s)) return rc;
-    MCK(cudaMemcpy2DAsync(Y_dev, sizeof(float) * gk::kOut, m->Y, sizeof(float) * gk::kOutPad,
-                          sizeof(float) * gk::kOut, (size_t)M, cudaMemcpyDeviceToDevice, s));
+    gk::MlpWeights W;
+    gk::model_weights(m, &W);
+    MCK(gk::launch_mlp_rows(W, (const bf16*)X_bf16_dev, M, nullptr, Y_dev, m->dflags, 0, s));
     return GAMMA_OK;
 }
 
@@ -1289,17 +1536,8 @@ int gamma_model_backward(gamma_model m, const void* X_bf16_dev, const float* T_d
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (reinterpret_cast<uintptr_t>(X_bf16_dev) % 16 != 0) return GAMMA_ERR_INVALID_ARG;
     if (int rc = ensure_ws(m, M)) return rc;
-    MCK(cudaMemsetAsync(m->dflags, 0, sizeof(unsigned), s));
-    if (int rc = forward_train(m, (const bf16*)X_bf16_dev, M, s)) return rc;
-    if (int rc = backward_train(m, (const bf16*)X_bf16_dev, T_dev, M, M, s)) return rc;
-    if (loss_out) {
-        unsigned flags = 0;
-        MCK(cudaMemcpyAsync(loss_out, m->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
-        MCK(cudaMemcpyAsync(&flags, m->dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-        MCK(cudaStreamSynchronize(s));
-        if (flags & gk::kFlagTimeout) return GAMMA_ERR_TIMEOUT;
-    }
-    return GAMMA_OK;
+    if (int rc = backward_train(m, (const bf16*)X_bf16_dev, T_dev, M, s)) return rc;
+    return read_loss(m, loss_out, s);
 }
 
 int gamma_model_train_step(gamma_model m, const void* X_bf16_dev, const float* T_dev, int64_t M,
@@ -1311,18 +1549,10 @@ int gamma_model_train_step(gamma_model m, const void* X_bf16_dev, const float* T
     m->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)m->step), c2 = 1.f - std::pow(b2, (float)m->step);
-    gk::k_adam<<<grid_for_n(kNParams), 256, 0, s>>>(kNParams, m->p, m->gr, m->m1, m->m2, m->mask, lr,
-                                                   b1, b2, 1e-8f, c1, c2);
+    gk::k_adam<<<(int)(kNParams + 255) / 256, 256, 0, s>>>((int)kNParams, m->p, m->gr, m->m1, m->m2, m->mask,
+                                                           weight_copies(m), lr, b1, b2, 1e-8f, c1, c2);
     MCK(cudaGetLastError());
-    if (int rc = refresh_bf16(m, s)) return rc;
-    if (loss_out) {
-        unsigned flags = 0;
-        MCK(cudaMemcpyAsync(loss_out, m->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
-        MCK(cudaMemcpyAsync(&flags, m->dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-        MCK(cudaStreamSynchronize(s));
-        if (flags & gk::kFlagTimeout) return GAMMA_ERR_TIMEOUT;
-    }
-    return GAMMA_OK;
+    return read_loss(m, loss_out, s);
 }
 
 // File format: 8-byte magic "GAMMAMLP", int32 version 1, int32 kIn, kInPad,
