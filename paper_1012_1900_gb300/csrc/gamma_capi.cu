@@ -127,6 +127,7 @@ struct gamma_ctx {
     unsigned* plane_raw = nullptr;    // ... the cells of the plane seeds (tail_cap entries each, allocated
                                       //     with fix_list)
     unsigned* plane_sorted = nullptr;
+    float2* range = nullptr;          // ... dose range of every cell (written when the queue is worth it)
     int group_bucket = 9;             // ... queued voxels of this cost bucket and above walk 4 lanes each
                                       //     (< 0: the walk chooses the parts from the queue)
     int group_auto_pct = 100;         // ... with this slack (percent)
@@ -278,7 +279,7 @@ int build_table(gamma_ctx* h)
         const int c[3] = {all[i].x, all[i].y, all[i].z};
         for (int a = 0; a < nd; ++a) margin = std::max(margin, std::max(-c[a], c[a] + 1));
         const int64_t lin = c[0] + (int64_t)c[1] * h->nx + (int64_t)c[2] * h->nx * h->ny;
-        walk[i] = gk::WalkEntry{h->table[i].key, (int)lin, h->table[i].off, margin};
+        walk[i] = gk::WalkEntry{h->table[i].key * h->table[i].key, (int)lin, h->table[i].off, margin};
     }
     if (keep) std::memcpy((char*)walk.data() + wbytes, h->table.data(), keep * sizeof(TableEntry));
     cudaFree(h->walk_dev);
@@ -346,6 +347,7 @@ Problem make_problem(const gamma_ctx* h, float* out)
     if (h->walk == 3) {
         P.plane_raw = h->plane_raw;
         P.plane_sorted = h->plane_sorted;
+        P.range = h->range;
     }
     P.cq_group_bucket = h->group_bucket;
     P.cq_group8_bucket = h->group8_bucket;
@@ -402,6 +404,7 @@ void free_ctx(gamma_ctx* h)
     cudaFree(h->row_bkt);
     cudaFree(h->row_sorted);
     cudaFree(h->fix_list);
+    cudaFree(h->range);
     cudaFree(h->seed_list);
     cudaFree(h->seed_X);
     cudaFree(h->seed_Y);
@@ -729,6 +732,11 @@ int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev,
     if ((e = cudaMalloc(&h->fix_list, 3 * sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
     h->plane_raw = h->fix_list + nvox;
     h->plane_sorted = h->plane_raw + nvox;
+    // only a gain: without room for it the walk takes the ranges from the doses
+    if (cudaMalloc(&h->range, sizeof(float2) * nvox) != cudaSuccess) {
+        cudaGetLastError();
+        h->range = nullptr;
+    }
     {
         Problem P0 = make_problem(h, nullptr);
         const int tiles = gk::block_tiles(P0);

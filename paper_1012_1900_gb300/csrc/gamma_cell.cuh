@@ -96,17 +96,35 @@ __device__ __noinline__ float cell_recheck(const Problem& P, uint32_t ok, int cx
     return cell_redo_f64<N>(P.ev, p, sy, sz, ok, cx, cy, cz, drd, invd, P.mtd, &P.ctr->fp64_cells);
 }
 
-// Every face of the cell with lower corner (x+cx, y+cy, z+cz) as squared
-// gamma, with the FP64 redo when a face's Gram matrix is near singular.  q
-// holds (D_e - dr) * inv of the cell's vertices.  Out of line: each kernel
-// keeps one copy, and the callers keep their own registers few.
+// Takes the voxel itself out of the vertices of a cell whose box contains it
+// (lower corner at 0 or -1 on every axis; q: relative doses), so that only the
+// cell's faces off the voxel remain: those through it have their value from the
+// reduced form before any table walk, and the general one could differ from it
+// in the last bit.  Other cells are left as they are.
 template <int N>
+__device__ __forceinline__ void drop_own_vertex(float (&q)[8], int cx, int cy, int cz)
+{
+    if ((unsigned)(cx + 1) < 2u && (unsigned)(cy + 1) < 2u && (N == 2 || (unsigned)(cz + 1) < 2u)) {
+        const int self = (cx & 1) | ((cy & 1) << 1) | (N == 3 ? (cz & 1) << 2 : 0);
+#pragma unroll
+        for (int u = 0; u < (1 << N); ++u)
+            if (u == self) q[u] = kNaN;
+    }
+}
+
+// Every face of the cell with lower corner (x+cx, y+cy, z+cz) as squared
+// gamma (WALK: of a cell whose box contains the voxel only those off the
+// voxel), with the FP64 redo of the cell when a face's Gram matrix is near
+// singular.  q holds (D_e - dr) * inv of the cell's vertices.  Out of line:
+// each kernel keeps one copy, and the callers keep their own registers few.
+template <int N, bool WALK>
 __device__ __noinline__ float cell_all_faces(const Problem& P, float q0, float q1, float q2,
                                              float q3, float q4, float q5, float q6, float q7,
                                              uint32_t ok, int cx, int cy, int cz, long long p,
                                              float dr, float dnorm)
 {
-    const float q[8] = {q0, q1, q2, q3, q4, q5, q6, q7};
+    float q[8] = {q0, q1, q2, q3, q4, q5, q6, q7};
+    if (WALK) drop_own_vertex<N>(q, cx, cy, cz);
     CellGeom<float> g;
     cell_geom<N, float>(cx, cy, cz, P.mt, g);
     bool ill = false;

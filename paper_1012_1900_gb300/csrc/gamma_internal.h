@@ -56,12 +56,12 @@ struct TableEntry {
 // one needs for its cell to lie in the grid with every vertex.  Padded with
 // kWalkPad entries of infinite key, which no walk reaches.
 struct alignas(16) WalkEntry {
-    float key;
+    float key2;              // the key's square (rounded as the product of the rounded key)
     int lin;
     uint32_t off;
     int margin;
 };
-constexpr int kWalkPad = 128;
+constexpr int kWalkPad = 256;
 
 __host__ __device__ inline int unpack10(uint32_t v, int shift)
 {
@@ -212,6 +212,7 @@ struct Problem {
     // evaluated, in discovery and in cost order (null: the other walks)
     unsigned* plane_raw;
     unsigned* plane_sorted;
+    float2* range;               // smallest and largest dose of each cell's vertices (null: not kept)
 };
 
 // Readiness of the evaluation dose by z slab, for a shell launch that starts

@@ -760,6 +760,29 @@ __global__ void __launch_bounds__(256, MINB)
 // of the bucket.
 __device__ __forceinline__ float bucket_cells(int b) { return b > 0 ? exp2f((2 * b - 1) * 0.25f) : 0.5f; }
 
+// The estimated cells of a whole queue, lane b of a full warp holding the count
+// of bucket b (every caller gets the same bits).
+__device__ __forceinline__ float queue_cells(unsigned count)
+{
+    float c = (float)count * bucket_cells(threadIdx.x & 31);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
+    return c;
+}
+
+// Whether the walk of a queue with this many estimated cells takes the cells'
+// dose ranges from an array, which the ordering kernel then writes: one read
+// per tested cell instead of eight and their minimum and maximum, for a pass
+// over the grid that reads 4 and writes 8 bytes per voxel.  The line lies where
+// the pass (2.8 us per million voxels) meets what it saves (1.3 to 2.2 us per
+// million cells), with a margin: 320x320x240 voxels, 395 M cells: 68 us for
+// 520 us; 1.05 G cells: 2.35 ms.
+constexpr float kRangeCells = 3.f;                 // tested cells per grid voxel
+__device__ __forceinline__ bool wants_range(const Problem& P, float cells)
+{
+    return P.range && P.plane_raw && cells > kRangeCells * (float)P.nvox;
+}
+
 // The queue's parts chosen from the queue itself (option group_bucket < 0):
 // a queued voxel of cost bucket b is estimated to key c(b) = 2^((2b - 1) / 4)
 // table cells (the middle of the bucket), the walk's W = sum of c over the
@@ -797,6 +820,7 @@ __device__ __forceinline__ void auto_part_buckets(unsigned count, unsigned lanes
 __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem P)
 {
     __shared__ unsigned start[kNumBuckets], cnt[kNumBuckets], base[kNumBuckets];
+    __shared__ float s_cells;
     if (threadIdx.x < kNumBuckets) {
         const unsigned own = P.ctr->hist[threadIdx.x];
         unsigned sum = own;                    // of this bucket and the costlier ones
@@ -806,7 +830,10 @@ __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem
             if (threadIdx.x + o < kNumBuckets) sum += u;
         }
         start[threadIdx.x] = sum - own;
+        const float cells = queue_cells(own);
+        if (threadIdx.x == 0) s_cells = cells;
     }
+    __syncthreads();
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     for (unsigned c0 = blockIdx.x * blockDim.x; c0 < total; c0 += gridDim.x * blockDim.x) {
         if (threadIdx.x < kNumBuckets) cnt[threadIdx.x] = 0;
@@ -827,6 +854,34 @@ __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem
             if (P.plane_raw) P.plane_sorted[base[b] + rank] = P.plane_raw[i];
         }
         __syncthreads();
+    }
+    if (!wants_range(P, s_cells)) return;
+    // the dose range of every cell whose vertices all lie in the grid: a warp
+    // takes a segment of 31 cells along x and marches along z, each node read once
+    const int lane = threadIdx.x & 31;
+    const int nx = P.nx, ny = P.ny, nz = P.nz, sz = nx * ny;
+    const int segs = (nx + 30) / 31;
+    constexpr int kRun = 16;                       // cells along z per turn
+    const int runs = P.ndim == 3 ? (nz + kRun - 1) / kRun : 1;
+    const long long work = (long long)segs * ny * runs;
+    for (long long wk = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); wk < work; wk += (long long)gridDim.x * 8) {
+        const int sg = (int)(wk % segs), y = (int)(wk / segs % ny), rn = (int)(wk / segs / ny);
+        const int x = sg * 31 + lane, z0 = rn * kRun;
+        if (y + 1 >= ny) continue;                 // warp-uniform
+        const bool inx = x < nx;
+        float lo = 0.f, hi = 0.f;                  // of the nodes (x, x + 1) x (y, y + 1) one plane below
+        for (int z = z0; z <= (P.ndim == 3 ? min(z0 + kRun, nz - 1) : 0); ++z) {
+            const float* q = P.ev + ((long long)z * sz + (long long)y * nx + x);
+            const float a = inx ? __ldg(q) : 0.f, c = inx ? __ldg(q + nx) : 0.f;
+            float l = fminf(a, c), h = fmaxf(a, c);
+            l = fminf(l, __shfl_down_sync(kFull, l, 1));
+            h = fmaxf(h, __shfl_down_sync(kFull, h, 1));
+            if (lane < 31 && x + 1 < nx && (P.ndim == 2 || z > z0))
+                P.range[(long long)(P.ndim == 3 ? z - 1 : 0) * sz + (long long)y * nx + x] =
+                    P.ndim == 3 ? make_float2(fminf(l, lo), fmaxf(h, hi)) : make_float2(l, h);
+            lo = l;
+            hi = h;
+        }
     }
 }
 
@@ -1069,7 +1124,7 @@ __device__ __forceinline__ float visit_cell(const Problem& P, int x, int y, int 
         return best;
     }
     if (P.stats) ++st.visited;
-    const float cb = cell_all_faces<N>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy,
+    const float cb = cell_all_faces<N, true>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy,
                                        cz, p, dr, dnorm);
     return fminf(best, cb);
 }
@@ -1313,43 +1368,17 @@ __global__ void __launch_bounds__(256)
             }
             if (same) break;                                  // e holds this cell's doses
         }
-        // of the cells around the voxel itself only the faces off the voxel
-        // (its vertex taken out), and the walk looks at them again: the faces
-        // through the voxel have their value from the reduced form, from
-        // which the general one could differ in the last bit
-        bool own = true;
-        int self = 0;                                         // the voxel as a vertex of the cell
-#pragma unroll
-        for (int a = 0; a < N; ++a) {
-            own = own && (unsigned)(c[a] + 1) < 2u;
-            self |= c[a] < 0 ? 1 << a : 0;
-        }
         float q[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            q[u] = u < (1 << N) && !(own && u == self) ? rel_dose(e[u], dr, inv) : kNaN;
+        for (int u = 0; u < 8; ++u) q[u] = u < (1 << N) ? rel_dose(e[u], dr, inv) : kNaN;
+        drop_own_vertex<N>(q, c[0], c[1], c[2]);
         CellGeom<float> g;
         cell_geom<N, float>(c[0], c[1], c[2], P.mt, g);
         bool ill = false;
         const float cb = cell_min_d2<N, float>(q, g, P.mt, ill_dmax(P), kInf, ill);
-        if (own) {
-            // the walk redoes the whole cell in FP64 if any of its faces is
-            // near singular: not a seed unless the range of its doses rules
-            // that out (D <= 1 + 3 range^2 / min hn2)
-            float qlo = e[0], qhi = e[0];
-#pragma unroll
-            for (int u = 1; u < (1 << N); ++u) {
-                qlo = fminf(qlo, e[u]);
-                qhi = fmaxf(qhi, e[u]);
-            }
-            const float rg = (qhi - qlo) * inv;
-            const float kmax = fmaxf(fmaxf(kap[0], kap[1]), N == 3 ? kap[2] : 0.f);
-            ill = fmaf(3.f * kmax * rg, rg, 1.f) > ill_dmax(P);
-        } else if (ill) {
-            ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, P.mt.kappa, P.tau);
-        }
+        if (ill) ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, P.mt.kappa, P.tau);
         // a near-singular cell is left to the walk (and its FP64 redo)
-        P.plane_raw[i] = ill || own ? kNoSeed : pack10(c[0], c[1], c[2]);
+        P.plane_raw[i] = ill ? kNoSeed : pack10(c[0], c[1], c[2]);
         if (!ill && cb < best) {
             P.out[v] = cb + 0.f;                              // -0 -> +0
             const int was = P.tail_bucket[i], now = cost_bucket_of(P.bucket_key, sqrtf(fmaxf(cb, 0.f)));
@@ -1371,7 +1400,7 @@ __global__ void __launch_bounds__(256)
 
 // A warp takes a batch of up to 32 queued voxels of about the same cost, sets
 // them up one per lane, and walks the table for 32 / g of them at a time, g
-// lanes each (a round): lane l of a voxel looks at entry t + l, and the round
+// lanes each (a round): lane l of a voxel looks at entries t + l and t + g + l, and the round
 // ends when no lane's key is below its voxel's bound (the exact stop of A1
 // step 4b-ii).  A cell below the bound is tested in three tiers, each of which
 // leaves a fraction of the cells, so each runs with a full warp on the cells
@@ -1398,10 +1427,11 @@ __global__ void __launch_bounds__(256)
 // three tiers; the dose loads hit L1 at 92 %.  Before, one walker per lane or
 // group collected the cells past the dose gap alone and evaluated all of them
 // (21.8 per queued voxel of a 320x320x240 map at 3 %/3 mm, 36.5 at 1 %/1 mm
-// local; now 3.9 and 8.5): 10.5 ms there and 23.6 ms, now 3.6 ms and 10.2 ms
-// (twelve warps in each of two blocks per SM); 420 us and 180 us on a
-// 200x200x150 map at 2 %/2 mm.
-constexpr int kCqRing = 64;               // cells in each ring of a warp
+// local; now 3.5 and 8.3): 10.5 ms there and 23.6 ms, now 3.04 ms and 7.87 ms
+// (twelve warps in each of two blocks per SM); 428 us and 176 us on a
+// 200x200x150 map at 2 %/2 mm.  Two entries per lane and step and the cells'
+// dose ranges (wants_range) are the last 0.5 ms and 2.3 ms of these.
+constexpr int kCqRing = 128;              // cells in each ring of a warp (up to 31 + 64 wait)
 
 struct CqWarp {
     unsigned ring[2][kCqRing]; // pending cells of tiers 2 and 3: table entry << 5 | slot of the voxel
@@ -1464,12 +1494,11 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                 h4 += __shfl_xor_sync(kFull, h4, o);
             }
             unsigned above = hb;               // items of this bucket and costlier ones
-            float cells = (float)hb * bucket_cells(lane);
+            const float cells = queue_cells(hb);
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const unsigned u = __shfl_down_sync(kFull, above, o);
                 if (lane + o < 32) above += u;
-                cells += __shfl_xor_sync(kFull, cells, o);
             }
             s_start[lane] = above - hb;
             if (lane == 0) {
@@ -1489,6 +1518,7 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
     const float dnorm0 = BATCH ? 0.f : resolve_dnorm(P0);
     const bool stats = !BATCH && P0.stats;
     const unsigned nwarps = gridDim.x * (blockDim.x >> 5);
+    const bool use_range = !BATCH && wants_range(P0, s_cells);
 
     for (int part = 0; part < kCqParts; ++part) {
         const unsigned lo = part ? s_end[part - 1] : 0u, hi = s_end[part];
@@ -1575,6 +1605,7 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                                 ok |= 1u << u;
                             }
                         }
+                        drop_own_vertex<N>(cq, cx, cy, cz);
                         auto evaluate = [&](const Metric& mt, float dmax, float tau) {
                             CellGeom<float> cg;
                             cell_geom<N, float>(cx, cy, cz, mt, cg);
@@ -1663,62 +1694,61 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                 if (N == 3) reach = min(reach, min(z, Q.nz - 1 - z));
                 const float* const ev = Q.ev + V.vox[sl];
                 const WalkEntry* const tab = Q.walk;
+                // the cells' dose ranges, where they are worth a pass over the grid
+                const float2* const range = BATCH || !use_range ? nullptr : P0.range + V.vox[sl];
                 const float dr = V.dr[sl], inv = V.inv[sl];
                 const float best = live ? __uint_as_float(V.best[sl]) : -1.f;   // < 0: nothing is below it
-                WalkEntry en = tab[t];
-                // ---- tier 1: one table entry per lane and step ----
-                do {
-                    const WalkEntry e = en;
-                    const bool keyed = e.key * e.key < best;
-                    if (!__any_sync(kFull, keyed)) {
-                        t = -1;
-                        break;
-                    }
-                    const unsigned ent = (unsigned)t;
-                    t += g;
-                    en = tab[t];                       // the table is padded with unreachable keys
-                    bool cand = false, edge = false;   // edge: a cell with vertices outside the grid
-                    if (keyed) {
-                        const float* q = ev + e.lin;
-                        float dlo, dhi;
-                        bool in = true;
-                        if (e.margin <= reach) {
+                WalkEntry en0 = tab[t], en1 = tab[t + g];
+                // ---- tier 1: two table entries per lane and step ----
+                auto test = [&](const WalkEntry& e, bool& edge) -> bool {
+                    edge = false;                  // a cell with vertices outside the grid
+                    if (!(e.key2 < best)) return false;
+                    const float* q = ev + e.lin;
+                    float dlo, dhi;
+                    bool in = true;
+                    if (e.margin <= reach) {
+                        if (range) {
+                            const float2 r = __ldg(range + e.lin);
+                            dlo = r.x;
+                            dhi = r.y;
+                        } else {
                             float d[8];
 #pragma unroll
                             for (int u = 0; u < (1 << N); ++u)
                                 d[u] = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
+                            dlo = fminf(min3(d[0], d[1], d[2]), d[3]);
+                            dhi = fmaxf(max3(d[0], d[1], d[2]), d[3]);
                             if constexpr (N == 3) {
-                                dlo = fminf(min3(min3(d[0], d[1], d[2]), d[3], d[4]), min3(d[5], d[6], d[7]));
-                                dhi = fmaxf(max3(max3(d[0], d[1], d[2]), d[3], d[4]), max3(d[5], d[6], d[7]));
-                            } else {
-                                dlo = fminf(min3(d[0], d[1], d[2]), d[3]);
-                                dhi = fmaxf(max3(d[0], d[1], d[2]), d[3]);
+                                dlo = min3(min3(dlo, d[4], d[5]), d[6], d[7]);
+                                dhi = max3(max3(dhi, d[4], d[5]), d[6], d[7]);
                             }
-                        } else {
-                            // near the grid's faces: a cell outside it does not exist, one with
-                            // vertices outside keeps the faces that lie inside
-                            const int px = x + unpack10(e.off, 0), py = y + unpack10(e.off, 10), pz = z + unpack10(e.off, 20);
-                            in = (unsigned)px < (unsigned)nx && (unsigned)py < (unsigned)Q.ny &&
-                                 (N == 2 || (unsigned)pz < (unsigned)Q.nz);
-                            const bool ex = px + 1 < nx, ey = py + 1 < Q.ny, ez = N == 3 && pz + 1 < Q.nz;
-                            edge = !(ex && ey && (N == 2 || ez));
-                            dlo = kInf;
-                            dhi = -kInf;
-                            if (in) {
+                        }
+                    } else {
+                        // near the grid's faces: a cell outside it does not exist, one with
+                        // vertices outside keeps the faces that lie inside
+                        const int px = x + unpack10(e.off, 0), py = y + unpack10(e.off, 10), pz = z + unpack10(e.off, 20);
+                        in = (unsigned)px < (unsigned)nx && (unsigned)py < (unsigned)Q.ny &&
+                             (N == 2 || (unsigned)pz < (unsigned)Q.nz);
+                        const bool ex = px + 1 < nx, ey = py + 1 < Q.ny, ez = N == 3 && pz + 1 < Q.nz;
+                        edge = !(ex && ey && (N == 2 || ez));
+                        dlo = kInf;
+                        dhi = -kInf;
+                        if (in) {
 #pragma unroll
-                                for (int u = 0; u < (1 << N); ++u) {
-                                    if ((!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
-                                        const float f = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
-                                        dlo = fminf(dlo, f);
-                                        dhi = fmaxf(dhi, f);
-                                    }
+                            for (int u = 0; u < (1 << N); ++u) {
+                                if ((!(u & 1) || ex) && (!(u & 2) || ey) && (!(u & 4) || ez)) {
+                                    const float f = __ldg(q + (u & 1) + ((u & 2) ? nx : 0) + ((u & 4) ? sz : 0));
+                                    dlo = fminf(dlo, f);
+                                    dhi = fmaxf(dhi, f);
                                 }
                             }
                         }
-                        const float gap = max3(dlo - dr, dr - dhi, 0.f) * inv;
-                        cand = in && fmaf(gap, gap, e.key * e.key) < best;
                     }
-                    // a whole cell goes to tier 2, one at the grid's edge to tier 3
+                    const float gap = max3(dlo - dr, dr - dhi, 0.f) * inv;
+                    return in && fmaf(gap, gap, e.key2) < best;
+                };
+                // a whole cell goes to tier 2, one at the grid's edge to tier 3
+                auto push = [&](bool cand, bool edge, unsigned ent) {
                     const unsigned cm = __ballot_sync(kFull, cand && !edge);
                     if (cand && !edge)
                         V.ring[0][(head1 + cnt1 + (unsigned)__popc(cm & lt_mask)) & (kCqRing - 1)] = ent << 5 | (unsigned)slot;
@@ -1729,12 +1759,29 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                             V.ring[1][(head2 + cnt2 + (unsigned)__popc(em & lt_mask)) & (kCqRing - 1)] = ent << 5 | (unsigned)slot;
                         cnt2 += (unsigned)__popc(em);
                     }
+                };
+                do {
+                    const WalkEntry e0 = en0, e1 = en1;
+                    if (!__any_sync(kFull, e0.key2 < best)) {  // (of a lane's two keys the smaller)
+                        t = -1;
+                        break;
+                    }
+                    const unsigned ent = (unsigned)t;
+                    t += 2 * g;
+                    en0 = tab[t];                  // the table is padded with unreachable keys
+                    en1 = tab[t + g];
+                    bool g0, g1;
+                    const bool c0 = test(e0, g0), c1 = test(e1, g1);
+                    push(c0, g0, ent);
+                    push(c1, g1, ent + (unsigned)g);
                     if (stats) {
-                        const unsigned km = __ballot_sync(kFull, keyed), pm = __ballot_sync(kFull, keyed && !cand);
+                        const unsigned k0 = __ballot_sync(kFull, e0.key2 < best), k1 = __ballot_sync(kFull, e1.key2 < best);
+                        const unsigned p0 = __ballot_sync(kFull, e0.key2 < best && !c0),
+                                       p1 = __ballot_sync(kFull, e1.key2 < best && !c1);
                         if (lane == 0) {
-                            atomicAdd(&s_stat[1], (unsigned long long)__popc(pm));
-                            atomicAdd(&s_stat[2], (unsigned long long)__popc(km));
-                            atomicAdd(&s_stat[3], 32ull);
+                            atomicAdd(&s_stat[1], (unsigned long long)(__popc(p0) + __popc(p1)));
+                            atomicAdd(&s_stat[2], (unsigned long long)(__popc(k0) + __popc(k1)));
+                            atomicAdd(&s_stat[3], 64ull);
                         }
                     }
                 } while (max(cnt1, cnt2) < 32u);
@@ -1951,7 +1998,7 @@ __device__ __forceinline__ float visit_cell_box(const Problem& P, const float* _
         return best;
     }
     if (P.stats) ++st.visited;
-    const float cb = cell_all_faces<N>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy,
+    const float cb = cell_all_faces<N, true>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy,
                                        cz, p, dr, dnorm);
     return fminf(best, cb);
 }

@@ -182,7 +182,7 @@ __device__ __forceinline__ float paper_cell(const Problem& P, int x, int y, int 
         }
     }
     if constexpr (!JU) {
-        return cell_all_faces<N>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy, cz,
+        return cell_all_faces<N, false>(P, q[0], q[1], q[2], q[3], q[4], q[5], q[6], q[7], ok, cx, cy, cz,
                                  p, dr, dnorm);
     } else {
         constexpr int full = (1 << N) - 1;

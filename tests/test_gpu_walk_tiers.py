@@ -55,3 +55,21 @@ def test_long_queue_takes_whole_batches_of_rounds():
     assert sb["tail_voxels"] > 100000
     np.testing.assert_array_equal(a, b)
     assert ca == cb
+
+
+@pytest.mark.parametrize("shape", [(17, 33, 31), (16, 20, 32), (34, 18, 63), (2, 40, 65), (90, 62), (47, 130)], ids=str)
+def test_costly_queue_reads_dose_ranges(shape):
+    # a dose offset of many gamma: hundreds of tested cells per voxel of the
+    # grid, far past the line where the cells' dose ranges come from an array;
+    # rows and columns around the 31 cells and 16 planes of its pass
+    rng = np.random.default_rng(sum(shape))
+    ref = rng.uniform(0.5, 0.6, shape).astype(np.float32)
+    ev = rng.uniform(0.7, 0.9, shape).astype(np.float32)
+    sp = (1.0, 1.5, 1.25)[3 - len(shape):]
+    c = synth.Criteria(0.03, 1.5)
+    a, ca, sa = gpu_gamma(ref, ev, sp, c, {"walk": 0, "stats": 1})
+    b, cb, sb = gpu_gamma(ref, ev, sp, c, {"walk": 3, "stats": 1})
+    assert sb["cells_keyed"] > 12 * ref.size
+    np.testing.assert_array_equal(a, b)
+    assert ca == cb
+    assert_parity(b, oracle_gamma(ref, ev, sp, c), cb)
