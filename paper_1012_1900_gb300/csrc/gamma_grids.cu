@@ -34,6 +34,7 @@
 #include "../../include/gamma.h"
 #include "gamma_cell.cuh"
 #include "gamma_internal.h"
+#include "gamma_launch.cuh"
 #include "gamma_plane.cuh"
 
 namespace gk {
@@ -68,6 +69,8 @@ __device__ __forceinline__ int grid_variant(const float (&fr)[3], int nd)
 
 __global__ void __launch_bounds__(256) k_grid_prepare(const __grid_constant__ GridProblem G)
 {
+    grid_release();
+    grid_wait();
     float m = -kInf;
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -154,6 +157,7 @@ __device__ __forceinline__ float grid_cell(const GridProblem& G, const int (&p)[
 template <int N, int GL>
 __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ GridProblem G)
 {
+    grid_wait();                       // (the last kernel: nothing is released early)
     const int lane = threadIdx.x & 31, gl = lane & (GL - 1), gbase = lane & ~(GL - 1);
     const unsigned gmask = GL == 32 ? kFull : (((1u << GL) - 1u) << gbase);
     const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
@@ -328,6 +332,8 @@ constexpr int kGridSteps = 3;
 template <int N>
 __global__ void __launch_bounds__(256) k_grid_seed(const __grid_constant__ GridProblem G)
 {
+    grid_release();
+    grid_wait();
     const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
     const float thr = cutoff_threshold(G.local, G.cutoff_frac, dnorm);
     const int sy = G.en[0], sz = G.en[0] * G.en[1], lane = threadIdx.x & 31;
@@ -427,6 +433,8 @@ template <int N>
 __global__ void __launch_bounds__(384, 2) k_grid_cq(const __grid_constant__ GridProblem G)
 {
     __shared__ GqWarp gqw[12];
+    grid_release();
+    grid_wait();
     GqWarp& W = gqw[threadIdx.x >> 5];
     volatile GqWarp& V = gqw[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31, g = G.lanes, gl = lane & (g - 1);
@@ -750,13 +758,13 @@ cudaError_t launch_grids(const GridProblem& G, cudaStream_t s)
     // voxels it left
     const int gs = (int)std::max<long long>(1, std::min<long long>((G.nref + 255) / 256, (long long)sms * 8));
     if (G.ndim == 3) {
-        k_grid_seed<3><<<gs, 256, 0, s>>>(G);
-        k_grid_cq<3><<<sms * 2, 384, 0, s>>>(G);
-        k_grid_walk<3, 32><<<sms * 2, 256, 0, s>>>(G);
+        launch_next(k_grid_seed<3>, gs, 256, 0, s, G);
+        launch_next(k_grid_cq<3>, sms * 2, 384, 0, s, G);
+        launch_next(k_grid_walk<3, 32>, sms * 2, 256, 0, s, G);
     } else {
-        k_grid_seed<2><<<gs, 256, 0, s>>>(G);
-        k_grid_cq<2><<<sms * 2, 384, 0, s>>>(G);
-        k_grid_walk<2, 32><<<sms * 2, 256, 0, s>>>(G);
+        launch_next(k_grid_seed<2>, gs, 256, 0, s, G);
+        launch_next(k_grid_cq<2>, sms * 2, 384, 0, s, G);
+        launch_next(k_grid_walk<2, 32>, sms * 2, 256, 0, s, G);
     }
     return cudaGetLastError();
 }

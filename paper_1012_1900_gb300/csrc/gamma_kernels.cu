@@ -25,6 +25,7 @@
 
 #include "gamma_cell.cuh"
 #include "gamma_internal.h"
+#include "gamma_launch.cuh"
 #include "gamma_near.cuh"
 #include "gamma_plane.cuh"
 #include "gamma_tma.cuh"
@@ -41,6 +42,8 @@ template <bool BATCH>
 __global__ void __launch_bounds__(256)
     k_prepare(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd, int part)
 {
+    grid_release();
+    grid_wait();
     const Problem& P = BATCH ? bd->probs[blockIdx.y] : P0;
     if constexpr (BATCH) {
         if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
@@ -444,6 +447,8 @@ __global__ void __launch_bounds__(256, MINB)
         mbar_fence_init();
     }
     __syncthreads();
+    grid_release();
+    grid_wait();
 
     // global tile -> (pair, tile of that pair)
     auto locate = [&](int t, int& pr, int& lt) {
@@ -821,6 +826,8 @@ __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem
 {
     __shared__ unsigned start[kNumBuckets], cnt[kNumBuckets], base[kNumBuckets];
     __shared__ float s_cells;
+    grid_release();
+    grid_wait();
     if (threadIdx.x < kNumBuckets) {
         const unsigned own = P.ctr->hist[threadIdx.x];
         unsigned sum = own;                    // of this bucket and the costlier ones
@@ -963,6 +970,8 @@ __global__ void __launch_bounds__(256) k_bucket_scan_batch(const BatchDesc* __re
     __shared__ unsigned sc[4][256];
     __shared__ unsigned hsum[kNumBuckets];
     __shared__ int sh_b[3];
+    grid_release();
+    grid_wait();
     const int np = bd->npairs, tid = threadIdx.x;
     if (bd->group_bucket < 0) {
         // parts chosen from the group's queue (auto_part_buckets over every pair's histogram)
@@ -1053,6 +1062,8 @@ __global__ void __launch_bounds__(256) k_bucket_scan_batch(const BatchDesc* __re
 __global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restrict__ bd)
 {
     __shared__ unsigned cnt[kNumBuckets], base[kNumBuckets];
+    grid_release();
+    grid_wait();
     const Problem& P = bd->probs[blockIdx.y];
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     for (unsigned c0 = blockIdx.x * blockDim.x; c0 < total; c0 += gridDim.x * blockDim.x) {
@@ -1311,6 +1322,8 @@ __global__ void __launch_bounds__(256)
     k_plane_seed(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd)
 {
     __shared__ unsigned sh_hist[kNumBuckets];
+    grid_release();
+    grid_wait();
     const Problem& P = BATCH ? bd->probs[blockIdx.y] : P0;
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     if (blockIdx.x * blockDim.x >= total) return;             // block-uniform
@@ -1465,6 +1478,8 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
     volatile CqWarp& V = cqw[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
+    grid_release();
+    grid_wait();
     if (threadIdx.x < 32) {
         if constexpr (BATCH) {
             // the group's queue: the parts of every pair, costliest part first
@@ -1854,6 +1869,7 @@ template <int N, bool BATCH>
 __global__ void __launch_bounds__(256) k_tail_fix(const __grid_constant__ Problem P0,
                                                   const BatchDesc* __restrict__ bd)
 {
+    grid_wait();                       // (the run's last kernel: nothing is released early)
     const int lane = threadIdx.x & 31;
     const unsigned nfix = BATCH ? *bd->fix_count : P0.ctr->fix_count;
     unsigned my_eval = 0, my_pass = 0, my_over = 0;
@@ -2677,10 +2693,10 @@ static void launch_shell_w_k(int per_sm, unsigned grid, cudaStream_t s, const Pr
                              unsigned* next, const SlabGate& gate, const BatchDesc* bd)
 {
     switch (per_sm) {
-    case 1: k_shell_w<N, 1, BATCH><<<grid, 256, 0, s>>>(P, map, use_tma, t_first, tiles, next, gate, bd); break;
-    case 2: k_shell_w<N, 2, BATCH><<<grid, 256, 0, s>>>(P, map, use_tma, t_first, tiles, next, gate, bd); break;
-    case 3: k_shell_w<N, 3, BATCH><<<grid, 256, 0, s>>>(P, map, use_tma, t_first, tiles, next, gate, bd); break;
-    default: k_shell_w<N, 4, BATCH><<<grid, 256, 0, s>>>(P, map, use_tma, t_first, tiles, next, gate, bd); break;
+    case 1: launch_next(k_shell_w<N, 1, BATCH>, grid, 256, 0, s, P, map, use_tma, t_first, tiles, next, gate, bd); break;
+    case 2: launch_next(k_shell_w<N, 2, BATCH>, grid, 256, 0, s, P, map, use_tma, t_first, tiles, next, gate, bd); break;
+    case 3: launch_next(k_shell_w<N, 3, BATCH>, grid, 256, 0, s, P, map, use_tma, t_first, tiles, next, gate, bd); break;
+    default: launch_next(k_shell_w<N, 4, BATCH>, grid, 256, 0, s, P, map, use_tma, t_first, tiles, next, gate, bd); break;
     }
 }
 
@@ -2760,15 +2776,15 @@ cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s)
 {
     if (!P.plane_raw) return cudaSuccess;
     const int grid = grid_for(P.nvox, 256, device_sm_count() * 8);
-    if (P.ndim == 3) k_plane_seed<3, false><<<grid, 256, 0, s>>>(P, nullptr);
-    else k_plane_seed<2, false><<<grid, 256, 0, s>>>(P, nullptr);
+    if (P.ndim == 3) launch_next(k_plane_seed<3, false>, grid, 256, 0, s, P, nullptr);
+    else launch_next(k_plane_seed<2, false>, grid, 256, 0, s, P, nullptr);
     return cudaGetLastError();
 }
 
 cudaError_t launch_order_tail(const Problem& P, cudaStream_t s)
 {
     if (!P.sort_tail) return cudaSuccess;
-    k_scatter<<<grid_for(P.nvox, 256, device_sm_count() * 8), 256, 0, s>>>(P);
+    launch_next(k_scatter, grid_for(P.nvox, 256, device_sm_count() * 8), 256, 0, s, P);
     return cudaGetLastError();
 }
 
@@ -2812,12 +2828,12 @@ static void launch_tail_cq_n(const Problem& P, const BatchDesc* bd, int per_sm, 
     // persistent: one wave of resident blocks (fewer where even a voxel per
     // lane group would leave blocks without work)
     const int grid = BATCH ? sms * per_sm : grid_for(P.nvox, cq_threads(per_sm) / 32, sms * per_sm);
-    if (per_sm >= 4) k_tail_cq<N, 4, BATCH><<<grid, cq_threads(4), 0, s>>>(P, bd);
-    else if (per_sm == 3) k_tail_cq<N, 3, BATCH><<<grid, cq_threads(3), 0, s>>>(P, bd);
-    else if (per_sm == 2) k_tail_cq<N, 2, BATCH><<<grid, cq_threads(2), 0, s>>>(P, bd);
-    else k_tail_cq<N, 1, BATCH><<<grid, cq_threads(1), 0, s>>>(P, bd);
+    if (per_sm >= 4) launch_next(k_tail_cq<N, 4, BATCH>, grid, cq_threads(4), 0, s, P, bd);
+    else if (per_sm == 3) launch_next(k_tail_cq<N, 3, BATCH>, grid, cq_threads(3), 0, s, P, bd);
+    else if (per_sm == 2) launch_next(k_tail_cq<N, 2, BATCH>, grid, cq_threads(2), 0, s, P, bd);
+    else launch_next(k_tail_cq<N, 1, BATCH>, grid, cq_threads(1), 0, s, P, bd);
     // (a warp per listed voxel; most often there is none)
-    k_tail_fix<N, BATCH><<<BATCH ? device_sm_count() * 2 : grid_for(P.nvox, 8, device_sm_count() * 2), 256, 0, s>>>(P, bd);
+    launch_next(k_tail_fix<N, BATCH>, BATCH ? sms * 2 : grid_for(P.nvox, 8, sms * 2), 256, 0, s, P, bd);
 }
 
 cudaError_t launch_tail_cq(const Problem& P, int tail_minblocks, cudaStream_t s)
@@ -2912,7 +2928,7 @@ cudaError_t launch_batch_prepare(const BatchGroup& g, cudaStream_t s)
     const int sms = device_sm_count();
     const int bx = grid_for(g.max_nvox, 256, std::max(1, sms * 8 / std::max(1, g.npairs)) + 1);
     Problem dummy{};
-    k_prepare<true><<<dim3(bx, g.npairs), 256, 0, s>>>(dummy, g.desc, 1);   // k_shell checks the evaluation dose
+    launch_next(k_prepare<true>, dim3(bx, g.npairs), 256, 0, s, dummy, g.desc, 1);   // k_shell checks the evaluation dose
     return cudaGetLastError();
 }
 
@@ -2937,19 +2953,19 @@ cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s)
     if (g.npairs <= 0) return cudaSuccess;
     Problem dummy{};
     const dim3 grid((unsigned)grid_for(g.max_nvox, 256, device_sm_count() * 4), (unsigned)g.npairs);
-    if (g.ndim == 3) k_plane_seed<3, true><<<grid, 256, 0, s>>>(dummy, g.desc);
-    else k_plane_seed<2, true><<<grid, 256, 0, s>>>(dummy, g.desc);
+    if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, 256, 0, s, dummy, g.desc);
+    else launch_next(k_plane_seed<2, true>, grid, 256, 0, s, dummy, g.desc);
     return cudaGetLastError();
 }
 
 cudaError_t launch_batch_order(const BatchGroup& g, cudaStream_t s)
 {
     if (g.npairs <= 0) return cudaSuccess;
-    k_bucket_scan_batch<<<1, 256, 0, s>>>(g.desc);
+    launch_next(k_bucket_scan_batch, 1, 256, 0, s, g.desc);
     // enough blocks per pair for the largest queue (one 256-voxel chunk per
     // block and pass); the blocks of small pairs leave at once
     const int sms = device_sm_count();
-    k_scatter_batch<<<dim3(sms * 4, g.npairs), 256, 0, s>>>(g.desc);
+    launch_next(k_scatter_batch, dim3(sms * 4, g.npairs), 256, 0, s, g.desc);
     return cudaGetLastError();
 }
 

@@ -21,6 +21,7 @@
 #include "../../include/gamma.h"
 #include "gamma_cell.cuh"
 #include "gamma_internal.h"
+#include "gamma_launch.cuh"
 #include "gamma_mlp.cuh"
 #include "gamma_plane.cuh"
 #include "gamma_tc.cuh"
@@ -123,6 +124,8 @@ __device__ __forceinline__ void row_features(const Problem& P, unsigned v, float
 // Queue items past the cost gate (bucket >= min_bucket), into P.seed_list.
 __global__ void __launch_bounds__(256) k_seed_select(const __grid_constant__ Problem P, int min_bucket)
 {
+    grid_release();
+    grid_wait();
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     const int lane = threadIdx.x & 31;
     const unsigned stride = gridDim.x * blockDim.x;
@@ -480,6 +483,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_rows(const __grid_consta
     unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     TcSmem& S = *reinterpret_cast<TcSmem*>(base);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    grid_release();
+    grid_wait();
     const long long nrows = count_dev ? min((long long)*count_dev, M) : M;
     const long long ntiles = (nrows + kRows - 1) / kRows;
     if ((long long)blockIdx.x >= ntiles) return;                  // block-uniform
@@ -642,7 +647,10 @@ cudaError_t launch_mlp_rows(const MlpWeights& W, const bf16* X, long long M, con
     if (e != cudaSuccess) return e;
     const long long tiles = (M + kRows - 1) / kRows;
     const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, device_sm_count()));
-    k_mlp_rows<<<grid, kMlpThreads, kTcSmemBytes, s>>>(W, xmap, M, count_dev, Y, flags, host_flags);
+    if (count_dev)       // within a run: the kernels before it on the stream are the run's own
+        launch_next(k_mlp_rows, grid, kMlpThreads, kTcSmemBytes, s, W, xmap, M, count_dev, Y, flags, host_flags);
+    else
+        k_mlp_rows<<<grid, kMlpThreads, kTcSmemBytes, s>>>(W, xmap, M, count_dev, Y, flags, host_flags);
     return cudaGetLastError();
 }
 
@@ -1052,6 +1060,8 @@ __global__ void __launch_bounds__(256) k_seed_features(const __grid_constant__ P
                                                        const BatchDesc* __restrict__ bd)
 {
     __shared__ float sh_e[8][FeatBox<N>::ELEMS], sh_r[8][FeatBox<N>::ELEMS];
+    grid_release();
+    grid_wait();
     const SeedRows<BATCH> rows{&P0, bd};
     const unsigned total = rows.count();
     bf16* X = rows.X();
@@ -1075,6 +1085,8 @@ template <int N, bool BATCH>
 __global__ void __launch_bounds__(256) k_seed_apply(const __grid_constant__ Problem P0,
                                                     const BatchDesc* __restrict__ bd)
 {
+    grid_release();
+    grid_wait();
     const SeedRows<BATCH> rows{&P0, bd};
     const unsigned total = rows.count();
     const float* Y = rows.Y();
@@ -1169,6 +1181,8 @@ __global__ void __launch_bounds__(256) k_seed_apply(const __grid_constant__ Prob
 __global__ void __launch_bounds__(256) k_seed_select_batch(const BatchDesc* __restrict__ bd,
                                                            int min_bucket)
 {
+    grid_release();
+    grid_wait();
     const Problem& P = bd->probs[blockIdx.y];
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
     const int lane = threadIdx.x & 31;
@@ -1196,18 +1210,18 @@ static cudaError_t launch_seeding_n(const Problem& P, const BatchDesc* bd, const
                                     unsigned* flags, cudaStream_t s)
 {
     const int sms = device_sm_count();
-    k_seed_features<N, BATCH><<<sms * 16, 256, 0, s>>>(P, bd);
+    launch_next(k_seed_features<N, BATCH>, sms * 16, 256, 0, s, P, bd);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if ((e = launch_mlp_rows(W, X, cap, count, Y, flags, 0, s)) != cudaSuccess) return e;
-    k_seed_apply<N, BATCH><<<sms * 8, 256, 0, s>>>(P, bd);
+    launch_next(k_seed_apply<N, BATCH>, sms * 8, 256, 0, s, P, bd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_seeding(const Problem& P, const MlpWeights& W, int min_bucket, cudaStream_t s)
 {
     if (!P.seed_list || !P.seed_X || !P.seed_Y || P.seed_cap == 0) return cudaErrorInvalidValue;
-    k_seed_select<<<device_sm_count() * 4, 256, 0, s>>>(P, min_bucket);
+    launch_next(k_seed_select, device_sm_count() * 4, 256, 0, s, P, min_bucket);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return P.ndim == 3
@@ -1222,7 +1236,7 @@ cudaError_t launch_batch_seeding(const BatchGroup& g, const MlpWeights& W, int m
 {
     if (g.npairs <= 0 || g.seed_cap == 0) return cudaSuccess;
     const int bx = std::max(1, device_sm_count() * 2 / std::max(1, g.npairs)) + 1;
-    k_seed_select_batch<<<dim3(bx, g.npairs), 256, 0, s>>>(g.desc, min_bucket);
+    launch_next(k_seed_select_batch, dim3(bx, g.npairs), 256, 0, s, g.desc, min_bucket);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     Problem dummy{};
