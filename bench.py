@@ -60,8 +60,8 @@ FLOP_PER_CELL = {3: 615, 2: 103}
 FP32_LANES_PER_SM = 128
 L2_FLUSH_BYTES = 256 << 20
 # kernels of one single-pair run: prepare, shell, scatter and the walk (the
-# warp-evaluated walk adds its finishing pass, k_tail_fix)
-WALKERS = {-1: ("k_tail_cq", 5), 3: ("k_tail_cq", 5), 0: ("k_tail", 4), 1: ("k_walk", 4),
+# warp-evaluated walk adds its plane seeds and its finishing pass, k_tail_fix)
+WALKERS = {-1: ("k_tail_cq", 6), 3: ("k_tail_cq", 6), 0: ("k_tail", 4), 1: ("k_walk", 4),
            2: ("k_walk_rows", 4)}
 LOAD_S = 1.5                 # back-to-back maps before the timed steps (clock samples)
 # gamma within this distance of 1 may pass on one side and fail on the other
@@ -783,8 +783,8 @@ def run_ours(args, pair, rank, world, local_rank):
         return
 
     # ---- roofline of the search ----
-    # The exact search runs as two phases, k_shell (faces through each voxel)
-    # and the queued voxels' table walks (k_tail_cq and its finishing pass by
+    # The exact search runs as two phases, k_shell (faces through each voxel,
+    # with the queued voxels' plane seeds by default) and the queued voxels' table walks (k_tail_cq and its finishing pass by
     # default); which phase certifies a voxel's remaining key-0 faces depends
     # on the pruning, so the implementation-independent census is charged to
     # the two together.  The per-kernel figures split it as census key-0

@@ -209,12 +209,16 @@ int gamma_get_timings(gamma_handle h, gamma_timings *out);
 
 /* Tuning and diagnostic options (take effect at the next run):
  *  "walk"             3 (default): voxel by voxel
- *                     from a queue ordered by cost; a cell that passes the
- *                     dose-gap test joins a per-warp buffer, and the warp
- *                     evaluates 32 such cells at a time, one per lane; the
- *                     most expensive voxels walk 4 lanes each (options
- *                     "group_bucket", "group8_bucket"; "lanes_per_voxel" does
- *                     not apply).  0: voxel by voxel, "lanes_per_voxel" lanes
+ *                     from a queue ordered by cost, each voxel starting from
+ *                     the bound of one cell near its nearest surface point; a
+ *                     cell that passes the dose-gap test joins a per-warp
+ *                     buffer, and the warp tests 32 such cells at a time, one
+ *                     per lane, by a plane bound and evaluates those that
+ *                     pass it, again 32 at a time; the most expensive voxels
+ *                     walk 4 lanes each (options "group_bucket",
+ *                     "group8_bucket"; "lanes_per_voxel" does not apply), and
+ *                     every voxel more lanes while the queue is too short to
+ *                     fill the chip.  0: voxel by voxel, "lanes_per_voxel" lanes
  *                     each, every lane evaluating its own cells
  *                     (gamma_run_noalloc always walks this way; batch handles
  *                     take 0 or 3 only); 1: tile by
@@ -232,7 +236,8 @@ int gamma_get_timings(gamma_handle h, gamma_timings *out);
  *  "group_bucket"     "walk" 3: queued voxels whose cost bucket (1 + floor(2
  *                     log2 of the cells below their starting bound)) is at
  *                     least this value walk 4 lanes each, the rest one lane
- *                     each (default 9; 32: every voxel one lane).  -1: the
+ *                     each (default 9; 32: every voxel one lane; more on short
+ *                     queues).  -1: the
  *                     walk chooses this and the next two thresholds from the
  *                     queue: with c(b) = 2^((2b - 1)/4) cells per voxel of
  *                     bucket b and T = (sum of c over the queue) / (the
@@ -277,7 +282,8 @@ int gamma_get_timings(gamma_handle h, gamma_timings *out);
  *                     every simplex of every cell; 2 the same without the
  *                     sort.  Same results; allocates 16 bytes per voxel.
  *  "seed_min_bucket"  with a model attached: only queued voxels whose cost
- *                     bucket (1 + floor(2 log2 cells with key < gamma0)) is
+ *                     bucket (1 + floor(2 log2 cells with key below its
+ *                     starting bound)) is
  *                     at least this get a proposal (default 13: >= 64 cells);
  *                     0 seeds every queued voxel
  *  "drop_slab_flag"   failure test: k + 1 leaves slab k's readiness flag
@@ -321,7 +327,7 @@ typedef struct {
 
 /* Create a batch handle over 1 <= n_pairs <= 65535 descriptors (copied;
  * device buffers borrowed).  Each pair gets its own cell table and scratch;
- * the handle adds 6 bytes per voxel of all pairs for the shared work order.
+ * the handle adds 10 bytes per voxel of all pairs for the shared work order.
  * Errors: INVALID_ARG, SHAPE, OOM, TABLE_TOO_LARGE, CUDA.  Synchronous. */
 int gamma_batch_create(gamma_handle *out, int n_pairs, const gamma_pair_desc *pairs);
 

@@ -1,20 +1,26 @@
 // CUDA kernels of the gamma search (sm_103a).
 //
-// One run over a dose pair is four stream-ordered launches:
-//   k_prepare   max of the reference dose (the global dose norm) and its
-//               finite check (k_shell checks the evaluation dose, every value
-//               of which is the centre of one tile voxel)  (Algorithm A2 step 2)
-//   k_shell     per reference voxel: criteria, low-dose cutoff, gamma0 =
-//               DD/dD (A1 step 4a) and every face through the voxel's node
-//               (reduced closed form), from a TMA-staged tile; voxels whose
-//               running gamma still exceeds the distance to any other face
-//               are queued with a cost bucket
-//   k_scatter   order the queue by estimated cost, most expensive first (the
-//               role the paper's DD sort plays, Section 2.2 and Table 2)
-//   k_tail      persistent: a group of G lanes takes one queued voxel and
-//               walks the sorted cell table G cells at a time, with the exact
-//               early exit of A1 step 4b-ii (key >= gamma) and a per-cell
-//               lower bound sqrt(key^2 + dose gap^2)
+// One run over a dose pair is six stream-ordered launches:
+//   k_prepare     max of the reference dose (the global dose norm) and its
+//                 finite check (the shell checks the evaluation dose, every
+//                 value of which is the centre of one tile voxel)  (Algorithm
+//                 A2 step 2)
+//   k_shell_w     per reference voxel: criteria, low-dose cutoff, gamma0 =
+//                 DD/dD (A1 step 4a) and every face through the voxel's node
+//                 (reduced closed form), from a TMA-staged tile; voxels whose
+//                 running gamma still exceeds the distance to any other face
+//                 are queued with a cost bucket
+//   k_plane_seed  a tight bound for every queued voxel from one cell near its
+//                 nearest surface point
+//   k_scatter     order the queue by estimated cost, most expensive first (the
+//                 role the paper's DD sort plays, Section 2.2 and Table 2)
+//   k_tail_cq     persistent: warps walk the sorted cell table for batches of
+//                 queued voxels with the exact early exit of A1 step 4b-ii
+//                 (key >= gamma), the dose gap and a plane bound, and evaluate
+//                 what is left 32 cells at a time
+//   k_tail_fix    the voxels with a near-singular cell or past a cut table
+// The other walks (options walk = 0, 1, 2) take k_tail, k_walk or k_walk_rows
+// in place of the seeds and the last two.
 // No kernel waits on another block or allocates memory.
 #include <cuda.h>
 #include <cuda_runtime.h>
