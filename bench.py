@@ -364,7 +364,7 @@ def shard_pairs(costs, world: int, rank: int):
 
 
 SEARCH_SOURCES = ("gamma_kernels.cu", "gamma_cell.cuh", "gamma_face.cuh", "gamma_near.cuh",
-                  "gamma_tma.cuh", "gamma_internal.h")
+                  "gamma_plane.cuh", "gamma_tma.cuh", "gamma_launch.cuh", "gamma_internal.h")
 
 
 def search_source_hash() -> str:
