@@ -1320,11 +1320,17 @@ constexpr int kPlaneSteps = 3;
 // here) are those of the walk that follows.  The bound is a true distance to
 // the surface, so the result does not depend on it.  One thread per voxel;
 // the cells differ per lane but every lane evaluates exactly one.  Bound by
-// the latency of the dependent dose loads on short queues, by issue on long
-// ones (53 %): 648 k voxels of a 200x200x150 map take 36 us, 5.9 M of a
-// 320x320x240 map 270 us, and spare the walk half of its time there.
+// the latency of the dependent dose loads: 136 k voxels of a 160x160x120 map
+// take 13.2 us, 648 k of a 200x200x150 map 35 us, 5.9 M of a 320x320x240 map
+// 263 us, and spare the walk half of its time there.  Batched volumes, whose
+// form needs 97 registers, take 64 (144 bytes spilled) in blocks of 128 for 32
+// instead of 16 warps per SM: a batch's eight volumes 55.6 to 38.8 us.  For
+// one pair the same (16 bytes spilled) is 10.4, 31 and 234 us, but a map of
+// 99 k queued voxels, one wave of blocks either way, lost 1 us in 89.
+__host__ __device__ constexpr int seed_threads(int n, bool batch) { return n == 3 && batch ? 128 : 256; }
+
 template <int N, bool BATCH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH) == 128 ? 8 : 0)
     k_plane_seed(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd)
 {
     __shared__ unsigned sh_hist[kNumBuckets];
@@ -2781,9 +2787,9 @@ cudaError_t launch_patch_host(const Problem& P, float* host_out_mapped, Counters
 cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s)
 {
     if (!P.plane_raw) return cudaSuccess;
-    const int grid = grid_for(P.nvox, 256, device_sm_count() * 8);
-    if (P.ndim == 3) launch_next(k_plane_seed<3, false>, grid, 256, 0, s, P, nullptr);
-    else launch_next(k_plane_seed<2, false>, grid, 256, 0, s, P, nullptr);
+    const int t = seed_threads(P.ndim, false), grid = grid_for(P.nvox, t, device_sm_count() * 8);
+    if (P.ndim == 3) launch_next(k_plane_seed<3, false>, grid, t, 0, s, P, nullptr);
+    else launch_next(k_plane_seed<2, false>, grid, t, 0, s, P, nullptr);
     return cudaGetLastError();
 }
 
@@ -2958,9 +2964,10 @@ cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s)
 {
     if (g.npairs <= 0) return cudaSuccess;
     Problem dummy{};
-    const dim3 grid((unsigned)grid_for(g.max_nvox, 256, device_sm_count() * 4), (unsigned)g.npairs);
-    if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, 256, 0, s, dummy, g.desc);
-    else launch_next(k_plane_seed<2, true>, grid, 256, 0, s, dummy, g.desc);
+    const int t = seed_threads(g.ndim, true);
+    const dim3 grid((unsigned)grid_for(g.max_nvox, t, device_sm_count() * (1024 / t)), (unsigned)g.npairs);
+    if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, t, 0, s, dummy, g.desc);
+    else launch_next(k_plane_seed<2, true>, grid, t, 0, s, dummy, g.desc);
     return cudaGetLastError();
 }
 
