@@ -1794,7 +1794,11 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                         break;
                     }
                     const unsigned ent = (unsigned)t;
-                    t += 2 * g;
+                    // A lane whose key is past its bound stays where it is: in a batch
+                    // the lanes' voxels may belong to pairs with tables of different
+                    // lengths, and one that went on with the others would leave its own.
+                    // (Of one pair the round ends within 2 g entries of the table's end.)
+                    if (!BATCH || e0.key2 < best) t += 2 * g;
                     en0 = tab[t];                  // the table is padded with unreachable keys
                     en1 = tab[t + g];
                     bool g0, g1;
