@@ -105,6 +105,7 @@ struct Counters {
     unsigned int row_cursor[kNumBuckets];
     unsigned int head_part[4];          // warp-evaluated walk: work counters of the queue's parts
     unsigned int fix_count;             // ... voxels it leaves to the finishing pass
+    unsigned int range_on;              // ... 1: this run's ordering pass wrote the cells' dose ranges
     unsigned long long lane_steps;      // stats mode: lane slots of its loop steps, idle lanes included
 };
 

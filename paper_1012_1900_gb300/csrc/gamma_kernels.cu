@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(256, MINB)
 __device__ __forceinline__ float bucket_cells(int b) { return b > 0 ? exp2f((2 * b - 1) * 0.25f) : 0.5f; }
 
 // The estimated cells of a whole queue, lane b of a full warp holding the count
-// of bucket b (every caller gets the same bits).
+// of bucket b.
 __device__ __forceinline__ float queue_cells(unsigned count)
 {
     float c = (float)count * bucket_cells(threadIdx.x & 31);
@@ -782,7 +782,8 @@ __device__ __forceinline__ float queue_cells(unsigned count)
 }
 
 // Whether the walk of a queue with this many estimated cells takes the cells'
-// dose ranges from an array, which the ordering kernel then writes: one read
+// dose ranges from an array, which the ordering kernel then writes (it decides,
+// and tells the walk with Counters::range_on): one read
 // per tested cell instead of eight and their minimum and maximum, for a pass
 // over the grid that reads 4 and writes 8 bytes per voxel.  The line lies where
 // the pass (2.8 us per million voxels) meets what it saves (1.3 to 2.2 us per
@@ -792,6 +793,16 @@ constexpr float kRangeCells = 3.f;                 // tested cells per grid voxe
 __device__ __forceinline__ bool wants_range(const Problem& P, float cells)
 {
     return P.range && P.plane_raw && cells > kRangeCells * (float)P.nvox;
+}
+
+// A dose range, by an ordinary load: the kernel before writes them, and this one
+// may have been set up meanwhile, so they are not read-only for its lifetime.
+// (Constant once the walk runs, so the compiler may move it like a read-only one.)
+__device__ __forceinline__ float2 load_range(const float2* p)
+{
+    float2 r;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
 }
 
 // The queue's parts chosen from the queue itself (option group_bucket < 0):
@@ -869,6 +880,7 @@ __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ Problem
         __syncthreads();
     }
     if (!wants_range(P, s_cells)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) P.ctr->range_on = 1u;
     // the dose range of every cell whose vertices all lie in the grid: a warp
     // takes a segment of 31 cells along x and marches along z, each node read once
     const int lane = threadIdx.x & 31;
@@ -1545,7 +1557,7 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
     const float dnorm0 = BATCH ? 0.f : resolve_dnorm(P0);
     const bool stats = !BATCH && P0.stats;
     const unsigned nwarps = gridDim.x * (blockDim.x >> 5);
-    const bool use_range = !BATCH && wants_range(P0, s_cells);
+    const bool use_range = !BATCH && P0.range && P0.ctr->range_on;
 
     for (int part = 0; part < kCqParts; ++part) {
         const unsigned lo = part ? s_end[part - 1] : 0u, hi = s_end[part];
@@ -1735,7 +1747,7 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                     bool in = true;
                     if (e.margin <= reach) {
                         if (range) {
-                            const float2 r = __ldg(range + e.lin);
+                            const float2 r = load_range(range + e.lin);
                             dlo = r.x;
                             dhi = r.y;
                         } else {
