@@ -290,8 +290,9 @@ __device__ __forceinline__ void near_gamma2_pair(const float* tile, int tix, flo
                                         Near2::pack(__fmul_rn(dD0, dD0), __fmul_rn(dD1, dD1)), kappa);
     float m0, m1;
     D.get(m0, m1);
-    r0 = __fmul_rn(g0, g0) / m0;
-    r1 = __fmul_rn(g1, g1) / m1;
+    // (0, not 0 / 0, where the doses agree and dD^2 underflows)
+    r0 = g0 != 0.f ? __fmul_rn(g0, g0) / m0 : 0.f;
+    r1 = g1 != 0.f ? __fmul_rn(g1, g1) / m1 : 0.f;
 }
 
 }  // namespace gk
