@@ -450,8 +450,9 @@ struct BatchState {
         unsigned* items_v = nullptr;
         unsigned short* items_p = nullptr;
         unsigned* items_s = nullptr;
+        uint2* blocks = nullptr;           // the blocks of the passes over the queues (BatchDesc::blocks)
         unsigned* head = nullptr;          // walk, shell tiles, seed rows, seeding work,
-                                           // warp-evaluated walk parts (3), its fix count
+                                           // warp-evaluated walk parts (4), its fix count
         float4* metric4 = nullptr;         // per pair: metric constants of the warp-evaluated walk
         unsigned* fix_v = nullptr;         // warp-evaluated walk: voxels for its finishing pass
         unsigned short* fix_p = nullptr;
@@ -483,6 +484,7 @@ void free_group(BatchState::Group& g)
     cudaFree(g.items_v);
     cudaFree(g.items_p);
     cudaFree(g.items_s);
+    cudaFree(g.blocks);
     cudaFree(g.head);
     cudaFree(g.fix_v);
     cudaFree(g.metric4);
@@ -564,6 +566,14 @@ int batch_upload(gamma_ctx* h)
             CK(cudaMalloc(&G.head, 12 * sizeof(unsigned)));
             CK(cudaMemset(G.head, 0, 12 * sizeof(unsigned)));
             CK(cudaMalloc(&G.desc, sizeof(gk::BatchDesc)));
+            std::vector<uint2> blocks;
+            for (int k = 0; k < np; ++k) {
+                const unsigned n = gk::queue_blocks(b->pairs[mem[k]]->nvox, gk::device_sm_count());
+                for (unsigned i = 0; i < n; ++i) blocks.push_back(make_uint2((unsigned)k, i | n << 16));
+            }
+            CK(cudaMalloc(&G.blocks, sizeof(uint2) * blocks.size()));
+            CK(cudaMemcpy(G.blocks, blocks.data(), sizeof(uint2) * blocks.size(), cudaMemcpyHostToDevice));
+            G.host.nblocks = (unsigned)blocks.size();
         }
         if (h->model && !G.seed_item) {
             size_t cap = 0;
@@ -596,6 +606,7 @@ int batch_upload(gamma_ctx* h)
         d.items_v = G.items_v;
         d.items_p = G.items_p;
         d.items_s = G.items_s;
+        d.blocks = G.blocks;
         d.head = G.head;
         d.shell_next = G.head + 1;
         d.group_bucket = h->walk == 3 ? h->group_bucket : 0;

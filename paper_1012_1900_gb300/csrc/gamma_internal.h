@@ -240,6 +240,9 @@ struct BatchDesc {
     unsigned* items_v;             // [sum of tail_cap] queued voxels in that order
     unsigned short* items_p;       // [sum of tail_cap] their pair
     unsigned* items_s;             // [sum of tail_cap] the cell of their plane seed
+    // the blocks of the passes over the pairs' queues: each block's pair (x), and
+    // which of how many blocks of that pair it is (y: bits 0-15, bits 16-31)
+    const uint2* blocks;           // [BatchGroup::nblocks]
     unsigned* head;                // work counter of the group's table walk
     // warp-evaluated walk: cost buckets from which the queued voxels walk 4,
     // 8 and 32 lanes each (the queue's parts, costliest first; all 0 keeps one
@@ -267,12 +270,24 @@ struct BatchDesc {
     unsigned seed_cap;             // rows past it go unseeded
 };
 
+// Blocks of 256 threads that the passes over a batched pair's queue take: one per
+// 256 voxels of the pair (its queue is at most that long), up to four per SM.  As
+// many for every pair as the largest needs are blocks without work in uneven
+// batches: 200 volumes of 8^3 voxels beside one of 160x160x120 take 306 us so,
+// 594 us with them.
+inline unsigned queue_blocks(long long nvox, int sms)
+{
+    const long long n = (nvox + 255) / 256;
+    return (unsigned)(n < 1 ? 1 : (n > 4ll * sms ? 4ll * sms : n));
+}
+
 // Host view of one batched launch group.
 struct BatchGroup {
     int ndim;
     int npairs;
     long long max_nvox;            // largest pair, for the prepare grid
     int total_tiles;               // shell tiles over all pairs
+    unsigned nblocks;              // entries of the descriptor's blocks
     const BatchDesc* desc;         // device copy of the descriptor
     unsigned* shell_next;          // device: the descriptor's shell tile counter
     // learned seeding (seed_cap 0: no model): the descriptor's row buffers and

@@ -1076,17 +1076,18 @@ __global__ void __launch_bounds__(256) k_bucket_scan_batch(const BatchDesc* __re
     }
 }
 
-// Scatter one pair (blockIdx.y) of a batch group into the group order: per
-// chunk of 256 queued voxels one atomic per cost bucket on the pair's cursor
-// (as k_scatter), not one per voxel.
+// Scatter the pairs of a batch group into the group order (the block's pair:
+// BatchDesc::blocks): per chunk of 256 queued voxels one atomic per cost bucket
+// on the pair's cursor (as k_scatter), not one per voxel.
 __global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restrict__ bd)
 {
     __shared__ unsigned cnt[kNumBuckets], base[kNumBuckets];
     grid_release();
     grid_wait();
-    const Problem& P = bd->probs[blockIdx.y];
+    const uint2 blk = bd->blocks[blockIdx.x];
+    const Problem& P = bd->probs[blk.x];
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
-    for (unsigned c0 = blockIdx.x * blockDim.x; c0 < total; c0 += gridDim.x * blockDim.x) {
+    for (unsigned c0 = (blk.y & 0xffffu) * 256u; c0 < total; c0 += (blk.y >> 16) * 256u) {
         if (threadIdx.x < kNumBuckets) cnt[threadIdx.x] = 0;
         __syncthreads();
         const unsigned i = c0 + threadIdx.x;
@@ -1103,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restri
         if (b >= 0) {
             const unsigned pos = base[b] + rank;
             bd->items_v[pos] = P.tail_raw[i];
-            bd->items_p[pos] = (unsigned short)blockIdx.y;
+            bd->items_p[pos] = (unsigned short)blk.x;
             if (P.plane_raw) bd->items_s[pos] = P.plane_raw[i];
         }
         __syncthreads();
@@ -1350,16 +1351,25 @@ __global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH)
     __shared__ unsigned sh_hist[kNumBuckets];
     grid_release();
     grid_wait();
-    const Problem& P = BATCH ? bd->probs[blockIdx.y] : P0;
+    // this block's first item, and the items from one turn of the pair's blocks to the next
+    unsigned first = blockIdx.x * blockDim.x, step = gridDim.x * blockDim.x, pr = 0;
+    if constexpr (BATCH) {
+        constexpr unsigned kSub = 256u / seed_threads(N, true);
+        const uint2 blk = bd->blocks[blockIdx.x / kSub];
+        pr = blk.x;
+        first = (blk.y & 0xffffu) * 256u + blockIdx.x % kSub * blockDim.x;
+        step = (blk.y >> 16) * 256u;
+    }
+    const Problem& P = BATCH ? bd->probs[pr] : P0;
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
-    if (blockIdx.x * blockDim.x >= total) return;             // block-uniform
+    if (first >= total) return;                               // block-uniform
     if (threadIdx.x < kNumBuckets) sh_hist[threadIdx.x] = 0;
     __syncthreads();
     const float dnorm = resolve_dnorm(P);
     const float hn2[3] = {P.mt.hn2[0], P.mt.hn2[1], P.mt.hn2[2]};
     const float kap[3] = {P.mt.kappa[1], P.mt.kappa[2], P.mt.kappa[4]};
     const int nx = P.nx, ny = P.ny, nz = P.nz, sz = nx * ny;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    for (unsigned i = first + threadIdx.x; i < total; i += step) {
         const unsigned v = P.tail_raw[i];
         const int x = (int)(v % (unsigned)nx);
         const unsigned r1 = v / (unsigned)nx;
@@ -2983,7 +2993,7 @@ cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s)
     if (g.npairs <= 0) return cudaSuccess;
     Problem dummy{};
     const int t = seed_threads(g.ndim, true);
-    const dim3 grid((unsigned)grid_for(g.max_nvox, t, device_sm_count() * (1024 / t)), (unsigned)g.npairs);
+    const unsigned grid = g.nblocks * (256u / (unsigned)t);
     if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, t, 0, s, dummy, g.desc);
     else launch_next(k_plane_seed<2, true>, grid, t, 0, s, dummy, g.desc);
     return cudaGetLastError();
@@ -2993,10 +3003,7 @@ cudaError_t launch_batch_order(const BatchGroup& g, cudaStream_t s)
 {
     if (g.npairs <= 0) return cudaSuccess;
     launch_next(k_bucket_scan_batch, 1, 256, 0, s, g.desc);
-    // enough blocks per pair for the largest queue (one 256-voxel chunk per
-    // block and pass); the blocks of small pairs leave at once
-    const int sms = device_sm_count();
-    launch_next(k_scatter_batch, dim3(sms * 4, g.npairs), 256, 0, s, g.desc);
+    launch_next(k_scatter_batch, g.nblocks, 256, 0, s, g.desc);
     return cudaGetLastError();
 }
 
