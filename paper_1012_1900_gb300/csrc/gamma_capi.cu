@@ -450,7 +450,7 @@ struct BatchState {
         unsigned* items_v = nullptr;
         unsigned short* items_p = nullptr;
         unsigned* items_s = nullptr;
-        uint2* blocks = nullptr;           // the blocks of the passes over the queues (BatchDesc::blocks)
+        gk::QueueBlock* blocks = nullptr;           // the blocks of the passes over the queues (BatchGroup::blocks)
         unsigned* head = nullptr;          // walk, shell tiles, seed rows, seeding work,
                                            // warp-evaluated walk parts (4), its fix count
         float4* metric4 = nullptr;         // per pair: metric constants of the warp-evaluated walk
@@ -566,13 +566,14 @@ int batch_upload(gamma_ctx* h)
             CK(cudaMalloc(&G.head, 12 * sizeof(unsigned)));
             CK(cudaMemset(G.head, 0, 12 * sizeof(unsigned)));
             CK(cudaMalloc(&G.desc, sizeof(gk::BatchDesc)));
-            std::vector<uint2> blocks;
+            std::vector<gk::QueueBlock> blocks;
             for (int k = 0; k < np; ++k) {
                 const unsigned n = gk::queue_blocks(b->pairs[mem[k]]->nvox, gk::device_sm_count());
-                for (unsigned i = 0; i < n; ++i) blocks.push_back(make_uint2((unsigned)k, i | n << 16));
+                for (unsigned i = 0; i < n; ++i) blocks.push_back({b->ctrs + mem[k], (unsigned)k, i | n << 16});
             }
-            CK(cudaMalloc(&G.blocks, sizeof(uint2) * blocks.size()));
-            CK(cudaMemcpy(G.blocks, blocks.data(), sizeof(uint2) * blocks.size(), cudaMemcpyHostToDevice));
+            CK(cudaMalloc(&G.blocks, sizeof(gk::QueueBlock) * blocks.size()));
+            CK(cudaMemcpy(G.blocks, blocks.data(), sizeof(gk::QueueBlock) * blocks.size(), cudaMemcpyHostToDevice));
+            G.host.blocks = G.blocks;
             G.host.nblocks = (unsigned)blocks.size();
         }
         if (h->model && !G.seed_item) {
@@ -606,7 +607,6 @@ int batch_upload(gamma_ctx* h)
         d.items_v = G.items_v;
         d.items_p = G.items_p;
         d.items_s = G.items_s;
-        d.blocks = G.blocks;
         d.head = G.head;
         d.shell_next = G.head + 1;
         d.group_bucket = h->walk == 3 ? h->group_bucket : 0;

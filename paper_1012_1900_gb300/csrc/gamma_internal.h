@@ -74,8 +74,9 @@ __host__ __device__ inline uint32_t pack10(int x, int y, int z)
     return (uint32_t(x) & 1023u) | ((uint32_t(y) & 1023u) << 10) | ((uint32_t(z) & 1023u) << 20);
 }
 
-// Device-side counters; zeroed at the start of every run.
-struct Counters {
+// Device-side counters; zeroed at the start of every run.  Whole cache lines, so
+// that the counters of a batch's pairs share none.
+struct alignas(128) Counters {
     unsigned long long n_eval;
     unsigned long long n_pass;
     unsigned long long cells_visited;   // stats mode: cells whose faces were evaluated
@@ -240,9 +241,6 @@ struct BatchDesc {
     unsigned* items_v;             // [sum of tail_cap] queued voxels in that order
     unsigned short* items_p;       // [sum of tail_cap] their pair
     unsigned* items_s;             // [sum of tail_cap] the cell of their plane seed
-    // the blocks of the passes over the pairs' queues: each block's pair (x), and
-    // which of how many blocks of that pair it is (y: bits 0-15, bits 16-31)
-    const uint2* blocks;           // [BatchGroup::nblocks]
     unsigned* head;                // work counter of the group's table walk
     // warp-evaluated walk: cost buckets from which the queued voxels walk 4,
     // 8 and 32 lanes each (the queue's parts, costliest first; all 0 keeps one
@@ -273,7 +271,7 @@ struct BatchDesc {
 // Blocks of 256 threads that the passes over a batched pair's queue take: one per
 // 256 voxels of the pair (its queue is at most that long), up to four per SM.  As
 // many for every pair as the largest needs are blocks without work in uneven
-// batches: 200 volumes of 8^3 voxels beside one of 160x160x120 take 306 us so,
+// batches: 200 volumes of 8^3 voxels beside one of 160x160x120 take 238 us so,
 // 594 us with them.
 inline unsigned queue_blocks(long long nvox, int sms)
 {
@@ -281,13 +279,22 @@ inline unsigned queue_blocks(long long nvox, int sms)
     return (unsigned)(n < 1 ? 1 : (n > 4ll * sms ? 4ll * sms : n));
 }
 
+// One of them: its pair, that pair's counters (most blocks find the queue too
+// short to have work, and so leave after two loads), and which of how many blocks
+// of the pair it is (bits 0-15, bits 16-31).
+struct alignas(16) QueueBlock {
+    const Counters* ctr;
+    unsigned pair, share;
+};
+
 // Host view of one batched launch group.
 struct BatchGroup {
     int ndim;
     int npairs;
     long long max_nvox;            // largest pair, for the prepare grid
     int total_tiles;               // shell tiles over all pairs
-    unsigned nblocks;              // entries of the descriptor's blocks
+    const QueueBlock* blocks;      // device: the blocks of the passes over the pairs' queues
+    unsigned nblocks;
     const BatchDesc* desc;         // device copy of the descriptor
     unsigned* shell_next;          // device: the descriptor's shell tile counter
     // learned seeding (seed_cap 0: no model): the descriptor's row buffers and

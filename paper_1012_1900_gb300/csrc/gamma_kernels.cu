@@ -1077,17 +1077,20 @@ __global__ void __launch_bounds__(256) k_bucket_scan_batch(const BatchDesc* __re
 }
 
 // Scatter the pairs of a batch group into the group order (the block's pair:
-// BatchDesc::blocks): per chunk of 256 queued voxels one atomic per cost bucket
+// BatchGroup::blocks): per chunk of 256 queued voxels one atomic per cost bucket
 // on the pair's cursor (as k_scatter), not one per voxel.
-__global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restrict__ bd)
+__global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restrict__ bd,
+                                                       const QueueBlock* __restrict__ blocks)
 {
     __shared__ unsigned cnt[kNumBuckets], base[kNumBuckets];
     grid_release();
     grid_wait();
-    const uint2 blk = bd->blocks[blockIdx.x];
-    const Problem& P = bd->probs[blk.x];
+    const QueueBlock blk = blocks[blockIdx.x];
+    const unsigned first = (blk.share & 0xffffu) * 256u;
+    if (first >= blk.ctr->tail_count) return;                 // block-uniform
+    const Problem& P = bd->probs[blk.pair];
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
-    for (unsigned c0 = (blk.y & 0xffffu) * 256u; c0 < total; c0 += (blk.y >> 16) * 256u) {
+    for (unsigned c0 = first; c0 < total; c0 += (blk.share >> 16) * 256u) {
         if (threadIdx.x < kNumBuckets) cnt[threadIdx.x] = 0;
         __syncthreads();
         const unsigned i = c0 + threadIdx.x;
@@ -1104,7 +1107,7 @@ __global__ void __launch_bounds__(256) k_scatter_batch(const BatchDesc* __restri
         if (b >= 0) {
             const unsigned pos = base[b] + rank;
             bd->items_v[pos] = P.tail_raw[i];
-            bd->items_p[pos] = (unsigned short)blk.x;
+            bd->items_p[pos] = (unsigned short)blk.pair;
             if (P.plane_raw) bd->items_s[pos] = P.plane_raw[i];
         }
         __syncthreads();
@@ -1346,7 +1349,8 @@ __host__ __device__ constexpr int seed_threads(int n, bool batch) { return n == 
 
 template <int N, bool BATCH>
 __global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH) == 128 ? 8 : 0)
-    k_plane_seed(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd)
+    k_plane_seed(const __grid_constant__ Problem P0, const BatchDesc* __restrict__ bd,
+                 const QueueBlock* __restrict__ blocks)
 {
     __shared__ unsigned sh_hist[kNumBuckets];
     grid_release();
@@ -1355,10 +1359,11 @@ __global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH)
     unsigned first = blockIdx.x * blockDim.x, step = gridDim.x * blockDim.x, pr = 0;
     if constexpr (BATCH) {
         constexpr unsigned kSub = 256u / seed_threads(N, true);
-        const uint2 blk = bd->blocks[blockIdx.x / kSub];
-        pr = blk.x;
-        first = (blk.y & 0xffffu) * 256u + blockIdx.x % kSub * blockDim.x;
-        step = (blk.y >> 16) * 256u;
+        const QueueBlock blk = blocks[blockIdx.x / kSub];
+        pr = blk.pair;
+        first = (blk.share & 0xffffu) * 256u + blockIdx.x % kSub * blockDim.x;
+        step = (blk.share >> 16) * 256u;
+        if (first >= blk.ctr->tail_count) return;             // block-uniform
     }
     const Problem& P = BATCH ? bd->probs[pr] : P0;
     const unsigned total = min(P.ctr->tail_count, P.tail_cap);
@@ -2816,8 +2821,8 @@ cudaError_t launch_plane_seed(const Problem& P, cudaStream_t s)
 {
     if (!P.plane_raw) return cudaSuccess;
     const int t = seed_threads(P.ndim, false), grid = grid_for(P.nvox, t, device_sm_count() * 8);
-    if (P.ndim == 3) launch_next(k_plane_seed<3, false>, grid, t, 0, s, P, nullptr);
-    else launch_next(k_plane_seed<2, false>, grid, t, 0, s, P, nullptr);
+    if (P.ndim == 3) launch_next(k_plane_seed<3, false>, grid, t, 0, s, P, nullptr, nullptr);
+    else launch_next(k_plane_seed<2, false>, grid, t, 0, s, P, nullptr, nullptr);
     return cudaGetLastError();
 }
 
@@ -2994,8 +2999,8 @@ cudaError_t launch_batch_plane_seed(const BatchGroup& g, cudaStream_t s)
     Problem dummy{};
     const int t = seed_threads(g.ndim, true);
     const unsigned grid = g.nblocks * (256u / (unsigned)t);
-    if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, t, 0, s, dummy, g.desc);
-    else launch_next(k_plane_seed<2, true>, grid, t, 0, s, dummy, g.desc);
+    if (g.ndim == 3) launch_next(k_plane_seed<3, true>, grid, t, 0, s, dummy, g.desc, g.blocks);
+    else launch_next(k_plane_seed<2, true>, grid, t, 0, s, dummy, g.desc, g.blocks);
     return cudaGetLastError();
 }
 
@@ -3003,7 +3008,7 @@ cudaError_t launch_batch_order(const BatchGroup& g, cudaStream_t s)
 {
     if (g.npairs <= 0) return cudaSuccess;
     launch_next(k_bucket_scan_batch, 1, 256, 0, s, g.desc);
-    launch_next(k_scatter_batch, g.nblocks, 256, 0, s, g.desc);
+    launch_next(k_scatter_batch, g.nblocks, 256, 0, s, g.desc, g.blocks);
     return cudaGetLastError();
 }
 
