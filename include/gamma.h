@@ -134,6 +134,10 @@ typedef struct {
  *  shape        (nz, ny, nx); nz = 1 for 2D.  nz*ny*nx < 2^31.
  *  spacing_mm   (hz, hy, hx) voxel size in mm, > 0 (hz ignored for 2D).
  *  crit         criteria (copied).
+ * Scratch: 13 bytes per voxel, and 16 more where the device has them, for the
+ * walk's starting bounds (8; without them the default walk takes the form of
+ * "walk" 0) and the cells' dose ranges (8; without them it reads the doses).
+ * The maps do not depend on it.
  * Errors: INVALID_ARG, SHAPE, OOM, TABLE_TOO_LARGE, CUDA.  Synchronous. */
 int gamma_create(gamma_handle *out, const float *ref_dev, const float *eval_dev, int ndim,
                  const int64_t shape[3], const float spacing_mm[3], const gamma_criteria *crit);
@@ -289,6 +293,9 @@ int gamma_get_timings(gamma_handle h, gamma_timings *out);
  *  "drop_slab_flag"   failure test: k + 1 leaves slab k's readiness flag
  *                     unwritten in overlapped runs, so that the gated shell's
  *                     bounded wait gives up (GAMMA_ERR_TIMEOUT); 0 (default)
+ *  "drop_lists"       failure test: run as a handle whose optional scratch
+ *                     found no room, 1 the dose ranges, 2 the starting bounds
+ *                     too; 0 (default)
  *  "face_eval"        design 1 / 2 only: 0 every face in closed form (the
  *                     paper's choice, Section 2.2); 1 the full simplices by
  *                     Ju's recursion (Section 2.1)
@@ -326,8 +333,9 @@ typedef struct {
 } gamma_pair_desc;
 
 /* Create a batch handle over 1 <= n_pairs <= 65535 descriptors (copied;
- * device buffers borrowed).  Each pair gets its own cell table and scratch;
- * the handle adds 10 bytes per voxel of all pairs for the shared work order.
+ * device buffers borrowed).  Each pair gets its own cell table and 9 bytes of
+ * scratch per voxel; the handle adds 16 per voxel of all pairs for the shared
+ * work order and finishing list.
  * Errors: INVALID_ARG, SHAPE, OOM, TABLE_TOO_LARGE, CUDA.  Synchronous. */
 int gamma_batch_create(gamma_handle *out, int n_pairs, const gamma_pair_desc *pairs);
 

@@ -124,10 +124,12 @@ struct gamma_ctx {
     unsigned long long* row_sorted = nullptr;
     // warp-evaluated walk: voxels left to its finishing pass (tail_cap entries)
     unsigned* fix_list = nullptr;
-    unsigned* plane_raw = nullptr;    // ... the cells of the plane seeds (tail_cap entries each, allocated
-                                      //     with fix_list)
-    unsigned* plane_sorted = nullptr;
-    float2* range = nullptr;          // ... dose range of every cell (written when the queue is worth it)
+    float2* range = nullptr;          // ... dose range of every cell, written when the queue is worth it
+                                      //     (null without room: the walk takes it from the doses)
+    unsigned* plane_raw = nullptr;    // ... the cells of the plane seeds, tail_cap entries each, behind
+    unsigned* plane_sorted = nullptr; //     the ranges or in plane_own (null without room: lane walk)
+    unsigned* plane_own = nullptr;
+    int drop_lists = 0;               // test hook: run as if those two had found no room
     int group_bucket = 9;             // ... queued voxels of this cost bucket and above walk 4 lanes each
                                       //     (< 0: the walk chooses the parts from the queue)
     int group_auto_pct = 100;         // ... with this slack (percent)
@@ -344,10 +346,10 @@ Problem make_problem(const gamma_ctx* h, float* out)
     P.seed_Y = h->seed_Y;
     P.seed_cap = h->seed_cap;
     P.fix_list = h->fix_list;
-    if (h->walk == 3) {
+    if (h->walk == 3 && h->drop_lists < 2) {
         P.plane_raw = h->plane_raw;
         P.plane_sorted = h->plane_sorted;
-        P.range = h->range;
+        if (h->drop_lists < 1) P.range = h->range;
     }
     P.cq_group_bucket = h->group_bucket;
     P.cq_group8_bucket = h->group8_bucket;
@@ -404,6 +406,7 @@ void free_ctx(gamma_ctx* h)
     cudaFree(h->row_bkt);
     cudaFree(h->row_sorted);
     cudaFree(h->fix_list);
+    cudaFree(h->plane_own);
     cudaFree(h->range);
     cudaFree(h->seed_list);
     cudaFree(h->seed_X);
@@ -728,8 +731,15 @@ Counters sum_counters(const std::vector<Counters>& cs)
 
 extern "C" {
 
-int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev, int ndim,
-                 const int64_t shape[3], const float spacing_mm[3], const gamma_criteria* crit)
+// A handle of one pair (batched: a pair of a batch handle, which has the group's
+// lists for the walk and its counters in the group's array).  Scratch per voxel:
+// the queue and its cost buckets, 5 bytes; the ordered queue and the finishing
+// list, 8; then, last, since a handle works without them, the cells of the plane
+// seeds, 8, and the cells' dose ranges, 8.  A pair of a batch has the queue, its
+// buckets and the seeds' cells: 9.
+static int create_pair(gamma_handle* out, const float* ref_dev, const float* eval_dev, int ndim,
+                       const int64_t shape[3], const float spacing_mm[3], const gamma_criteria* crit,
+                       bool batched)
 {
     if (!out || !shape || !spacing_mm) return GAMMA_ERR_INVALID_ARG;
     *out = nullptr;
@@ -760,28 +770,25 @@ int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev,
     auto fail = [&](int code) { free_ctx(h); return code; };
     if ((rc = build_table(h)) != GAMMA_OK) return fail(rc);
     cudaError_t e;
+    const int tiles = gk::block_tiles(make_problem(h, nullptr));
+    if (tiles < 0) return fail(GAMMA_ERR_SHAPE);
+    h->tail_cap = (unsigned)nvox;
+    if ((e = cudaMalloc(&h->tail_raw, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
+    if ((e = cudaMalloc(&h->tail_bucket, nvox)) != cudaSuccess) return fail(cuda_fail(e));
+    if (batched) {
+        if ((e = cudaMalloc(&h->plane_own, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
+        h->plane_raw = h->plane_own;
+        *out = h;
+        return GAMMA_OK;
+    }
     for (auto& te : h->tev)
         if ((e = cudaEventCreate(&te)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = cudaMalloc(&h->ctr, sizeof(Counters))) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = cudaStreamCreateWithFlags(&h->sg_cap, cudaStreamNonBlocking)) != cudaSuccess)
         return fail(cuda_fail(e));
-    h->tail_cap = (unsigned)nvox;
-    if ((e = cudaMalloc(&h->tail_raw, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
     if ((e = cudaMalloc(&h->tail_sorted, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
-    if ((e = cudaMalloc(&h->tail_bucket, nvox)) != cudaSuccess) return fail(cuda_fail(e));
-    // one allocation for the three lists of the warp-evaluated walk
-    if ((e = cudaMalloc(&h->fix_list, 3 * sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
-    h->plane_raw = h->fix_list + nvox;
-    h->plane_sorted = h->plane_raw + nvox;
-    // only a gain: without room for it the walk takes the ranges from the doses
-    if (cudaMalloc(&h->range, sizeof(float2) * nvox) != cudaSuccess) {
-        cudaGetLastError();
-        h->range = nullptr;
-    }
+    if ((e = cudaMalloc(&h->fix_list, sizeof(unsigned) * nvox)) != cudaSuccess) return fail(cuda_fail(e));
     {
-        Problem P0 = make_problem(h, nullptr);
-        const int tiles = gk::block_tiles(P0);
-        if (tiles < 0) return fail(GAMMA_ERR_SHAPE);
         const size_t nt = (size_t)std::max(tiles, 1);
         if ((e = cudaMalloc(&h->tile_mask, sizeof(unsigned) * 8 * nt)) != cudaSuccess ||
             (e = cudaMalloc(&h->tile_list, sizeof(unsigned) * nt)) != cudaSuccess ||
@@ -799,8 +806,25 @@ int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev,
         h->ref = h->own_ref;
         h->ev = h->own_ev;
     }
+    // only gains, so after everything that the handle must have: the ranges, then
+    // the lists, in one allocation, or the lists alone
+    if (cudaMalloc(&h->range, (sizeof(float2) + 2 * sizeof(unsigned)) * nvox) == cudaSuccess) {
+        h->plane_raw = (unsigned*)(h->range + nvox);
+    } else {
+        h->range = nullptr;
+        if (cudaMalloc(&h->plane_own, 2 * sizeof(unsigned) * nvox) != cudaSuccess) h->plane_own = nullptr;
+        h->plane_raw = h->plane_own;
+    }
+    if (h->plane_raw) h->plane_sorted = h->plane_raw + nvox;
+    cudaGetLastError();
     *out = h;
     return GAMMA_OK;
+}
+
+int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev, int ndim,
+                 const int64_t shape[3], const float spacing_mm[3], const gamma_criteria* crit)
+{
+    return create_pair(out, ref_dev, eval_dev, ndim, shape, spacing_mm, crit, false);
 }
 
 // The nine cell tables of a two-grid handle (variants of gk::build_grid_table,
@@ -958,7 +982,7 @@ static int enqueue_walk(gamma_handle h, const Problem& P, cudaStream_t s, bool t
     } else {
         CK(gk::launch_order_tail(P, s));
         if (tm) CK(cudaEventRecord(h->tev[4], s));
-        if (h->walk == 3) CK(gk::launch_tail_cq(P, h->tail_minblocks, s));
+        if (P.plane_raw) CK(gk::launch_tail_cq(P, h->tail_minblocks, s));
         else CK(gk::launch_tail(P, h->lanes, h->tail_minblocks, s));
     }
     return GAMMA_OK;
@@ -1492,6 +1516,11 @@ int gamma_set_option(gamma_handle h, const char* key, int64_t value)
         h->drop_slab_flag = (int)value;
         return GAMMA_OK;
     }
+    if (!std::strcmp(key, "drop_lists")) {
+        if (h->batch || value < 0 || value > 2) return GAMMA_ERR_INVALID_ARG;
+        h->drop_lists = (int)value;
+        return GAMMA_OK;
+    }
     if (!std::strcmp(key, "face_eval")) {
         if (h->batch || value < 0 || value > 1) return GAMMA_ERR_INVALID_ARG;
         h->face_eval = (int)value;
@@ -1556,10 +1585,9 @@ int gamma_batch_create(gamma_handle* out, int n_pairs, const gamma_pair_desc* pa
         const gamma_pair_desc& d = pairs[i];
         if (!d.ref_dev || !d.eval_dev || !d.gamma_out_dev) return fail(GAMMA_ERR_INVALID_ARG);
         gamma_ctx* c = nullptr;
-        if (int rc = gamma_create(&c, d.ref_dev, d.eval_dev, d.ndim, d.shape, d.spacing_mm, &d.crit))
+        if (int rc = create_pair(&c, d.ref_dev, d.eval_dev, d.ndim, d.shape, d.spacing_mm, &d.crit, true))
             return fail(rc);
-        cudaFree(c->ctr);                        // counters live in one shared array
-        c->ctr = b->ctrs + i;
+        c->ctr = b->ctrs + i;                    // counters live in one shared array
         b->pairs[i] = c;
         b->outs[i] = d.gamma_out_dev;
         b->members[d.ndim == 2 ? 0 : 1].push_back(i);
