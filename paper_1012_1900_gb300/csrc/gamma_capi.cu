@@ -192,14 +192,14 @@ namespace {
 // lower-corner offset c whose cell can hold faces for some voxel, keyed by the
 // distance from the reference voxel to the closed cell box [c, c + 1] divided
 // by the DTA (for the key-0 cells: to their faces off the voxel), sorted
-// ascending (ties by z, y, x), cut to `cap` entries.
-int build_table(gamma_ctx* h)
+// ascending (ties by z, y, x), cut to `cap` entries.  The handle keeps the table
+// that it has until the new one is complete on the device.
+int build_table(gamma_ctx* h, int64_t cap) try
 {
     const double dta = h->crit.dta_mm;
     const double hn[3] = {h->h[0] / dta, h->h[1] / dta, h->h[2] / dta};
     const int nd = h->ndim;
     const int64_t n[3] = {h->nx, h->ny, h->nz};
-    const int64_t cap = h->table_cap;
     if (cap < (1 << nd)) return GAMMA_ERR_INVALID_ARG;
     // radius from a ball-volume estimate of about 2 * cap cells
     double cellvol = hn[0] * hn[1] * (nd == 3 ? hn[2] : 1.0);
@@ -222,7 +222,7 @@ int build_table(gamma_ctx* h)
     }
     double far[8];
     gk::key0_far(hn, nd, far);
-    for (int s = 0; s < 8; ++s) {
+    for (int s = 0; s < 8; ++s) {            // (of the spacing alone: the same for every cap)
         const double f2 = far[s] * far[s];
         float r = (float)f2;
         if ((double)r > f2) r = std::nextafterf(r, -INFINITY);
@@ -230,19 +230,15 @@ int build_table(gamma_ctx* h)
     }
     struct Tmp { double key; int x, y, z; };
     std::vector<Tmp> all;
-    try {
-        for (int64_t z = lo[2]; z <= hi[2]; ++z)
-            for (int64_t y = lo[1]; y <= hi[1]; ++y)
-                for (int64_t x = lo[0]; x <= hi[0]; ++x) {
-                    double ax = axis_gap((int)x) * hn[0], ay = axis_gap((int)y) * hn[1];
-                    double az = nd == 3 ? axis_gap((int)z) * hn[2] : 0.0;
-                    double key = std::sqrt(ax * ax + ay * ay + az * az);
-                    if (key == 0.0) key = far[(x & 1) | ((y & 1) << 1) | ((z & 1) << 2)];
-                    if (key < R) all.push_back({key, (int)x, (int)y, (int)z});
-                }
-    } catch (const std::bad_alloc&) {
-        return GAMMA_ERR_OOM;
-    }
+    for (int64_t z = lo[2]; z <= hi[2]; ++z)
+        for (int64_t y = lo[1]; y <= hi[1]; ++y)
+            for (int64_t x = lo[0]; x <= hi[0]; ++x) {
+                double ax = axis_gap((int)x) * hn[0], ay = axis_gap((int)y) * hn[1];
+                double az = nd == 3 ? axis_gap((int)z) * hn[2] : 0.0;
+                double key = std::sqrt(ax * ax + ay * ay + az * az);
+                if (key == 0.0) key = far[(x & 1) | ((y & 1) << 1) | ((z & 1) << 2)];
+                if (key < R) all.push_back({key, (int)x, (int)y, (int)z});
+            }
     std::sort(all.begin(), all.end(), [](const Tmp& a, const Tmp& b) {
         if (a.key != b.key) return a.key < b.key;
         if (a.z != b.z) return a.z < b.z;
@@ -260,37 +256,40 @@ int build_table(gamma_ctx* h)
         keep = (size_t)cap;
         cover = std::min(cover, all[keep].key);
     }
-    h->table.resize(keep);
+    std::vector<TableEntry> table(keep);
     for (size_t i = 0; i < keep; ++i) {
-        h->table[i].off = gk::pack10(all[i].x, all[i].y, all[i].z);
-        h->table[i].key = round_down(all[i].key);
+        table[i].off = gk::pack10(all[i].x, all[i].y, all[i].z);
+        table[i].key = round_down(all[i].key);
     }
-    h->r_cover = cover;
     // both forms of the table in one buffer and one copy: the walk's entries
     // (16-byte aligned), then the plain ones
     const size_t nwalk = keep + gk::kWalkPad, wbytes = nwalk * sizeof(gk::WalkEntry);
-    std::vector<gk::WalkEntry> walk;
-    try {
-        walk.resize(nwalk + (keep * sizeof(TableEntry) + sizeof(gk::WalkEntry) - 1) / sizeof(gk::WalkEntry),
-                    gk::WalkEntry{INFINITY, 0, 0u, 0});
-    } catch (const std::bad_alloc&) {
-        return GAMMA_ERR_OOM;
-    }
+    std::vector<gk::WalkEntry> walk(nwalk + (keep * sizeof(TableEntry) + sizeof(gk::WalkEntry) - 1) /
+                                                sizeof(gk::WalkEntry), gk::WalkEntry{INFINITY, 0, 0u, 0});
     int margin = 0;
     for (size_t i = 0; i < keep; ++i) {
         const int c[3] = {all[i].x, all[i].y, all[i].z};
         for (int a = 0; a < nd; ++a) margin = std::max(margin, std::max(-c[a], c[a] + 1));
         const int64_t lin = c[0] + (int64_t)c[1] * h->nx + (int64_t)c[2] * h->nx * h->ny;
-        walk[i] = gk::WalkEntry{h->table[i].key * h->table[i].key, (int)lin, h->table[i].off, margin};
+        walk[i] = gk::WalkEntry{table[i].key * table[i].key, (int)lin, table[i].off, margin};
     }
-    if (keep) std::memcpy((char*)walk.data() + wbytes, h->table.data(), keep * sizeof(TableEntry));
+    if (keep) std::memcpy((char*)walk.data() + wbytes, table.data(), keep * sizeof(TableEntry));
+    gk::WalkEntry* dev = nullptr;
+    CK(cudaMalloc(&dev, walk.size() * sizeof(gk::WalkEntry)));
+    const cudaError_t e = cudaMemcpy(dev, walk.data(), walk.size() * sizeof(gk::WalkEntry), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaFree(dev);
+        return cuda_fail(e);
+    }
     cudaFree(h->walk_dev);
-    h->walk_dev = nullptr;
-    h->table_dev = nullptr;
-    CK(cudaMalloc(&h->walk_dev, walk.size() * sizeof(gk::WalkEntry)));
-    h->table_dev = (TableEntry*)((char*)h->walk_dev + wbytes);
-    CK(cudaMemcpy(h->walk_dev, walk.data(), walk.size() * sizeof(gk::WalkEntry), cudaMemcpyHostToDevice));
+    h->walk_dev = dev;
+    h->table_dev = (TableEntry*)((char*)dev + wbytes);
+    h->table.swap(table);
+    h->r_cover = cover;
+    h->table_cap = cap;
     return GAMMA_OK;
+} catch (const std::bad_alloc&) {
+    return GAMMA_ERR_OOM;
 }
 
 Problem make_problem(const gamma_ctx* h, float* out)
@@ -524,7 +523,7 @@ namespace {
 
 // (Re)build every pair's Problem with the batch handle's options and upload
 // the per-group descriptors.
-int batch_upload(gamma_ctx* h)
+int batch_upload(gamma_ctx* h) try
 {
     BatchState* b = h->batch;
     for (int gi = 0; gi < 2; ++gi) {
@@ -646,6 +645,8 @@ int batch_upload(gamma_ctx* h)
         G.host.flags = &b->ctrs[mem[0]].flags;
     }
     return GAMMA_OK;
+} catch (const std::bad_alloc&) {
+    return GAMMA_ERR_OOM;
 }
 
 // One group's launches, on stream s.
@@ -768,7 +769,7 @@ static int create_pair(gamma_handle* out, const float* ref_dev, const float* eva
     h->ev = eval_dev;
     int rc = GAMMA_OK;
     auto fail = [&](int code) { free_ctx(h); return code; };
-    if ((rc = build_table(h)) != GAMMA_OK) return fail(rc);
+    if ((rc = build_table(h, h->table_cap)) != GAMMA_OK) return fail(rc);
     cudaError_t e;
     const int tiles = gk::block_tiles(make_problem(h, nullptr));
     if (tiles < 0) return fail(GAMMA_ERR_SHAPE);
@@ -829,7 +830,7 @@ int gamma_create(gamma_handle* out, const float* ref_dev, const float* eval_dev,
 
 // The nine cell tables of a two-grid handle (variants of gk::build_grid_table,
 // each capped at `cap` entries), concatenated in one device array.
-static int upload_grid_tables(gamma_ctx* h, long long cap)
+static int upload_grid_tables(gamma_ctx* h, long long cap) try
 {
     gk::GridProblem& G = h->grids->G;
     const double hn[3] = {G.eh[0], G.eh[1], G.eh[2]};
@@ -864,6 +865,8 @@ static int upload_grid_tables(gamma_ctx* h, long long cap)
         G.tcover[k] = cov[k];
     }
     return GAMMA_OK;
+} catch (const std::bad_alloc&) {
+    return GAMMA_ERR_OOM;
 }
 
 int gamma_create_grids(gamma_handle* out, const float* ref_dev, const float* eval_dev, int ndim,
@@ -1475,8 +1478,7 @@ int gamma_set_option(gamma_handle h, const char* key, int64_t value)
         DeviceGuard dg(h->device);
         if (!dg.ok) return GAMMA_ERR_CUDA;
         if (h->ran) { CK(cudaStreamSynchronize(h->last_stream)); }
-        h->table_cap = value;
-        return build_table(h);
+        return build_table(h, value);
     }
     if (!std::strcmp(key, "fp64_tau_exp10")) {
         if (value > 30) return GAMMA_ERR_INVALID_ARG;
@@ -1577,8 +1579,13 @@ int gamma_batch_create(gamma_handle* out, int n_pairs, const gamma_pair_desc* pa
     for (auto& te : h->tev)
         if ((e = cudaEventCreate(&te)) != cudaSuccess) return fail(cuda_fail(e));
     b->n = n_pairs;
-    b->pairs.assign(n_pairs, nullptr);
-    b->outs.assign(n_pairs, nullptr);
+    try {
+        b->pairs.assign(n_pairs, nullptr);
+        b->outs.assign(n_pairs, nullptr);
+        for (auto& m : b->members) m.reserve(n_pairs);
+    } catch (const std::bad_alloc&) {
+        return fail(GAMMA_ERR_OOM);
+    }
     if ((e = cudaMalloc(&b->ctrs, sizeof(Counters) * n_pairs)) != cudaSuccess)
         return fail(cuda_fail(e));
     for (int i = 0; i < n_pairs; ++i) {
