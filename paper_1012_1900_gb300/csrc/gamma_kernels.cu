@@ -2973,7 +2973,8 @@ cudaError_t launch_batch_prepare(const BatchGroup& g, cudaStream_t s)
     const int sms = device_sm_count();
     const int bx = grid_for(g.max_nvox, 256, std::max(1, sms * 8 / std::max(1, g.npairs)) + 1);
     Problem dummy{};
-    launch_next(k_prepare<true>, dim3(bx, g.npairs), 256, 0, s, dummy, g.desc, 1);   // k_shell checks the evaluation dose
+    // (the run's first kernel: a plain launch; the shell checks the evaluation dose)
+    k_prepare<true><<<dim3(bx, g.npairs), 256, 0, s>>>(dummy, g.desc, 1);
     return cudaGetLastError();
 }
 

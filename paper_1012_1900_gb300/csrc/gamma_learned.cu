@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_rows(const __grid_consta
     unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     TcSmem& S = *reinterpret_cast<TcSmem*>(base);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    grid_release();
+    if (count_dev) grid_release();       // within a run; by itself it is the call's last kernel
     grid_wait();
     const long long nrows = count_dev ? min((long long)*count_dev, M) : M;
     const long long ntiles = (nrows + kRows - 1) / kRows;
