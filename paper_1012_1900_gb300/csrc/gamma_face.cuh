@@ -50,8 +50,10 @@ __host__ __device__ __forceinline__ double fma_(double a, double b, double c) { 
 // one kernel to the next would give the walks other last bits for one cell.
 __device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
-// a / b for b >= 1 (D of a face): one reciprocal, without the scaling that
-// __fdividef adds for divisors near the largest float
+// a / b for b >= 1 (D of a face): the approximate reciprocal, whose documented
+// error is at most 2^-23 for b in [1, 2) (2^-22 of its value, and the same for
+// b scaled by a power of two), and one rounded product: within 3e-7 of the
+// quotient.  0 for b > 2^126, whose reciprocal is subnormal and flushed.
 __device__ __forceinline__ float div_(float a, float b)
 {
     float r;
