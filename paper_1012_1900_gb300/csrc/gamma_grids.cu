@@ -148,24 +148,23 @@ __device__ __forceinline__ float grid_cell(const GridProblem& G, const int (&p)[
     return fminf(best, cb);
 }
 
-// GL lanes per reference voxel (GL-aligned groups of a warp) over the voxels
-// that k_grid_cq left in walk_list, each from an infinite bound.  The table
-// starts with the voxel's own cell (offset 0), so the first round of G
-// cells gives a finite bound; later cells are skipped when the distance from
-// the point itself to the cell's box, with the dose gap, already reaches the
-// running gamma.  The exact stop (A1 step 4b-ii) takes the table's key.
-template <int N, int GL>
+// A warp per reference voxel over those that k_grid_cq left in walk_list, each
+// from an infinite bound.  The table starts with the voxel's own cell (offset
+// 0), so the first round of 32 cells gives a finite bound; later cells are
+// skipped when the distance from the point itself to the cell's box, with the
+// dose gap, already reaches the running gamma.  The exact stop (A1 step 4b-ii)
+// takes the table's key.
+template <int N>
 __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ GridProblem G)
 {
     grid_wait();                       // (the last kernel: nothing is released early)
-    const int lane = threadIdx.x & 31, gl = lane & (GL - 1), gbase = lane & ~(GL - 1);
-    const unsigned gmask = GL == 32 ? kFull : (((1u << GL) - 1u) << gbase);
+    const int lane = threadIdx.x & 31;
     const float dnorm = G.dose_norm > 0.f ? G.dose_norm : fdec(G.ctr->dnorm_enc);
     unsigned my_eval = 0, my_pass = 0, my_over = 0;
-    const long long ngroups = ((long long)gridDim.x * blockDim.x) / GL;
+    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
     const long long nwork = (long long)G.ctr->fix_count;
-    for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / GL; i < nwork;
-         i += ngroups) {                                     // group-uniform
+    for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < nwork;
+         i += nwarps) {                                      // warp-uniform
         const long long v = (long long)G.walk_list[i];
         const float dr = __ldg(G.ref + v);
         const long long ix[3] = {v % G.rn[0], (v / G.rn[0]) % G.rn[1], v / ((long long)G.rn[0] * G.rn[1])};
@@ -178,12 +177,12 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
 #pragma unroll
         for (int a = 0; a < N; ++a) {
             double ua = 0.0, f = 0.0;
-            if (gl == 0) {
+            if (lane == 0) {
                 ua = (G.ro[a] + (double)ix[a] * G.rh[a] - G.eo[a]) / G.eh[a];
                 f = fmin(fmax(floor(ua), 0.0), (double)(G.en[a] - 2));
             }
-            u[a] = __shfl_sync(gmask, ua, gbase);
-            c0[a] = (int)__shfl_sync(gmask, f, gbase);
+            u[a] = __shfl_sync(kFull, ua, 0);
+            c0[a] = (int)__shfl_sync(kFull, f, 0);
             fr[a] = (float)(u[a] - (double)c0[a]);
             ehf[a] = (float)G.eh[a];
         }
@@ -197,7 +196,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
         float best = kInf;
         int t = 0;
         while (t < ntable) {
-            const int idx = t + gl;
+            const int idx = t + lane;
             float key = kInf;
             uint32_t off = 0;
             if (idx < ntable) {
@@ -205,7 +204,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
                 key = e.key;
                 off = e.off;
             }
-            const float k0 = __shfl_sync(gmask, key, gbase);
+            const float k0 = __shfl_sync(kFull, key, 0);
             if (k0 * k0 >= best) break;                       // A1 step 4b-ii, exact
             float cb = best;
             if (key * key < best) {
@@ -232,13 +231,13 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
                 }
             }
 #pragma unroll
-            for (int o = GL / 2; o > 0; o >>= 1) cb = fminf(cb, __shfl_xor_sync(gmask, cb, o));
+            for (int o = 16; o > 0; o >>= 1) cb = fminf(cb, __shfl_xor_sync(kFull, cb, o));
             best = cb;
-            t += GL;
+            t += 32;
         }
         if (t >= ntable && best > rc2) {
             // past a truncated table: every remaining cell of the search box
-            if (gl == 0) ++my_over;
+            if (lane == 0) ++my_over;
             const float gm = sqrtf(best);
             int dlo[3] = {0, 0, 0}, dhi[3] = {0, 0, 0};
 #pragma unroll
@@ -252,7 +251,7 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
             const long long tot = wx * wy * wz;
             const float cut = rc2 * 0.99999f;
             float lb = best;
-            for (long long b = gl; b < tot; b += GL) {
+            for (long long b = lane; b < tot; b += 32) {
                 const int d[3] = {dlo[0] + (int)(b % wx), dlo[1] + (int)((b / wx) % wy), dlo[2] + (int)(b / (wx * wy))};
                 const int p[3] = {c0[0] + d[0], c0[1] + d[1], c0[2] + d[2]};
                 bool in = true;
@@ -268,10 +267,10 @@ __global__ void __launch_bounds__(256, 2) k_grid_walk(const __grid_constant__ Gr
                 lb = grid_cell<N>(G, p, u, cf, sqrtf(k2), dr, inv, dnorm, lb);
             }
 #pragma unroll
-            for (int o = GL / 2; o > 0; o >>= 1) lb = fminf(lb, __shfl_xor_sync(gmask, lb, o));
+            for (int o = 16; o > 0; o >>= 1) lb = fminf(lb, __shfl_xor_sync(kFull, lb, o));
             best = lb;
         }
-        if (gl == 0) {
+        if (lane == 0) {
             const float gam = sqrtf(best);
             G.out[v] = gam;
             ++my_eval;
@@ -378,7 +377,7 @@ __global__ void __launch_bounds__(256, 4) k_grid_seed(const __grid_constant__ Gr
             bool same = true;
 #pragma unroll
             for (int a = 0; a < N; ++a) {
-                // at most 500 cells away: the packed offset's range
+                // at most 500 cells away, within the packed offset's range
                 const float s = fminf(fmaxf(at.fr[a] - r * gk[a], -500.f), 500.f);
                 const int t = max(0, min(G.en[a] - 2, at.c0[a] + __float2int_rd(s)));
                 same = same && t == c[a];
@@ -396,13 +395,9 @@ __global__ void __launch_bounds__(256, 4) k_grid_seed(const __grid_constant__ Gr
         bool ill = false;
         const float cb = cell_min_d2<N, float>(q, g, G.mt, dmax, kInf, ill);
         if (ill) ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, G.mt.kappa, G.tau);
-        bool near = true;                                     // the offset fits its packed form
-#pragma unroll
-        for (int a = 0; a < N; ++a) near = near && abs(c[a] - at.c0[a]) <= 510;
         G.out[v] = ill ? kInf : cb + 0.f;
         G.queue[pos] = v;
-        G.skip[pos] = ill || !near ? 0xffffffffu
-                                   : pack10(c[0] - at.c0[0], c[1] - at.c0[1], N == 3 ? c[2] - at.c0[2] : 0);
+        G.skip[pos] = ill ? 0xffffffffu : pack10(c[0] - at.c0[0], c[1] - at.c0[1], N == 3 ? c[2] - at.c0[2] : 0);
     }
 }
 
@@ -762,11 +757,11 @@ cudaError_t launch_grids(const GridProblem& G, cudaStream_t s)
     if (G.ndim == 3) {
         launch_next(k_grid_seed<3>, gs, 256, 0, s, G);
         launch_next(k_grid_cq<3>, sms * 2, 384, 0, s, G);
-        launch_next(k_grid_walk<3, 32>, sms * 2, 256, 0, s, G);
+        launch_next(k_grid_walk<3>, sms * 2, 256, 0, s, G);
     } else {
         launch_next(k_grid_seed<2>, gs, 256, 0, s, G);
         launch_next(k_grid_cq<2>, sms * 2, 384, 0, s, G);
-        launch_next(k_grid_walk<2, 32>, sms * 2, 256, 0, s, G);
+        launch_next(k_grid_walk<2>, sms * 2, 256, 0, s, G);
     }
     return cudaGetLastError();
 }

@@ -133,11 +133,4 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Byte offset of element (row, k) of a K-major bf16 tile in the core-matrix
-// layout with LBO = rows/8 * 128 (k-chunks outermost) and SBO = 128.
-__device__ __forceinline__ uint32_t core_offset(int row, int k, int rows)
-{
-    return (uint32_t)(((k >> 3) * (rows >> 3) + (row >> 3)) * 128 + (row & 7) * 16 + (k & 7) * 2);
-}
-
 }  // namespace gk
