@@ -234,9 +234,10 @@ int gamma_get_timings(gamma_handle h, gamma_timings *out);
  *                     with queued voxels, stages the doses around it in shared
  *                     memory (one TMA copy) and walks the table for the row's
  *                     queued voxels.  Every walk gives the same map.  Handles
- *                     of gamma_create_grids take 0 (default: lanes_per_voxel
- *                     lanes per reference voxel) or 3 (8 lanes per voxel); the
- *                     cells that pass the bounds are evaluated by the warp.
+ *                     of gamma_create_grids take 0 (default) or 3, which are
+ *                     one search: lanes_per_voxel lanes walk a reference
+ *                     voxel, and the cells that pass the bounds are evaluated
+ *                     by the warp.
  *  "group_bucket"     "walk" 3: queued voxels whose cost bucket (1 + floor(2
  *                     log2 of the cells below their starting bound)) is at
  *                     least this value walk 4 lanes each, the rest one lane

@@ -1017,7 +1017,7 @@ int gamma_run(gamma_handle h, float* gamma_out_dev, void* cuda_stream)
         G.out = gamma_out_dev;
         G.ctr = h->ctr;
         G.tau = (float)h->tau;
-        G.lanes = h->walk == 3 ? gk::kDefaultLanesPerVoxel : h->lanes;
+        G.lanes = h->lanes;
         G.walk_list = h->grids->walk_list;
         G.queue = G.walk_list + h->nvox;
         G.skip = G.queue + h->nvox;
