@@ -86,7 +86,7 @@ typedef struct {
     int64_t n_voxels;        /* grid voxels */
     int64_t n_eval;          /* evaluated voxels (passed the cutoff) */
     int64_t n_pass;          /* evaluated voxels with gamma <= 1 */
-    int64_t tail_voxels;     /* voxels that searched past the key-0 cells */
+    int64_t tail_voxels;     /* voxels that searched past the key-0 cells (0 on two grids) */
     int64_t overflow_voxels; /* voxels that ran past the table and scanned their box */
     int64_t fp64_cells;      /* cells recomputed in FP64 (near-singular Gram matrix) */
     int64_t seeded;          /* queued voxels seeded by an attached model */
@@ -99,8 +99,9 @@ typedef struct {
     int64_t table_entries;   /* cell table length */
     double table_radius;     /* every cell with key < table_radius is in the table */
     uint32_t flags;          /* internal flags (non-finite input, queue overflow) */
-    int64_t lane_slot_steps; /* stats mode, default walk: 32 x the warps' loop steps of the
-                                queue walk, idle lanes included (0 for the other walks) */
+    int64_t lane_slot_steps; /* stats mode, default walk: table entries that the warps' loop
+                                steps of the queue walk have room for (two per lane), idle
+                                lanes included (0 for the other walks) */
 } gamma_stats;
 
 /* Per-phase device times of the last run, in ms, measured with CUDA events

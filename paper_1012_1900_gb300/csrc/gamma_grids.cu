@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(256, 4) k_grid_seed(const __grid_constant__ Gr
         }
         const unsigned tk = __ballot_sync(kFull, take);
         unsigned pos = 0;
-        if (tk && lane == 0) pos = atomicAdd(&G.ctr->tail_count, (unsigned)__popc(tk));
+        if (tk && lane == 0) pos = atomicAdd(&G.ctr->grid_count, (unsigned)__popc(tk));
         pos = __shfl_sync(kFull, pos, 0) + (unsigned)__popc(tk & ((1u << lane) - 1u));
         if (!take) continue;
         const unsigned v = (unsigned)i;
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(384, 2) k_grid_cq(const __grid_constant__ Grid
     const float dmax = G.tau > 0.f ? 0.99f * rsqrtf(G.tau) : kInf;
     const float eh[3] = {(float)G.eh[0], (float)G.eh[1], (float)G.eh[2]};
     const int sy = G.en[0], sz = G.en[0] * G.en[1];
-    const unsigned total = G.ctr->tail_count, nwarps = gridDim.x * (blockDim.x >> 5);
+    const unsigned total = G.ctr->grid_count, nwarps = gridDim.x * (blockDim.x >> 5);
     const unsigned nv = 32u / (unsigned)g;         // voxels per round
     const unsigned nb = min(32u, max(nv, total / (8u * nwarps) / nv * nv));
     unsigned my_eval = 0, my_pass = 0;

@@ -107,6 +107,7 @@ struct alignas(128) Counters {
     unsigned int head_part[4];          // warp-evaluated walk: work counters of the queue's parts
     unsigned int fix_count;             // ... voxels it leaves to the finishing pass
     unsigned int range_on;              // ... 1: this run's ordering pass wrote the cells' dose ranges
+    unsigned int grid_count;            // two grids: evaluated voxels in the walk's queue
     unsigned long long lane_steps;      // stats mode: lane slots of its loop steps, idle lanes included
 };
 
