@@ -96,21 +96,54 @@ __device__ __noinline__ float cell_recheck(const Problem& P, uint32_t ok, int cx
     return cell_redo_f64<N>(P.ev, p, sy, sz, ok, cx, cy, cz, drd, invd, P.mtd, &P.ctr->fp64_cells);
 }
 
-// Takes the voxel itself out of the vertices of a cell whose box contains it
-// (lower corner at 0 or -1 on every axis; q: relative doses), so that only the
-// cell's faces off the voxel remain: those through it have their value from the
-// reduced form before any table walk, and the general one could differ from it
-// in the last bit.  Other cells are left as they are.
+// The voxel itself among the vertices of a cell whose box contains it (lower
+// corner at 0 or -1 on every axis): taken out for the walks, so that only the
+// cell's faces off the voxel remain.  Those through it have their value from the
+// reduced form before any table walk, and the general one could differ from it in
+// the last bit.  Other cells are left as they are.
+//
+// The reduced form's conditions lose their digits where a dose step is some 1e5
+// Delta D, and a valid face through the voxel may be left out.  A cell that is
+// near singular with the voxel's vertex therefore gets its FP64 evaluation like
+// any other: steep says that it may be (D of a face is at most 1 + N (range of the
+// vertices)^2 kappa_max; below dmax the Gram matrices need no look), and the test
+// of the Gram matrices is asked with the vertex put back.
 template <int N>
-__device__ __forceinline__ void drop_own_vertex(float (&q)[8], int cx, int cy, int cz)
-{
-    if ((unsigned)(cx + 1) < 2u && (unsigned)(cy + 1) < 2u && (N == 2 || (unsigned)(cz + 1) < 2u)) {
-        const int self = (cx & 1) | ((cy & 1) << 1) | (N == 3 ? (cz & 1) << 2 : 0);
+struct OwnVertex {
+    int self;           // its index, or -1
+    float q;            // its relative dose
+    bool steep;
+
+    __device__ __forceinline__ void take(float (&v)[8], int cx, int cy, int cz, const float (&kappa)[8], float dmax)
+    {
+        self = -1;
+        q = 0.f;
+        steep = false;
+        if ((unsigned)(cx + 1) < 2u && (unsigned)(cy + 1) < 2u && (N == 2 || (unsigned)(cz + 1) < 2u)) {
+            self = (cx & 1) | ((cy & 1) << 1) | (N == 3 ? (cz & 1) << 2 : 0);
+            float lo = v[0], hi = v[0];
+#pragma unroll
+            for (int u = 1; u < (1 << N); ++u) {              // (NaN: no such vertex)
+                lo = fminf(lo, v[u]);
+                hi = fmaxf(hi, v[u]);
+            }
+            const float range = hi - lo, k2 = fmaxf(kappa[1], kappa[2]), kmax = N == 3 ? fmaxf(k2, kappa[4]) : k2;
+            steep = fmaf((float)N * kmax * range, range, 1.f) > dmax;
+#pragma unroll
+            for (int u = 0; u < (1 << N); ++u)
+                if (u == self) {
+                    q = v[u];
+                    v[u] = kNaN;
+                }
+        }
+    }
+    __device__ __forceinline__ void put(float (&v)[8]) const
+    {
 #pragma unroll
         for (int u = 0; u < (1 << N); ++u)
-            if (u == self) q[u] = kNaN;
+            if (u == self) v[u] = q;
     }
-}
+};
 
 // Every face of the cell with lower corner (x+cx, y+cy, z+cz) as squared
 // gamma (WALK: of a cell whose box contains the voxel only those off the
@@ -124,11 +157,16 @@ __device__ __noinline__ float cell_all_faces(const Problem& P, float q0, float q
                                              float dr, float dnorm)
 {
     float q[8] = {q0, q1, q2, q3, q4, q5, q6, q7};
-    if (WALK) drop_own_vertex<N>(q, cx, cy, cz);
+    OwnVertex<N> own;
+    if (WALK) own.take(q, cx, cy, cz, P.mt.kappa, ill_dmax(P));
     CellGeom<float> g;
     cell_geom<N, float>(cx, cy, cz, P.mt, g);
     bool ill = false;
     float cb = cell_min_d2<N, float>(q, g, P.mt, ill_dmax(P), kInf, ill);
+    if (WALK && (ill || own.steep)) {
+        own.put(q);
+        ill = true;
+    }
     if (ill) ill = cell_gram_ill<N>(q, ok, P.mt.kappa, P.tau);
     if (ill) {
         const double drd = dr;

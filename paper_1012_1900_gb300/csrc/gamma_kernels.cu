@@ -1425,12 +1425,16 @@ __global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH)
         float q[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) q[u] = u < (1 << N) ? rel_dose(e[u], dr, inv) : kNaN;
-        drop_own_vertex<N>(q, c[0], c[1], c[2]);
+        OwnVertex<N> own;
+        own.take(q, c[0], c[1], c[2], P.mt.kappa, ill_dmax(P));
         CellGeom<float> g;
         cell_geom<N, float>(c[0], c[1], c[2], P.mt, g);
         bool ill = false;
         const float cb = cell_min_d2<N, float>(q, g, P.mt, ill_dmax(P), kInf, ill);
-        if (ill) ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, P.mt.kappa, P.tau);
+        if (ill || own.steep) {
+            own.put(q);
+            ill = cell_gram_ill<N>(q, (1u << (1 << N)) - 1u, P.mt.kappa, P.tau);
+        }
         // a near-singular cell is left to the walk (and its FP64 redo)
         P.plane_raw[i] = ill ? kNoSeed : pack10(c[0], c[1], c[2]);
         if (!ill && cb < best) {
@@ -1661,13 +1665,18 @@ __global__ void __launch_bounds__(cq_threads(MINB), MINB)
                                 ok |= 1u << u;
                             }
                         }
-                        drop_own_vertex<N>(cq, cx, cy, cz);
                         auto evaluate = [&](const Metric& mt, float dmax, float tau) {
+                            OwnVertex<N> self;
+                            self.take(cq, cx, cy, cz, mt.kappa, dmax);
                             CellGeom<float> cg;
                             cell_geom<N, float>(cx, cy, cz, mt, cg);
                             bool ill = false;
                             const float cb = cell_min_d2<N, float>(cq, cg, mt, dmax, kInf, ill);
-                            if (ill && cell_gram_ill<N>(cq, ok, mt.kappa, tau))
+                            if (ill || self.steep) {
+                                self.put(cq);
+                                ill = cell_gram_ill<N>(cq, ok, mt.kappa, tau);
+                            }
+                            if (ill)
                                 atomicOr(&W.fixm, 1u << own);                  // k_tail_fix redoes it
                             else
                                 atomicMin(&W.best[own], __float_as_uint(cb + 0.f));   // -0 -> +0

@@ -1,0 +1,41 @@
+"""Voxels of the evaluation dose far above or below the others, by up to some
+1e6 Delta D: the faces through them are near singular, and their conditions
+need more digits than FP32 has.  Such a voxel's own cells get an FP64
+evaluation, which finds a face that FP32 left out."""
+import functools
+
+import numpy as np
+import pytest
+
+import synth
+from tests.test_gpu_parity import gpu_gamma, oracle_gamma
+
+pytestmark = pytest.mark.gpu
+
+CRITS = [synth.Criteria(0.03, 3.0, cutoff_frac=0.0), synth.Criteria(0.01, 1.0, cutoff_frac=0.0)]
+
+
+@functools.lru_cache(maxsize=None)
+def _spiky(nd, value):
+    """Pair with a spike of 0.5 to 1.5 `value` at every seventh voxel per axis,
+    and its oracle maps."""
+    if nd == 2:
+        p = synth.make_pair_2d(shape=(300, 300), seed=4)
+    else:
+        p = synth.make_pair_3d(shape=(40, 61, 62), spacing=(2.5, 2.0, 2.0), seed=3, shift_mm=(0.5, 1.0, 1.0), scale=1.02)
+    rng = np.random.default_rng(11)
+    at = tuple(np.meshgrid(*[np.arange(3, n - 3, 7) for n in p.eval.shape], indexing="ij"))
+    p.eval[at] = (value * rng.uniform(0.5, 1.5, at[0].shape)).astype(np.float32)
+    return p, [oracle_gamma(p.ref, p.eval, p.spacing, c) for c in CRITS]
+
+
+@pytest.mark.parametrize("walk", [3, 0])
+@pytest.mark.parametrize("nd,value", [(2, 1e4), (2, 3e4), (2, 1e5), (2, -1e4), (3, 3e4), (3, 1e5)])
+def test_no_face_through_a_spike_is_left_out(nd, value, walk):
+    p, wants = _spiky(nd, value)
+    for crit, want in zip(CRITS, wants):
+        got, _, stats = gpu_gamma(p.ref, p.eval, p.spacing, crit, {"walk": walk})
+        ok = ~np.isnan(want)
+        assert np.array_equal(ok, ~np.isnan(got))
+        assert stats["fp64_cells"] > 0
+        assert (got - want)[ok].max() <= 1e-4
