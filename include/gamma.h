@@ -111,8 +111,10 @@ typedef struct {
 typedef struct {
     float h2d_ms;       /* host-to-device copies (gamma_run_host) */
     float prepare_ms;   /* dose norm and finite check */
-    float shell_ms;     /* gamma0 and the key-0 cells, every voxel */
-    float order_ms;     /* cost ordering of the queued voxels */
+    float shell_ms;     /* gamma0 and the key-0 cells, every voxel; then the queued voxels'
+                         * starting bounds and, with a model, its passes */
+    float order_ms;     /* cost ordering of the queued voxels (overlapped: their starting
+                         * bounds first) */
     float tail_ms;      /* table walk of the queued voxels */
     float d2h_ms;       /* device-to-host copy of the gamma map (gamma_run_host) */
     float total_ms;     /* first to last event */
@@ -123,6 +125,8 @@ typedef struct {
                          * shell: the last z slab; d2h: the map copy-out;
                          * total: the final patch of the queued voxels);
                          * 2: the same, with the shell gated per z slab */
+    /* A batch handle with option "timing" runs its planes and its volumes one
+     * after the other on one stream; without it they run side by side. */
 } gamma_timings;
 
 /* Create a handle for one dose-pair geometry (Algorithm A1 steps 2-3: builds

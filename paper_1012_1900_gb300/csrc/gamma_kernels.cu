@@ -1340,11 +1340,13 @@ constexpr int kPlaneSteps = 3;
 // the cells differ per lane but every lane evaluates exactly one.  Bound by
 // the latency of the dependent dose loads: 136 k voxels of a 160x160x120 map
 // take 13.2 us, 648 k of a 200x200x150 map 35 us, 5.9 M of a 320x320x240 map
-// 263 us, and spare the walk half of its time there.  Batched volumes, whose
-// form needs 97 registers, take 64 (144 bytes spilled) in blocks of 128 for 32
-// instead of 16 warps per SM: a batch's eight volumes 55.6 to 38.8 us.  For
-// one pair the same (16 bytes spilled) is 10.4, 31 and 234 us, but a map of
-// 99 k queued voxels, one wave of blocks either way, lost 1 us in 89.
+// 261 us, and spare the walk half of its time there.  Batched volumes, whose
+// form needs 97 registers, take 64 (84 bytes spilled) in blocks of 128 for 32
+// instead of 16 warps per SM: a batch's eight volumes 55.6 to 42 us.  For one
+// pair the same (16 bytes spilled) was 10.4, 31 and 234 us, but a map of 99 k
+// queued voxels, one wave of blocks either way, lost 1 us in 89.  What decides
+// is the length of the queue, which the host does not know when it launches:
+// a batch's is long as a rule.
 __host__ __device__ constexpr int seed_threads(int n, bool batch) { return n == 3 && batch ? 128 : 256; }
 
 template <int N, bool BATCH>
@@ -1485,8 +1487,8 @@ __global__ void __launch_bounds__(seed_threads(N, BATCH), seed_threads(N, BATCH)
 // three tiers; the dose loads hit L1 at 92 %.  Before, one walker per lane or
 // group collected the cells past the dose gap alone and evaluated all of them
 // (21.8 per queued voxel of a 320x320x240 map at 3 %/3 mm, 36.5 at 1 %/1 mm
-// local; now 3.5 and 8.3): 10.5 ms there and 23.6 ms, now 3.04 ms and 7.87 ms
-// (twelve warps in each of two blocks per SM); 428 us and 176 us on a
+// local; now 3.5 and 8.3): 10.5 ms there and 23.6 ms, now 2.95 ms and 7.11 ms
+// (twelve warps in each of two blocks per SM); 428 us and 185 us on a
 // 200x200x150 map at 2 %/2 mm.  Two entries per lane and step and the cells'
 // dose ranges (wants_range) are the last 0.5 ms and 2.3 ms of these.
 constexpr int kCqRing = 128;              // cells in each ring of a warp (up to 31 + 64 wait)

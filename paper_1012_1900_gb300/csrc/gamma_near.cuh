@@ -36,7 +36,7 @@
 //
 // Measured on a 160x160x120 map (1.21 M evaluated voxels, k_shell_w alone):
 // 61.5 us and 45.9 M warp instructions with a comparison per condition and one
-// voxel per lane (ALU pipe 64 %), 52.9 us and 33.4 M now (ALU 43 %, issue 56 %
+// voxel per lane (ALU pipe 64 %), 52.9 us and 34.1 M now (ALU 43 %, issue 56 %
 // with four warps per scheduler: bound by the latency of its own chains at the
 // 128 registers that two blocks per SM leave).
 #pragma once
